@@ -180,11 +180,10 @@ void worker_main(sigw_server_s* s, int max_N) {
     // Budget the oldest queued request keeps reserved: its footprint while no plan of its size class exists.
     // If even evicting every idle plan would not make room for it, it is blocked: no later request may start
     // (idle plans then stay idle until enough of them can be evicted for the oldest one).
-    size_t reserve = 0;
+    size_t reserve = 0, idle = 0;
     bool blocked = false;
     if (!s->queue.empty() && !any_plan(s, s->queue.front()->N, s->queue.front()->L)) {
       reserve = footprint_of(s, s->queue.front()->N);
-      size_t idle = 0;
       for (PoolPlan* p : s->pool)
         if (!p->busy && !p->creating) idle += p->bytes;
       blocked = s->in_use - idle + reserve > s->budget;
@@ -194,6 +193,12 @@ void worker_main(sigw_server_s* s, int max_N) {
       if (qi > 0 && blocked) break;
       if (max_N > 0 && r->N > max_N) continue;
       if ((use = idle_plan(s, r->N, r->L))) {
+        // an idle plan the oldest request would have to evict is left to it (a slot that may not take the oldest
+        // request would otherwise keep the plan busy from one small request to the next)
+        if (qi > 0 && reserve && s->in_use - idle + use->bytes + reserve > s->budget) {
+          use = nullptr;
+          continue;
+        }
         head = r;
         break;
       }
