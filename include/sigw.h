@@ -243,10 +243,11 @@ sigw_status sigw_server_destroy(sigw_server srv);
  * (N, precision, max_batch, n_alpha) from which later plans with alpha_batch = 0 start; then times both radix
  * forms of the last inverse pass (FP32, N = 128, 256, 512) on the terms just produced; at FP32 N = 128, 256, 512 it
  * also times the first pass with its Phi~ tile and cells in tensor memory and the radix-16 last pass with its
- * accumulators in tensor memory.  An untuned FP32 plan starts from the bits measured fastest on GB300 (26 at
- * N = 128 and 256, 15 at N = 512).  Outputs nullable: chosen terms per launch, variant bits (1: alternative radix of
+ * accumulators in tensor memory, and at FP32 N = 64 the fused second and last pass against the three passes.  An
+ * untuned FP32 plan starts from the bits measured fastest on GB300 (8 at N = 64, 26 at N = 128 and 256, 15 at N = 512).  Outputs nullable: chosen terms per launch, variant bits (1: alternative radix of
  * the first strided pass, 2: radix-16 last pass, 4: alternative radix of the second strided pass, 8: radix-16 last
- * pass with its accumulators in tensor memory, 16: first pass with its tile in tensor memory) and the time in ms of the
+ * pass with its accumulators in tensor memory, which at N = 64 also takes in the second pass and runs all terms in one
+ * launch whatever the terms per launch, 16: first pass with its tile in tensor memory) and the time in ms of the
  * chosen strided passes plus last pass for one kernel (m = s).  Waits for the stream.
  * Errors: SIGW_ESTATE (no field), SIGW_EINVAL, SIGW_ECUDA. */
 sigw_status sigw_plan_autotune(sigw_plan plan, int n_c, int* out_alpha_batch, int* out_variant, double* out_ms);

@@ -37,9 +37,9 @@ sigw::DecompParams params_of(const sigw_opts& o) {
   return p;
 }
 
-int auto_alpha_batch(const sigw_opts& o) {
+int auto_alpha_batch(int N, const sigw_opts& o) {
   if (o.alpha_batch > 0) return std::min(o.alpha_batch, o.n_alpha);
-  return std::min(o.n_alpha, 10);
+  return std::min(o.n_alpha, N <= 64 ? 16 : 10);
 }
 
 // Largest terms-per-launch the first-pass output buffer holds (the autotuner's largest candidate).
@@ -81,7 +81,11 @@ Sizes sizes_of(int N, const sigw_opts& o) {
   // the jackknife reuses W after each shell: two standard + two packed half spectra + two real fields
   s.W = std::max(s.W, mb * 2 * (NN * NH * cel + NN * H * cel + NN * (size_t)N * rel) + 1024);
   s.synth = mb * (NN * H * cel + NN * NH * cel + 3 * NN * (size_t)N * rel) + 1024;  // + two real fields (non-local map)
-  s.F = mb * 6 * NN * NH * cel;
+  size_t parts = 1;  // partial fields of the last pass
+  for (int v : {0, 8})
+    parts = std::max(parts, (size_t)(o.precision == 64 ? sigw::OpsRT<double>::last_groups(N, v, o.n_alpha)
+                                                       : sigw::OpsRT<float>::last_groups(N, v, o.n_alpha)));
+  s.F = parts * mb * 6 * NN * NH * cel;
   s.F2 = mb * 6 * NN * NH * cel;
   s.partial = mb * H * 2 * (size_t)s.maxblk * sizeof(double);
   s.out = mb * H * 4 * sizeof(double) + H * (sizeof(int) + sizeof(double));
@@ -429,11 +433,11 @@ sigw_status sigw_plan_create(int N, double L, const sigw_opts* opts, void* cuda_
   p->N = N;
   p->L = L;
   p->opts = o;
-  p->B = auto_alpha_batch(o);
+  p->B = auto_alpha_batch(N, o);
   // Untuned default: the choices measured fastest on GB300 (at 128^3 and 256^3 the first and the radix-16 last pass
   // with their per-thread state in tensor memory; at 512^3 the 512-specific strided passes and the tensor-memory
   // last pass).  sigw_plan_autotune or the table may override it.
-  p->variant = o.precision == 32 ? (N == 512 ? 15 : (N >= 128 ? 26 : 0)) : 0;
+  p->variant = o.precision == 32 ? (N == 512 ? 15 : (N >= 128 ? 26 : (N == 64 ? 8 : 0))) : 0;
   std::string e;
   if (!sigw::build_decomposition(params_of(o), &p->dec, &e)) {
     delete p;
@@ -716,9 +720,12 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, con
   const int n_alpha = p->opts.n_alpha, nm1 = p->opts.n_modes + 1;
   const size_t NN = (size_t)N * N;
   const size_t cel = p->celem();
-  void* Ta = p->d_T;
-  void* Tb = (char*)p->d_T + (size_t)batch * p->B * NN * H * cel;
   const int var = p->variant;
+  // the fused second and last pass takes the first pass's output of all terms, kept in W's place (it needs no W)
+  const bool fused = OPS(p, fused, N, var);
+  void* Ta = fused ? p->d_work : p->d_T;
+  void* Tb = (char*)Ta + (size_t)batch * (fused ? n_alpha : p->B) * NN * H * cel;
+  const int groups = OPS(p, last_groups, N, var, n_alpha);
   const long pbs = (long)ns * 2 * p->sz.maxblk;
   const double fieldb = (double)batch * NN * H * cel;  // one packed complex field per realisation batch
   const double phib = (double)batch * NN * (H + 1) * cel;
@@ -732,18 +739,26 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, con
     for (int n1 = n1lo; n1 < n1lo + nk1; ++n1)
       for (int n2 = 0; n2 <= n_c; ++n2) disk += (n1 * n1 + n2 * n2 <= n_c * n_c + n_c);
     for (int m = 0; m < 2; ++m) {
-      for (int a0 = 0; a0 < n_alpha; a0 += p->B) {
+      if (fused) {
+        RUN(p, 1, phib + 2.0 * n_alpha * fieldb, "P1",
+            OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[m], nm1, 0, n_alpha, batch, p->d_tw, var, st));
+        RUN(p, 3, 2.0 * n_alpha * fieldb + 6.0 * groups * batch * NN * ncp * cel, "P23",
+            OPS(p, p23, N, Ta, Tb, p->d_sigma[m], n_alpha, p->d_F, groups, n_c, batch, p->d_tw, p->d_err, p->wait_limit,
+                st));
+      }
+      for (int a0 = 0; a0 < n_alpha && !fused; a0 += p->B) {
         const int nb = std::min(p->B, n_alpha - a0);
         RUN(p, 1, phib + 2.0 * nb * fieldb, "P1",
             OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[m], nm1, a0, nb, batch, p->d_tw, var, st));
         RUN(p, 2, 5.0 * nb * fieldb, "P2",
             OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, var, st));
       }
-      RUN(p, 3, 3.0 * n_alpha * fieldb + 6.0 * batch * NN * ncp * cel, "P3",
-          OPS(p, p3, N, p->d_work, p->d_sigma[m], n_alpha, p->d_F, n_c, batch, p->d_tw, p->d_err, p->wait_limit,
-              var, st));
-      RUN(p, 4, 6.0 * batch * ((double)NN * ncp + (double)N * nk1 * ncp) * cel, "F2",
-          OPS(p, f2, N, p->d_F, p->d_F2, n_c, batch, p->d_tw, st));
+      if (!fused)
+        RUN(p, 3, 3.0 * n_alpha * fieldb + 6.0 * groups * batch * NN * ncp * cel, "P3",
+            OPS(p, p3, N, p->d_work, p->d_sigma[m], n_alpha, p->d_F, groups, n_c, batch, p->d_tw, p->d_err,
+                p->wait_limit, var, st));
+      RUN(p, 4, 6.0 * batch * (groups * (double)NN * ncp + (double)N * nk1 * ncp) * cel, "F2",
+          OPS(p, f2, N, p->d_F, groups, p->d_F2, n_c, batch, p->d_tw, st));
       if (!jk) {
         RUN(p, 5, 6.0 * batch * (double)N * disk * cel, "F3",
             OPS(p, f3, N, p->d_F2, n_c, p->d_partial + ((long)si * 2 + m) * p->sz.maxblk, pbs, batch, p->d_tw, st));
@@ -1079,9 +1094,11 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
     }
     if (p->opts.alpha_batch > 0) break;
   }
-  // last inverse pass: radix variants on the W just produced by the best strided choice
+  // last inverse pass: radix variants on the W just produced by the best strided choice; then, where it exists, the
+  // fused second and last pass (with the best first pass) against the three passes together
   int bestP3 = 0;
-  if (status == SIGW_OK && OPS(p, p3_variants, N) > 1) {
+  const bool has_fused = OPS(p, fused, N, 8);
+  if (status == SIGW_OK && (OPS(p, p3_variants, N) > 1 || has_fused)) {
     {
       void* Ta = p->d_T;
       void* Tb = (char*)p->d_T + (size_t)batch * bestB * NN * H * cel;
@@ -1092,28 +1109,47 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
         if (e != cudaSuccess) status = cuda_fail(p, e, "autotune launch");
       }
     }
+    auto time_last = [&](float* ms, auto&& launch) {  // second of two runs
+      for (int rep = 0; rep < 2 && status == SIGW_OK; ++rep) {
+        cudaEventRecord(e0, st);
+        cudaError_t e = launch();
+        cudaEventRecord(e1, st);
+        if (e != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+            cudaEventElapsedTime(ms, e0, e1) != cudaSuccess)
+          status = cuda_fail(p, e != cudaSuccess ? e : cudaGetLastError(), "autotune last pass");
+      }
+    };
     const int np3 = OPS(p, p3_variants, N);  // 2: radix 8 / 16; 3: also radix 16 with TMEM accumulators
     const int p3bits[3] = {0, 2, 8};
     float t3[3] = {1e30f, 1e30f, 1e30f};
-    for (int v3 = 0; v3 < np3 && status == SIGW_OK; ++v3) {
-      for (int rep = 0; rep < 2; ++rep) {
-        cudaEventRecord(e0, st);
-        cudaError_t e = OPS(p, p3, N, p->d_work, p->d_sigma[0], n_alpha, p->d_F, n_c, batch, p->d_tw, p->d_err,
-                            sigw::kDefaultWaitLimit, p3bits[v3], st);
-        cudaEventRecord(e1, st);
-        if (e != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-            cudaEventElapsedTime(&t3[v3], e0, e1) != cudaSuccess) {
-          status = cuda_fail(p, e != cudaSuccess ? e : cudaGetLastError(), "autotune last pass");
-          break;
-        }
-      }
+    for (int v3 = 0; v3 < np3; ++v3) {
+      const int bits = p3bits[v3], groups = has_fused ? OPS(p, last_groups, N, 0, n_alpha) : 1;
+      time_last(&t3[v3], [&]() {
+        return OPS(p, p3, N, p->d_work, p->d_sigma[0], n_alpha, p->d_F, groups, n_c, batch, p->d_tw, p->d_err,
+                   sigw::kDefaultWaitLimit, bits, st);
+      });
     }
     int bv = 0;
     for (int v3 = 1; v3 < np3; ++v3)
       if (t3[v3] < t3[bv]) bv = v3;
-    if (status == SIGW_OK) {
-      bestP3 = p3bits[bv];
-      best += t3[bv];
+    bestP3 = p3bits[bv];
+    best += t3[bv];
+    if (has_fused) {
+      float tf = 1e30f;
+      void* Ta = p->d_work;
+      void* Tb = (char*)p->d_work + (size_t)batch * n_alpha * NN * H * cel;
+      time_last(&tf, [&]() {
+        cudaError_t e = OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, 0, n_alpha, batch, p->d_tw, bestV | 8,
+                            st);
+        if (e == cudaSuccess)
+          e = OPS(p, p23, N, Ta, Tb, p->d_sigma[0], n_alpha, p->d_F, OPS(p, last_groups, N, 8, n_alpha), n_c, batch,
+                  p->d_tw, p->d_err, sigw::kDefaultWaitLimit, st);
+        return e;
+      });
+      if (status == SIGW_OK && tf < best) {
+        best = tf;
+        bestP3 = 8;
+      }
     }
   }
   cudaEventDestroy(e0);

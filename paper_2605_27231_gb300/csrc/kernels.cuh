@@ -378,24 +378,27 @@ __global__ void k_reduce_mean(const double* __restrict__ part, int nblk, double*
 // P1: first inverse pass along axis 0 for a tile of TC packed columns at fixed k1.
 //   V_a(n) = phi_a(cell(|n|^2)) Phi~(n)          (column 0: V(k2=0) + i V(k2=H), each with its own cell)
 //   Ta_a = IDFT_0[V_a],  Tb_a = IDFT_0[i n0^D V_a]
+// The nb terms of a launch are split over nag CTAs per tile (blockIdx.z = b * nag + group), see p1_groups.  With
+// swz = 8 the column index is stored as cc ^ (8 (k1 mod 2)) (the fused second and last pass reads it that way).
 template <typename T, int N, int E_ = Shape<T, N>::ES, int TC_ = Shape<T, N>::TC>
 __global__ void __launch_bounds__(256) k_p1(const cx<T>* __restrict__ phi, cx<T>* __restrict__ Ta,
                                             cx<T>* __restrict__ Tb, const int16_t* __restrict__ lut,
-                                            const T* __restrict__ phitab, int nm1, int alpha0, int nb,
-                                            const cx<T>* __restrict__ tw) {
+                                            const T* __restrict__ phitab, int nm1, int alpha0, int nb, int nag,
+                                            int swz, const cx<T>* __restrict__ tw) {
   constexpr int E = E_, P = N / E_, TC = TC_, H = N / 2, NH = H + 1;
   using Lay = StridedLay<T, N, TC, E>;
   extern __shared__ __align__(16) unsigned char smraw[];
   cx<T>* sm_nyq = reinterpret_cast<cx<T>*>(smraw) + Lay::SIZE;  // N values (column 0 only)
   int* sm_cn = reinterpret_cast<int*>(sm_nyq + N);              // N cells
-  T* sm_tab = reinterpret_cast<T*>(sm_cn + N);                  // nb * nm1
+  T* sm_tab = reinterpret_cast<T*>(sm_cn + N);                  // (terms of this CTA) * nm1
   const int c = threadIdx.x % TC, j = threadIdx.x / TC;
   const Lay L{reinterpret_cast<cx<T>*>(smraw), c};
   const int cc = blockIdx.x * TC + c;
   const int k1 = blockIdx.y;
-  const int b = blockIdx.z;
+  const int b = blockIdx.z / nag, ag = blockIdx.z % nag;
+  const int alo = (int)((long)nb * ag / nag), ahi = (int)((long)nb * (ag + 1) / nag);  // terms of this CTA
   const int n1 = wrapn(k1, N);
-  for (int i = threadIdx.x; i < nb * nm1; i += blockDim.x) sm_tab[i] = phitab[(long)alpha0 * nm1 + i];
+  for (int i = threadIdx.x; i < (ahi - alo) * nm1; i += blockDim.x) sm_tab[i] = phitab[(long)(alpha0 + alo) * nm1 + i];
   const cx<T>* pb = phi + ((long)b * N * N + k1) * NH;  // + k0 * N * NH + k2
   if (blockIdx.x == 0) {
     for (int k0 = threadIdx.x; k0 < N; k0 += blockDim.x) {
@@ -416,8 +419,9 @@ __global__ void __launch_bounds__(256) k_p1(const cx<T>* __restrict__ phi, cx<T>
   __syncthreads();
   const long fstride = (long)N * N * H;  // one field
   const T fj = (T)j;
-  for (int a = 0; a < nb; ++a) {
-    const T* tab = sm_tab + a * nm1;
+  const int cs = cc ^ ((k1 & 1) * swz);
+  for (int a = alo; a < ahi; ++a) {
+    const T* tab = sm_tab + (a - alo) * nm1;
     // D = 0: V_a; D = 1: i n0 V_a.  V_a is formed again for the second transform instead of being kept,
     // so only one value array is live next to the Phi~ tile.
 #pragma unroll 1
@@ -440,7 +444,7 @@ __global__ void __launch_bounds__(256) k_p1(const cx<T>* __restrict__ phi, cx<T>
         v[r] = x;
       }
       fft_pencil<T, N, E, +1, Lay, SyncBlock>(v, j, L, tw, SyncBlock());
-      cx<T>* dst = (D ? Tb : Ta) + ((long)b * nb + a) * fstride + (long)k1 * H + cc;
+      cx<T>* dst = (D ? Tb : Ta) + ((long)b * nb + a) * fstride + (long)k1 * H + cs;
 #pragma unroll
       for (int r = 0; r < E; ++r) dst[(long)(j + r * P) * N * H] = v[r];
     }
@@ -552,7 +556,9 @@ template <typename T, int N, int E_ = ((N >= 16) ? 8 : 4)> struct P3Cfg {
     return (size_t)STAGES * 6 * rpc * H * sizeof(cx<T>) + (size_t)rpc * Lay::SIZE * sizeof(cx<T>) +
            STAGES * sizeof(uint64_t);
   }
-  static constexpr int RPC0 = 16384 / (H * (int)sizeof(cx<T>));  // one 16 KB bulk copy per (field, term)
+  // One 16 KB bulk copy per (field, term).  On the small lattices 64 threads: a realisation at N = 32 then has 64 CTAs
+  // (times the groups of term pairs) instead of 16 or 8 (FP64, 50 terms: 976 -> 253 us, the FP64 pipe of 128 SMs).
+  static constexpr int RPC0 = N <= 32 ? 64 / P : 16384 / (H * (int)sizeof(cx<T>));
   static constexpr int RPC1 = RPC0 > N * N ? N * N : RPC0;
   static constexpr int RPC = smem_for(RPC1) <= 227 * 1024 ? RPC1 : RPC1 / 2;
   static constexpr int THREADS = RPC * P;
@@ -673,7 +679,7 @@ __device__ __forceinline__ void accum6<float, true>(float sa, float g0, float2 z
 template <typename T, int N, int E_ = ((N >= 16) ? 8 : 4)>
 __global__ void __launch_bounds__(P3Cfg<T, N, E_>::THREADS, 1) k_p3(const cx<T>* __restrict__ W,
                                                                    const T* __restrict__ sigma, int n_alpha,
-                                                                   cx<T>* __restrict__ F, int n_c,
+                                                                   cx<T>* __restrict__ F, long fgstride, int n_c,
                                                                    const cx<T>* __restrict__ tw,
                                                                    int* __restrict__ err, long long wait_limit) {
   using CF = P3Cfg<T, N, E_>;
@@ -690,7 +696,11 @@ __global__ void __launch_bounds__(P3Cfg<T, N, E_>::THREADS, 1) k_p3(const cx<T>*
   const long row = row0 + rr;
   const int b = blockIdx.y;
   const long fstride = (long)N * N * H;
-  const int npairs = (n_alpha + 1) / 2;
+  // term pairs pr0 .. pr0 + npairs - 1 (blockIdx.z of gridDim.z groups; each group writes its own partial F)
+  const int allpairs = (n_alpha + 1) / 2;
+  const int pr0 = allpairs * (int)blockIdx.z / (int)gridDim.z;
+  const int npairs = allpairs * ((int)blockIdx.z + 1) / (int)gridDim.z - pr0;
+  F += (long)blockIdx.z * fgstride;
   constexpr uint32_t COPY = RPC * H * sizeof(cx<T>);
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) mbar_init(bars + s, 1);
@@ -698,7 +708,7 @@ __global__ void __launch_bounds__(P3Cfg<T, N, E_>::THREADS, 1) k_p3(const cx<T>*
   }
   __syncthreads();
   auto issue = [&](int pr) {  // thread 0: the six rows blocks of term pair pr into stage pr % STAGES
-    const int s = pr % STAGES, a = 2 * pr;
+    const int s = pr % STAGES, a = 2 * (pr0 + pr);
     const bool two = a + 1 < n_alpha;
     cx<T>* dst = ring + s * CF::STAGE_ELEMS;
     fence_proxy_async();
@@ -728,7 +738,7 @@ __global__ void __launch_bounds__(P3Cfg<T, N, E_>::THREADS, 1) k_p3(const cx<T>*
       issued = pr + STAGES;
     }
     if (ok) ok = mbar_wait(bars + s, (uint32_t)((pr / STAGES) & 1), err, wait_limit);
-    const int a = 2 * pr;
+    const int a = 2 * (pr0 + pr);
     const bool two = a + 1 < n_alpha;
     const cx<T>* st = ring + s * CF::STAGE_ELEMS + rr * H;
     const cx<T>* wb0 = st;
@@ -1202,24 +1212,26 @@ template <int N>
 __global__ void __launch_bounds__(P1TCfg<N>::THREADS, 3) k_p1_tm(const float2* __restrict__ phi, float2* __restrict__ Ta,
                                                                   float2* __restrict__ Tb, const int16_t* __restrict__ lut,
                                                                   const float* __restrict__ phitab, int nm1, int alpha0,
-                                                                  int nb, const float2* __restrict__ tw) {
+                                                                  int nb, int nag, int swz,
+                                                                  const float2* __restrict__ tw) {
   using CF = P1TCfg<N>;
   constexpr int E = CF::E, P = CF::P, TC = CF::TC, H = CF::H, NH = H + 1;
   using Lay = typename CF::Lay;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm_nyq = reinterpret_cast<float2*>(smraw) + Lay::SIZE;  // N values (column 0 only)
   int* sm_cn = reinterpret_cast<int*>(sm_nyq + N);                // N cells
-  float* sm_tab = reinterpret_cast<float*>(sm_cn + N);            // nb * nm1
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm_tab + nb * nm1);
+  float* sm_tab = reinterpret_cast<float*>(sm_cn + N);            // (terms of this CTA) * nm1
+  const int b = blockIdx.z / nag, ag = blockIdx.z % nag;
+  const int alo = (int)((long)nb * ag / nag), ahi = (int)((long)nb * (ag + 1) / nag);  // terms of this CTA
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm_tab + (ahi - alo) * nm1);
   const int c = threadIdx.x % TC, j = threadIdx.x / TC;
   const Lay L{reinterpret_cast<float2*>(smraw), c};
   const int cc = blockIdx.x * TC + c;
   const int k1 = blockIdx.y;
-  const int b = blockIdx.z;
   const int n1 = wrapn(k1, N);
   const int warp = threadIdx.x >> 5;
   if (warp == 0) tmem_alloc(tslot, CF::NCOLS);
-  for (int i = threadIdx.x; i < nb * nm1; i += blockDim.x) sm_tab[i] = phitab[(long)alpha0 * nm1 + i];
+  for (int i = threadIdx.x; i < (ahi - alo) * nm1; i += blockDim.x) sm_tab[i] = phitab[(long)(alpha0 + alo) * nm1 + i];
   const float2* pb = phi + ((long)b * N * N + k1) * NH;  // + k0 * N * NH + k2
   if (blockIdx.x == 0) {
     for (int k0 = threadIdx.x; k0 < N; k0 += blockDim.x) {
@@ -1256,8 +1268,9 @@ __global__ void __launch_bounds__(P1TCfg<N>::THREADS, 3) k_p1_tm(const float2* _
   }
   const long fstride = (long)N * N * H;  // one field
   const float fj = (float)j;
-  for (int a = 0; a < nb; ++a) {
-    const float* tab = sm_tab + a * nm1;
+  const int cs = cc ^ ((k1 & 1) * swz);
+  for (int a = alo; a < ahi; ++a) {
+    const float* tab = sm_tab + (a - alo) * nm1;
 #pragma unroll 1
     for (int D = 0; D < 2; ++D) {
       float2 v[E];
@@ -1313,7 +1326,7 @@ __global__ void __launch_bounds__(P1TCfg<N>::THREADS, 3) k_p1_tm(const float2* _
       }
       if constexpr (N <= 256) fft_pencil_tw8_tm<N, Lay, SyncBlock>(v, j, L, tw, tbase + 48, SyncBlock());
       else fft_pencil<float, N, E, +1, Lay, SyncBlock>(v, j, L, tw, SyncBlock());
-      float2* dst = (D ? Tb : Ta) + ((long)b * nb + a) * fstride + (long)k1 * H + cc;
+      float2* dst = (D ? Tb : Ta) + ((long)b * nb + a) * fstride + (long)k1 * H + cs;
 #pragma unroll
       for (int r = 0; r < E; ++r) dst[(long)(j + r * P) * N * H] = v[r];
     }
@@ -1324,10 +1337,409 @@ __global__ void __launch_bounds__(P1TCfg<N>::THREADS, 3) k_p1_tm(const float2* _
   if (warp == 0) tmem_dealloc(*tslot, CF::NCOLS);
 }
 
-// F2: forward DFT along axis 1 of F[b][comp][a0][a1][k2] (k2 = 0..n_c), keeping n1 in [n1lo, n1lo + nk1).
+// ---------------------------------------------------------------- second and last inverse pass in one kernel
+// P23 (FP32, N = 64): from Ta, Tb (the first pass's output for all terms) straight to the product, without storing the
+// three fields per term that k_p2 hands to the last pass.  A CTA owns one plane a0, 64 x 64 points, whose six product
+// components stay in tensor memory for the whole sum over its group of term pairs.
+//   Z_A = (i n2^D - n1^D) Ta^a  -> g2^a + i g1^a      Z_0 = Tb^a + i Tb^{a+1}  -> g0^a + i g0^{a+1}
+// over the full range of k2 (the half spectrum is mirrored as it is read), so a term pair costs three complex 2-D
+// transforms.
+//   - Planes [k1][c] (16 KB) arrive by cp.async.bulk in a ring of NSLOT; their columns are stored as c ^ 8 (k1 mod 2), so
+//     that the two rows of a half warp fall into different halves of the banks.
+//   - Axis 1: a warp takes 8 columns of k2, thread (c, j) 16 of the 64 points (radix 16 then 4); its exchange uses the
+//     memory that holds the rows the warp owns afterwards, so only warp barriers are needed.
+//   - Rows: the transformed columns go to the row buffer (two block barriers a transform, the only ones), a warp owns
+//     8 rows, and the exchange of the row transform (radix 16 then 4) is in place.
+// Bounded waits, error flag and the drain before exit as in k_p3.
+// What bounds it: the shared-memory path (ncu, 50 terms of one realisation: 277 wavefronts a warp and transform, 62 % of
+// the path's cycles while active) with 16 warps a SM, issue 50 %; DRAM 17 %.  Four groups of term pairs fill the SMs for
+// one realisation (64 planes, two CTAs a SM).  50 terms of one realisation take 82 us (k_p2 122 + k_p3 94 before), of
+// eight 496 us (664 + 358).  The same split at N = 128 (two residue classes of a1 per plane) was slower than the three
+// passes there (715 against 690 us): its shared-memory traffic grows while HBM already carries the passes.
+template <int N>
+struct P23Cfg {
+  static_assert(N == 64, "one plane per CTA, two CTAs per SM");
+  static constexpr int H = N / 2, M = 64, E = 16;
+  static constexpr int THREADS = M * N / E, WARPS = THREADS / 32;  // 256, 8
+  static constexpr int P = N / E;             // threads per row: 4
+  static constexpr int RPW = M / WARPS;       // rows per warp: 8
+  static constexpr int NSLOT = 3;
+  static constexpr int TILE = N * H;          // complex values of one plane
+  static constexpr uint32_t NCOLS = 128 * (WARPS / 4);  // per warp: 96 accumulators, 32 for row twiddles
+  static constexpr int CTAS = 2;
+  // Row buffer: element p of a row at p + 2 (p / 16) (16-byte pairs of the radix-16 outputs), rows PITCH apart, the rows
+  // of a warp in bit-reversed order.  PITCH mod 16 = 16 / RPW, so the RPW rows x (16 / RPW) threads of a half warp
+  // read 16 different 8-byte banks, and the two rows of a half warp's column store lie 8 banks apart.
+  static constexpr int PITCH = 82;
+  static constexpr size_t SMEM = (size_t)NSLOT * TILE * 8 + (size_t)M * PITCH * 8 + (size_t)N * 8 + 64;
+  static __host__ __device__ constexpr int slot_of(int row) {  // place of row a1 in the row buffer (its own inverse)
+    return (row & ~7) | ((row & 1) << 2) | (row & 2) | ((row >> 2) & 1);
+  }
+};
+
+template <int N> struct P23RowLay {
+  static constexpr bool SINGLE = true;
+  static constexpr bool VEC = true;
+  float2* base;
+  __device__ __forceinline__ float2* buf(int) const { return base; }
+  __device__ __forceinline__ int idx(int p) const { return p + 2 * (p >> 4); }
+};
+
+// 32 consecutive columns of this thread's lane into registers (one wait).
+__device__ __forceinline__ void tmem_ld32(uint32_t t0, float (&v)[32]) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(t0)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) {
+  uint32_t r[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(v[i]);
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
+      "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
+      "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+
+template <int N>
+__global__ void __launch_bounds__(P23Cfg<N>::THREADS, P23Cfg<N>::CTAS) k_p23(
+    const float2* __restrict__ Ta, const float2* __restrict__ Tb, const float* __restrict__ sigma, int n_alpha,
+    float2* __restrict__ F, long fgstride, int n_c, const float2* __restrict__ tw, int* __restrict__ err,
+    long long wait_limit) {
+  using CF = P23Cfg<N>;
+  using RL = P23RowLay<N>;
+  constexpr int E = 16, H = CF::H, P = CF::P, RPW = CF::RPW, NSLOT = CF::NSLOT, PITCH = CF::PITCH;
+  constexpr int RLAST = N / 16, NB = 16 / RLAST;  // radix of the rows' last stage, butterflies per thread
+  extern __shared__ __align__(128) unsigned char smraw[];
+  float2* ring = reinterpret_cast<float2*>(smraw);
+  float2* rows = ring + NSLOT * CF::TILE;       // [64][PITCH]
+  float2* twN = rows + CF::M * PITCH;           // e^{+2 pi i k / N}
+  uint64_t* bars = reinterpret_cast<uint64_t*>(twN + N);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + NSLOT);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int a0 = blockIdx.x;
+  const int b = blockIdx.y;
+  const int allpairs = (n_alpha + 1) / 2;
+  const int pr0 = allpairs * (int)blockIdx.z / (int)gridDim.z;
+  const int pr1 = allpairs * ((int)blockIdx.z + 1) / (int)gridDim.z;
+  const int nterms = min(2 * pr1, n_alpha) - 2 * pr0;  // terms of this group
+  const int ntiles = 2 * nterms;
+  F += (long)blockIdx.z * fgstride;
+  const long fstride = (long)N * N * H;
+  const long poff = ((long)b * n_alpha + 2 * pr0) * fstride + (long)a0 * CF::TILE;
+  if (warp == 0) tmem_alloc(tslot, CF::NCOLS);
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < NSLOT; ++s) mbar_init(bars + s, 1);
+    mbar_init_fence();
+  }
+  for (int i = threadIdx.x; i < N; i += CF::THREADS) twN[i] = conjg<float>(__ldg(tw + i));
+  tmem_fence_before_sync();
+  __syncthreads();
+  tmem_fence_after_sync();
+  // Planes of this group in the order they are used: Tb^a, Tb^{a+1}, Ta^a, Ta^{a+1} of each pair.
+  auto issue = [&](int q) {  // thread 0
+    const int lp = q >> 2, left = nterms - 2 * lp;  // terms from this pair on
+    const int e = q & 3;
+    const bool two = left >= 2;
+    const int term = 2 * lp + (two ? (e & 1) : 0);
+    const bool isb = two ? e < 2 : e < 1;
+    const int s = q % NSLOT;
+    fence_proxy_async();
+    mbar_expect_tx(bars + s, CF::TILE * 8);
+    bulk_g2s(ring + s * CF::TILE, (isb ? Tb : Ta) + poff + (long)term * fstride, CF::TILE * 8, bars + s);
+  };
+  int issued = min(NSLOT, ntiles);  // planes whose copies thread 0 has issued
+  if (threadIdx.x == 0)
+    for (int q = 0; q < issued; ++q) issue(q);
+  const uint32_t tbase = *tslot + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(128 * (warp >> 2));
+  auto tcol = [&](int c) { return tbase + (uint32_t)(16 * c); };
+  // axis 1: column c2 of the full spectrum, points j + 4 r;  rows: place 8 warp + rr, points jj + P r
+  const int c8 = lane & 7, j = lane >> 3, jo = j & 1;
+  const int c2 = 8 * warp + c8;
+  const int cm = c2 == H ? 0 : (c2 > H ? N - c2 : c2);  // stored column
+  const float fn2 = c2 < H ? (float)c2 : (c2 == H ? 0.f : (float)(c2 - N));
+  const float fj = (float)j;
+  const int jj = lane / RPW, rr = lane % RPW;
+  const RL L{rows + (warp * RPW + rr) * PITCH};
+  const int arow = CF::slot_of(warp * RPW + rr);  // a1 of this row
+  // plane offsets of (k1 = j, stored column) and, mirrored, of (N - j, column); k1 steps of 4 are constants
+  const int od = j * H + (cm ^ (jo << 3)), om = (N - j) * H + (cm ^ (jo << 3));
+  const int om0 = j == 0 ? cm : om;  // mirrored k1 = 0
+  // axis-1 exchange in the warp's own rows: point p of column c at 8 (p ^ (p / 16 mod 2)) + c, so that two threads of a
+  // pencil (16 or 1 points apart) fall into different halves of the banks
+  float2* const xb = rows + warp * (RPW * PITCH) + c8;
+  float2* const xw0 = xb + 8 * (16 * j + jo);
+  float2* const xw1 = xb + 8 * (16 * j + 1 - jo);
+  const float2* const xr0 = xb + 8 * j;
+  const float2* const xr1 = xb + 8 * (j ^ 1);
+  // column stores: row a1 = j + 4 m
+  float2* const zc0 = rows + CF::slot_of(j) * PITCH + c2 + 2 * (c2 >> 4);
+  {
+    float z0[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) z0[i] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) tmem_st16(tcol(c), z0);
+    // last-stage row twiddles: W_N^{r k}, k = (jj + t P) mod 16
+    float w[2][16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) w[0][i] = w[1][i] = 0.f;
+#pragma unroll
+    for (int t = 0; t < NB; ++t)
+#pragma unroll
+      for (int r = 1; r < RLAST; ++r) {
+        const int q = t * (RLAST - 1) + r - 1;
+        const float2 x = twN[r * ((jj + t * P) & 15)];
+        w[q >> 3][2 * (q & 7)] = x.x;
+        w[q >> 3][2 * (q & 7) + 1] = x.y;
+      }
+    tmem_st16(tcol(6), w[0]);
+    tmem_st16(tcol(7), w[1]);
+    tmem_wait_st();
+  }
+  // Stored value behind the full spectrum at (k1 = j + 4 r, c2); MIR: from (-k1, -c2), to be conjugated by the caller;
+  // SPEC: the warp holds c2 = 0 or c2 = N/2, both unpacked from column 0 (X(k1, 0) + i X(k1, N/2)).
+  auto spec = [&](auto mir, auto special, const float2* t, int r) -> float2 {
+    constexpr bool MIR = decltype(mir)::value, SPEC = decltype(special)::value;
+    float2 x = MIR ? t[r == 0 ? om0 : om - 4 * r * H] : t[od + 4 * r * H];
+    if (SPEC && cm == 0) {  // one lane column
+      const int k1 = j + 4 * r, ko = MIR ? k1 : (N - k1) & (N - 1);
+      const float2 o = t[ko * H + (jo << 3)];
+      // X(k1, 0) = (Y + conj Y-) / 2; X(k1, N/2) = -i (Y - conj Y-) / 2, here conjugated for the mirrored caller
+      x = MIR ? make_float2(0.5f * (o.y + x.y), 0.5f * (o.x - x.x)) : make_float2(0.5f * (x.x + o.x), 0.5f * (x.y - o.y));
+    }
+    return x;
+  };
+  // the 16 axis-1 inputs of a transform: Z_0 (FIRST) from two planes or Z_A from one
+  auto load = [&](auto mir, auto special, auto first, float2 (&v)[E], const float2* t0, const float2* t1) {
+    constexpr bool MIR = decltype(mir)::value, FIRST = decltype(first)::value;
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+      const float2 x = spec(mir, special, t0, r);
+      if constexpr (FIRST) {
+        const float2 y = t1 ? spec(mir, special, t1, r) : make_float2(0.f, 0.f);
+        v[r] = MIR ? make_float2(x.x + y.y, y.x - x.y) : make_float2(x.x - y.y, x.y + y.x);
+      } else {
+        const float n = r < 8 ? fj + (float)(4 * r) : ((r == 8 && j == 0) ? 0.f : fj + (float)(4 * r - 64));
+        const float2 d = __fmul2_rn(x, make_float2(n, n));
+        v[r] = MIR ? make_float2(fmaf(fn2, x.y, -d.x), fmaf(fn2, x.x, d.y))
+                   : make_float2(fmaf(-fn2, x.y, -d.x), fmaf(fn2, x.x, -d.y));
+      }
+    }
+  };
+  auto load_any = [&](auto first, float2 (&v)[E], const float2* t0, const float2* t1) {
+    const std::true_type yes{};
+    const std::false_type no{};
+    if (warp == 0) load(no, yes, first, v, t0, t1);
+    else if (warp < H / 8) load(no, no, first, v, t0, t1);
+    else if (warp == H / 8) load(yes, yes, first, v, t0, t1);
+    else load(yes, no, first, v, t0, t1);
+  };
+  bool ok = true;
+  int q = 0;  // planes used so far
+  for (int lp = 0; 2 * lp < nterms; ++lp) {
+    const bool two = nterms - 2 * lp >= 2;
+    float2 zB[E];
+    const float* sg = sigma + 2 * (pr0 + lp);
+#pragma unroll 1
+    for (int ph = 0; ph < (two ? 3 : 2); ++ph) {
+      float2 v[E];
+      const int used = (ph == 0 && two) ? 2 : 1;
+      for (int u = 0; u < used; ++u)
+        if (ok) ok = mbar_wait(bars + (q + u) % NSLOT, (uint32_t)(((q + u) / NSLOT) & 1), err, wait_limit);
+      const float2* t0 = ring + (q % NSLOT) * CF::TILE;
+      if (ph == 0) load_any(std::true_type{}, v, t0, two ? ring + ((q + 1) % NSLOT) * CF::TILE : nullptr);
+      else load_any(std::false_type{}, v, t0, nullptr);
+      // ---- axis 1, 64 points: radix 16, exchange, radix 4
+      dftR<float, +1, E>(v);
+      __syncwarp();  // the warp's rows of the transform before have been read
+#pragma unroll
+      for (int r = 0; r < E; ++r) (r & 1 ? xw1 : xw0)[16 * (r >> 1)] = v[r];
+      __syncwarp();
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        float2 a[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) a[r] = (r & 1 ? xr1 : xr0)[8 * (4 * t + 16 * r)];
+#pragma unroll
+        for (int r = 1; r < 4; ++r) a[r] = mul<float>(a[r], twN[r * j + 4 * r * t]);
+        dftR<float, +1, 4>(a);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[t + 4 * r] = a[r];
+      }
+      __syncthreads();  // every exchange and every plane read is over
+      if (threadIdx.x == 0 && ok) {
+        for (int u = 0; u < used; ++u)
+          if (q + u + NSLOT < ntiles) {
+            issue(q + u + NSLOT);
+            issued = q + u + NSLOT + 1;
+          }
+      }
+      q += used;
+#pragma unroll
+      for (int m = 0; m < E; ++m)  // row a1 = j + 4 m, column c2
+        zc0[(CF::slot_of(4 * m)) * PITCH] = v[m];
+      __syncthreads();
+      // ---- rows: radix 16, exchange in place, radix 4
+#pragma unroll
+      for (int r = 0; r < E; ++r) v[r] = L.base[jj + L.idx(P * r)];
+      dftR<float, +1, E>(v);
+      __syncwarp();
+#pragma unroll
+      for (int m = 0; m < E / 2; ++m)
+        *reinterpret_cast<float4*>(L.base + 18 * jj + 2 * m) =
+            make_float4(v[2 * m].x, v[2 * m].y, v[2 * m + 1].x, v[2 * m + 1].y);
+      __syncwarp();
+      {
+        float w[32];
+        tmem_ld32(tcol(6), w);
+#pragma unroll
+        for (int t = 0; t < NB; ++t) {
+          float2 a[RLAST];
+#pragma unroll
+          for (int r = 0; r < RLAST; ++r) a[r] = L.base[jj + t * P + 18 * r];
+#pragma unroll
+          for (int r = 1; r < RLAST; ++r) {
+            const int i = t * (RLAST - 1) + r - 1;
+            a[r] = mul<float>(a[r], make_float2(w[2 * i], w[2 * i + 1]));
+          }
+          dftR<float, +1, RLAST>(a);
+#pragma unroll
+          for (int r = 0; r < RLAST; ++r) v[t + r * NB] = a[r];
+        }
+      }
+      if (ph == 0) {
+#pragma unroll
+        for (int r = 0; r < E; ++r) zB[r] = v[r];
+        continue;
+      }
+      // ---- the term's products: v = (g2, g1), g0 = Re or Im of zB.  Columns: s00, s12 (16 each), (s22, s11) and
+      // (s02, s01) interleaved (32 each).
+      const float sa = __ldg(sg + ph - 1);
+      if (ph == 2) {
+#pragma unroll
+        for (int r = 0; r < E; ++r) zB[r].x = zB[r].y;
+      }
+      {
+        float u[32];
+        tmem_ld32(tcol(0), u);
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+          u[r] = fmaf(sa * zB[r].x, zB[r].x, u[r]);
+          u[16 + r] = fmaf(sa * v[r].y, v[r].x, u[16 + r]);
+        }
+        tmem_st32(tcol(0), u);
+      }
+      {
+        float u[32];
+        tmem_ld32(tcol(2), u);
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+          const float2 c = __ffma2_rn(__fmul2_rn(v[r], make_float2(sa, sa)), v[r], make_float2(u[2 * r], u[2 * r + 1]));
+          u[2 * r] = c.x;
+          u[2 * r + 1] = c.y;
+        }
+        tmem_st32(tcol(2), u);
+        tmem_ld32(tcol(4), u);
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+          const float t0s = sa * zB[r].x;
+          const float2 d = __ffma2_rn(make_float2(t0s, t0s), v[r], make_float2(u[2 * r], u[2 * r + 1]));
+          u[2 * r] = d.x;
+          u[2 * r + 1] = d.y;
+        }
+        tmem_st32(tcol(4), u);
+      }
+      tmem_wait_st();
+    }
+  }
+  if (threadIdx.x == 0) {  // the last copy issued into each slot has landed before the CTA may exit
+    for (int s = 0; s < NSLOT && s < issued; ++s) {
+      const int last = s + ((issued - 1 - s) / NSLOT) * NSLOT;
+      mbar_wait(bars + s, (uint32_t)((last / NSLOT) & 1), err);
+    }
+  }
+  // ---- forward R2C of the six real rows along axis 2, two per complex transform: (s00, s11), (s22, s01), (s02, s12)
+  __syncwarp();
+  const long row = (long)a0 * N + arow;
+  const int ncp = n_c + 1;
+#pragma unroll 1
+  for (int h3 = 0; h3 < 3; ++h3) {
+    float2 z[E];
+    {
+      float u[16], w[16];
+      if (h3 == 0) {
+        tmem_ld16(tcol(0), u);
+#pragma unroll
+        for (int r = 0; r < E; ++r) z[r].x = u[r];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          tmem_ld16(tcol(2) + 16 * h, w);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) z[8 * h + i].y = w[2 * i + 1];
+        }
+      } else if (h3 == 1) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          tmem_ld16(tcol(2) + 16 * h, u);
+          tmem_ld16(tcol(4) + 16 * h, w);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) z[8 * h + i] = make_float2(u[2 * i], w[2 * i + 1]);
+        }
+      } else {
+        tmem_ld16(tcol(1), u);
+#pragma unroll
+        for (int r = 0; r < E; ++r) z[r].y = u[r];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          tmem_ld16(tcol(4) + 16 * h, w);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) z[8 * h + i].x = w[2 * i];
+        }
+      }
+    }
+    fft_pencil<float, N, E, -1, RL, SyncWarp>(z, jj, L, tw, SyncWarp());
+#pragma unroll
+    for (int r = 0; r < E; ++r) L.base[L.idx(jj + r * P)] = z[r];
+    __syncwarp();
+    // stored component order of F: (00, 11, 22, 01, 02, 12) = 0..5
+    float2* f1 = F + (((long)b * 6 + 2 * h3) * N * N + row) * ncp;
+    float2* f2 = f1 + (long)N * N * ncp;
+    for (int k = jj; k <= n_c; k += P) {
+      const float2 zk = L.base[L.idx(k)];
+      const float2 zm = conjg<float>(L.base[L.idx((N - k) & (N - 1))]);
+      f1[k] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y + zm.y));
+      f2[k] = make_float2(0.5f * (zk.y - zm.y), -0.5f * (zk.x - zm.x));
+    }
+    __syncwarp();
+  }
+  tmem_fence_before_sync();
+  __syncthreads();
+  tmem_fence_after_sync();
+  if (warp == 0) tmem_dealloc(*tslot, CF::NCOLS);
+}
+
+// F2: forward DFT along axis 1 of F[b][comp][a0][a1][k2] (k2 = 0..n_c), keeping n1 in [n1lo, n1lo + nk1).  F is the
+// sum, in order, of `parts` partial fields fgstride elements apart (one per term group of the pass before).
 template <typename T, int N>
-__global__ void __launch_bounds__(256) k_f2(const cx<T>* __restrict__ F, cx<T>* __restrict__ F2, int n_c, int n1lo,
-                                            int nk1, const cx<T>* __restrict__ tw) {
+__global__ void __launch_bounds__(256) k_f2(const cx<T>* __restrict__ F, int parts, long fgstride,
+                                            cx<T>* __restrict__ F2, int n_c, int n1lo, int nk1,
+                                            const cx<T>* __restrict__ tw) {
   using SH = Shape<T, N>;
   constexpr int E = SH::ES, P = SH::PS, TC = SH::TC;
   // one exchange buffer (a CTA runs one transform): half the shared memory of two, so more CTAs share an SM
@@ -1344,6 +1756,12 @@ __global__ void __launch_bounds__(256) k_f2(const cx<T>* __restrict__ F, cx<T>* 
   cx<T> v[E];
 #pragma unroll
   for (int r = 0; r < E; ++r) v[r] = valid ? in[(long)(j + r * P) * ncp] : mk<T>((T)0, (T)0);
+  for (int g = 1; g < parts; ++g) {
+    in += fgstride;
+#pragma unroll
+    for (int r = 0; r < E; ++r)
+      if (valid) v[r] = add<T>(v[r], in[(long)(j + r * P) * ncp]);
+  }
   fft_pencil<T, N, E, -1, Lay, SyncBlock, false>(v, j, L, tw, SyncBlock());
   if (valid) {
     cx<T>* out = F2 + (bc * N + a0) * (long)nk1 * ncp + cc;

@@ -67,27 +67,38 @@ struct OpsT {
     return cudaGetLastError();
   }
   // ------------------------------------------------------------ hot path
+  // CTAs that share the nb terms of one first-pass tile: enough for about four waves of the 456 CTAs that fit the SMs
+  // (three a SM), at least four terms each, so that the tile's set-up (Phi~, cells, twiddles) stays small against its
+  // transforms.  One realisation at N = 64 has 64 tiles: 50 terms took 114 us on 64 SMs (five launches), 37 us in 768
+  // CTAs; FP64 N = 32 (32 tiles of 64 threads) 119 us for 10 terms, 45 us for 16.  From 256^3 on there is one group.
+  static int p1_groups(long tiles, int nb) {
+    const long want = (1700 + tiles - 1) / tiles;
+    const int most = nb / 4 < 1 ? 1 : nb / 4;
+    return (int)(want < most ? want : most);
+  }
   template <int N, int E, int TC>
   static cudaError_t p1_v(const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* phitab, int nm1,
-                          int alpha0, int nb, int batch, const void* tw, cudaStream_t st) {
-    const size_t sm = strided_bytes<N, TC, E>() + N * sizeof(C) + N * sizeof(int) + (size_t)nb * nm1 * sizeof(T);
+                          int alpha0, int nb, int batch, const void* tw, int swz, cudaStream_t st) {
+    const int nag = p1_groups((long)(N / 2) / TC * N * batch, nb), per = (nb + nag - 1) / nag;
+    const size_t sm = strided_bytes<N, TC, E>() + N * sizeof(C) + N * sizeof(int) + (size_t)per * nm1 * sizeof(T);
     auto k = k_p1<T, N, E, TC>;
     SIGW_CHECK_LAUNCH(allow_smem(k, 227 * 1024));
-    dim3 grid((N / 2) / TC, N, batch);
-    k<<<grid, TC * (N / E), sm, st>>>((const C*)phi, (C*)Ta, (C*)Tb, lut, (const T*)phitab, nm1, alpha0, nb,
+    dim3 grid((N / 2) / TC, N, batch * nag);
+    k<<<grid, TC * (N / E), sm, st>>>((const C*)phi, (C*)Ta, (C*)Tb, lut, (const T*)phitab, nm1, alpha0, nb, nag, swz,
                                       (const C*)tw);
     return cudaGetLastError();
   }
   template <int N>
   static cudaError_t p1_tm_v(const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* phitab, int nm1,
-                             int alpha0, int nb, int batch, const void* tw, cudaStream_t st) {
+                             int alpha0, int nb, int batch, const void* tw, int swz, cudaStream_t st) {
     using CF = P1TCfg<N>;
-    const size_t sm = CF::smem(nb, nm1);
+    const int nag = p1_groups((long)(N / 2) / CF::TC * N * batch, nb), per = (nb + nag - 1) / nag;
+    const size_t sm = CF::smem(per, nm1);
     auto k = k_p1_tm<N>;
     SIGW_CHECK_LAUNCH(allow_smem(k, 227 * 1024));
-    dim3 grid((N / 2) / CF::TC, N, batch);
+    dim3 grid((N / 2) / CF::TC, N, batch * nag);
     k<<<grid, CF::THREADS, sm, st>>>((const float2*)phi, (float2*)Ta, (float2*)Tb, lut, (const float*)phitab, nm1,
-                                     alpha0, nb, (const float2*)tw);
+                                     alpha0, nb, nag, swz, (const float2*)tw);
     return cudaGetLastError();
   }
   template <int N>
@@ -95,14 +106,52 @@ struct OpsT {
                           int alpha0, int nb, int batch, const void* tw, int variant, cudaStream_t st) {
     using SH = Shape<T, N>;
     using AL = AltStrided<T, N>;
+    const int swz = fused_n<N>(variant) ? 8 : 0;  // the fused second and last pass reads swizzled columns
     if constexpr (sizeof(T) == 4 && (N == 128 || N == 256 || N == 512)) {  // Phi~ tile and cells in tensor memory
-      if (variant & 16) return p1_tm_v<N>(phi, Ta, Tb, lut, phitab, nm1, alpha0, nb, batch, tw, st);
+      if (variant & 16) return p1_tm_v<N>(phi, Ta, Tb, lut, phitab, nm1, alpha0, nb, batch, tw, swz, st);
     }
     if constexpr (AL::exists) {
       if (variant & 1)
-        return p1_v<N, AL::E, AL::TC>(phi, Ta, Tb, lut, phitab, nm1, alpha0, nb, batch, tw, st);
+        return p1_v<N, AL::E, AL::TC>(phi, Ta, Tb, lut, phitab, nm1, alpha0, nb, batch, tw, swz, st);
     }
-    return p1_v<N, SH::ES, SH::TC>(phi, Ta, Tb, lut, phitab, nm1, alpha0, nb, batch, tw, st);
+    return p1_v<N, SH::ES, SH::TC>(phi, Ta, Tb, lut, phitab, nm1, alpha0, nb, batch, tw, swz, st);
+  }
+  template <int N>
+  static constexpr bool fused_n(int variant) {
+    return sizeof(T) == 4 && N == 64 && (variant & 8);
+  }
+  template <int N>
+  static cudaError_t p23_n(const void* Ta, const void* Tb, const void* sigma, int n_alpha, void* F, int groups, int n_c,
+                           int batch, const void* tw, int* err, long long wait_limit, cudaStream_t st) {
+    if constexpr (sizeof(T) == 4 && N == 64) {
+      using CF = P23Cfg<N>;
+      auto k = k_p23<N>;
+      SIGW_CHECK_LAUNCH(allow_smem(k, CF::SMEM));
+      dim3 grid(N, batch, groups);
+      k<<<grid, CF::THREADS, CF::SMEM, st>>>((const float2*)Ta, (const float2*)Tb, (const float*)sigma, n_alpha,
+                                             (float2*)F, 6L * batch * N * N * (n_c + 1), n_c, (const float2*)tw, err,
+                                             wait_limit);
+      return cudaGetLastError();
+    } else {
+      return cudaErrorInvalidValue;
+    }
+  }
+  // Groups of term pairs the last pass splits a launch into (each writes a partial F, which the second forward pass
+  // adds up): enough for the SMs where one realisation has few tiles.  Not a function of the batch, so a
+  // realisation's sums are grouped the same way, and have the same bits, alone and in a batch.
+  template <int N>
+  static int last_groups_n(int variant, int n_alpha) {
+    long tiles, slots;
+    if (fused_n<N>(variant)) {
+      tiles = N;
+      slots = 304;
+    } else {
+      using CF = P3Cfg<T, N, ((N >= 16) ? 8 : 4)>;
+      tiles = (long)N * N / CF::RPC;
+      slots = 152;
+    }
+    const long g = slots / tiles, pairs = (n_alpha + 1) / 2;
+    return (int)(g < 1 ? 1 : (g > 8 ? (pairs < 8 ? pairs : 8) : (g > pairs ? pairs : g)));
   }
   template <int N, int E, int TC>
   static cudaError_t p2_v(const void* Ta, const void* Tb, void* W, int n_alpha, int alpha0, int nb, int batch,
@@ -125,14 +174,14 @@ struct OpsT {
     return p2_v<N, SH::ES, SH::TC>(Ta, Tb, W, n_alpha, alpha0, nb, batch, tw, st);
   }
   template <int N, int E>
-  static cudaError_t p3_v(const void* W, const void* sigma, int n_alpha, void* F, int n_c, int batch, const void* tw,
-                          int* err, long long wait_limit, cudaStream_t st) {
+  static cudaError_t p3_v(const void* W, const void* sigma, int n_alpha, void* F, int groups, int n_c, int batch,
+                          const void* tw, int* err, long long wait_limit, cudaStream_t st) {
     using CF = P3Cfg<T, N, E>;
     auto k = k_p3<T, N, E>;
     SIGW_CHECK_LAUNCH(allow_smem(k, CF::SMEM));
-    dim3 grid((N * N) / CF::RPC, batch);
-    k<<<grid, CF::THREADS, CF::SMEM, st>>>((const C*)W, (const T*)sigma, n_alpha, (C*)F, n_c, (const C*)tw, err,
-                                           wait_limit);
+    dim3 grid((N * N) / CF::RPC, batch, groups);
+    k<<<grid, CF::THREADS, CF::SMEM, st>>>((const C*)W, (const T*)sigma, n_alpha, (C*)F, 6L * batch * N * N * (n_c + 1),
+                                           n_c, (const C*)tw, err, wait_limit);
     return cudaGetLastError();
   }
   template <int N>
@@ -147,15 +196,16 @@ struct OpsT {
     return cudaGetLastError();
   }
   template <int N>
-  static cudaError_t p3_n(const void* W, const void* sigma, int n_alpha, void* F, int n_c, int batch, const void* tw,
-                          int* err, long long wait_limit, int variant, cudaStream_t st) {
+  static cudaError_t p3_n(const void* W, const void* sigma, int n_alpha, void* F, int groups, int n_c, int batch,
+                          const void* tw, int* err, long long wait_limit, int variant, cudaStream_t st) {
     if constexpr (sizeof(T) == 4 && (N == 128 || N == 256 || N == 512)) {  // accumulators in tensor memory
       if (variant & 8) return p3_tm_v<N>(W, sigma, n_alpha, F, n_c, batch, tw, err, wait_limit, st);
     }
     if constexpr (AltP3<T, N>::exists) {
-      if (variant & 2) return p3_v<N, AltP3<T, N>::E>(W, sigma, n_alpha, F, n_c, batch, tw, err, wait_limit, st);
+      if (variant & 2)
+        return p3_v<N, AltP3<T, N>::E>(W, sigma, n_alpha, F, groups, n_c, batch, tw, err, wait_limit, st);
     }
-    return p3_v<N, ((N >= 16) ? 8 : 4)>(W, sigma, n_alpha, F, n_c, batch, tw, err, wait_limit, st);
+    return p3_v<N, ((N >= 16) ? 8 : 4)>(W, sigma, n_alpha, F, groups, n_c, batch, tw, err, wait_limit, st);
   }
   static void n1_range(int N, int n_c, int* lo, int* nk1) {
     const int H = N / 2;
@@ -165,7 +215,7 @@ struct OpsT {
     *nk1 = bhi - a + 1;
   }
   template <int N>
-  static cudaError_t f2_n(const void* F, void* F2, int n_c, int batch, const void* tw, cudaStream_t st) {
+  static cudaError_t f2_n(const void* F, int groups, void* F2, int n_c, int batch, const void* tw, cudaStream_t st) {
     using SH = Shape<T, N>;
     const size_t sm = (size_t)ColLayout<T, N, SH::TC, SH::ES, true>::SIZE * sizeof(C);  // single exchange buffer
     auto k = k_f2<T, N>;
@@ -173,7 +223,8 @@ struct OpsT {
     int lo, nk1;
     n1_range(N, n_c, &lo, &nk1);
     dim3 grid((n_c + 1 + SH::TC - 1) / SH::TC, N, batch * 6);
-    k<<<grid, SH::TC * SH::PS, sm, st>>>((const C*)F, (C*)F2, n_c, lo, nk1, (const C*)tw);
+    k<<<grid, SH::TC * SH::PS, sm, st>>>((const C*)F, groups, 6L * batch * N * N * (n_c + 1), (C*)F2, n_c, lo, nk1,
+                                         (const C*)tw);
     return cudaGetLastError();
   }
   template <int N>
@@ -325,14 +376,36 @@ cudaError_t OpsRT<T>::p2(int N, const void* Ta, const void* Tb, void* W, int n_a
   SIGW_DISPATCH_N(N, return (OpsT<T>::template p2_n<NN>(Ta, Tb, W, n_alpha, alpha0, nb, batch, tw, variant, st)));
 }
 template <typename T>
-cudaError_t OpsRT<T>::p3(int N, const void* W, const void* sigma, int n_alpha, void* F, int n_c, int batch,
+bool OpsRT<T>::fused(int N, int variant) {
+  return N == 64 && OpsT<T>::template fused_n<64>(variant);
+}
+template <typename T>
+int OpsRT<T>::last_groups(int N, int variant, int n_alpha) {
+  switch (N) {
+    case 8: return OpsT<T>::template last_groups_n<8>(variant, n_alpha);
+    case 16: return OpsT<T>::template last_groups_n<16>(variant, n_alpha);
+    case 32: return OpsT<T>::template last_groups_n<32>(variant, n_alpha);
+    case 64: return OpsT<T>::template last_groups_n<64>(variant, n_alpha);
+    case 128: return OpsT<T>::template last_groups_n<128>(variant, n_alpha);
+  }
+  return 1;
+}
+template <typename T>
+cudaError_t OpsRT<T>::p23(int N, const void* Ta, const void* Tb, const void* sigma, int n_alpha, void* F, int groups,
+                          int n_c, int batch, const void* tw, int* err, long long wait_limit, cudaStream_t st) {
+  if (N != 64) return cudaErrorInvalidValue;
+  return OpsT<T>::template p23_n<64>(Ta, Tb, sigma, n_alpha, F, groups, n_c, batch, tw, err, wait_limit, st);
+}
+template <typename T>
+cudaError_t OpsRT<T>::p3(int N, const void* W, const void* sigma, int n_alpha, void* F, int groups, int n_c, int batch,
                       const void* tw, int* err, long long wait_limit, int variant, cudaStream_t st) {
-  SIGW_DISPATCH_N(N, return (OpsT<T>::template p3_n<NN>(W, sigma, n_alpha, F, n_c, batch, tw, err, wait_limit,
+  SIGW_DISPATCH_N(N, return (OpsT<T>::template p3_n<NN>(W, sigma, n_alpha, F, groups, n_c, batch, tw, err, wait_limit,
                                                        variant, st)));
 }
 template <typename T>
-cudaError_t OpsRT<T>::f2(int N, const void* F, void* F2, int n_c, int batch, const void* tw, cudaStream_t st) {
-  SIGW_DISPATCH_N(N, return (OpsT<T>::template f2_n<NN>(F, F2, n_c, batch, tw, st)));
+cudaError_t OpsRT<T>::f2(int N, const void* F, int groups, void* F2, int n_c, int batch, const void* tw,
+                         cudaStream_t st) {
+  SIGW_DISPATCH_N(N, return (OpsT<T>::template f2_n<NN>(F, groups, F2, n_c, batch, tw, st)));
 }
 template <typename T>
 cudaError_t OpsRT<T>::f3(int N, const void* F2, int n_c, double* partial, long pbs, int batch, const void* tw,
