@@ -16,44 +16,13 @@
 #include <type_traits>
 
 #include "fft.cuh"
+#include "noise.cuh"
 #include "ops.h"
 
 namespace sigw {
 
 __device__ __forceinline__ int wrapn(int k, int N) { return k <= (N >> 1) ? k : k - N; }
 __device__ __forceinline__ int derivn(int k, int N) { return k == (N >> 1) ? 0 : wrapn(k, N); }
-
-// ---------------------------------------------------------------- Philox4x32-10 (SC'11)
-// counter (c0, c1, c2, c3), key (k0, k1); 10 rounds, Weyl key schedule between rounds.
-__device__ __forceinline__ void philox10(uint32_t& c0, uint32_t& c1, uint32_t& c2, uint32_t& c3, uint32_t k0,
-                                         uint32_t k1) {
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    if (r) {
-      k0 += 0x9E3779B9u;
-      k1 += 0xBB67AE85u;
-    }
-    const uint32_t lo0 = 0xD2511F53u * c0, hi0 = __umulhi(0xD2511F53u, c0);
-    const uint32_t lo1 = 0xCD9E8D57u * c2, hi1 = __umulhi(0xCD9E8D57u, c2);
-    const uint32_t n0 = hi1 ^ c1 ^ k0, n2 = hi0 ^ c3 ^ k1;
-    c0 = n0;
-    c1 = lo1;
-    c2 = n2;
-    c3 = lo0;
-  }
-}
-
-// N(0,1) draw for lattice cell `cell` (row-major linear index) and key `seed`: Box-Muller in FP64 on
-// two 53-bit uniforms made from the four output words, u1 in (0, 1], u2 in [0, 1).
-__device__ __forceinline__ double gauss_draw(uint32_t cell, uint64_t seed) {
-  uint32_t c0 = cell, c1 = 0u, c2 = 0u, c3 = 0u;
-  philox10(c0, c1, c2, c3, (uint32_t)(seed & 0xffffffffull), (uint32_t)(seed >> 32));
-  const uint64_t a = ((((uint64_t)c0) << 32) | c1) >> 11;
-  const uint64_t bb = ((((uint64_t)c2) << 32) | c3) >> 11;
-  const double u1 = ((double)a + 1.0) * 1.1102230246251565404e-16;  // 2^-53
-  const double u2 = (double)bb * 1.1102230246251565404e-16;
-  return sqrt(-2.0 * log(u1)) * cospi(2.0 * u2);
-}
 
 // ---------------------------------------------------------------- shapes
 template <typename T, int N> struct Shape {
@@ -141,8 +110,13 @@ __global__ void __launch_bounds__(256) k_rows_r2c(const T* __restrict__ R, cx<T>
     if (live) {
       if (MODE == 1) {
         const uint64_t sd = seeds[b];
-        x1 = (T)gauss_draw((uint32_t)(row0 * N + x), sd);
-        x2 = (T)gauss_draw((uint32_t)((row0 + 1) * N + x), sd);
+        if constexpr (sizeof(T) == 4) {
+          x1 = gauss_draw_f32((uint32_t)(row0 * N + x), sd);
+          x2 = gauss_draw_f32((uint32_t)((row0 + 1) * N + x), sd);
+        } else {
+          x1 = gauss_draw((uint32_t)(row0 * N + x), sd);
+          x2 = gauss_draw((uint32_t)((row0 + 1) * N + x), sd);
+        }
       } else {
         const long ro = ((long)b * N * N + row0) * N;
         const T* rb = R + ro;

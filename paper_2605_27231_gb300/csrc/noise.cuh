@@ -2,10 +2,11 @@
 //
 // gauss_draw evaluates it in FP64 (the FP64 path).  gauss_draw_f32 gives the same number rounded to FP32 (the FP32
 // path's noise) from pairs of FP32 values (an unevaluated sum hi + lo, about 48 bits): GB300 issues 64 FP32
-// operations for one FP64 operation, and the FP64 logarithm, root and cosine of every cell were 74-95 % of the
-// synthesis time from 256^3 on (512^3 noise + rows: see k_rows_r2c).  Both uniforms enter as the exact integers, and
-// the argument reductions are exact, so the relative error of the pair before the final rounding is below 2^-31
-// everywhere (also where the logarithm or the cosine is near zero).
+// operations for one FP64 operation, and the FP64 logarithm, root and cosine of every cell were most of the synthesis
+// (four USR realisations at 256^3: 9.5 -> 2.7 ms in all; one local one at 512^3: 20.6 -> 7.0 ms).  Both uniforms enter
+// as the exact integers, and the argument reductions are exact, so the relative error of the pair before the final
+// rounding is below 2^-30 everywhere, also where the logarithm or the cosine is near zero (2e7 draws against extended
+// precision: RMS error 0.288546 ulp of FP32, 0.288545 for the rounded FP64 value).
 #pragma once
 #ifdef __CUDACC__
 #include <cuda_runtime.h>
