@@ -93,7 +93,7 @@ Sizes sizes_of(int N, const sigw_opts& o) {
   s.lut = H * msq * sizeof(int16_t);
   s.tab = 2 * ((size_t)o.n_alpha * (o.n_modes + 1) + o.n_alpha) * rel;
   s.tw = (size_t)N * cel;
-  s.amp = mb * msq * rel + mb * sizeof(sigw::MapArgs);
+  s.amp = mb * msq * rel + mb * (sizeof(sigw::MapArgs) + sizeof(sigw::PzArgs));
   const int rb = o.precision == 64 ? sigw::OpsRT<double>::rows_blocks(N) : sigw::OpsRT<float>::rows_blocks(N);
   s.rows_sq = mb * ((size_t)rb * sizeof(double) + 2 * sizeof(double) + 2 * sizeof(uint64_t));
   return s;
@@ -129,7 +129,9 @@ struct sigw_plan_s {
   void* d_F = nullptr;
   void* d_F2 = nullptr;
   double* d_partial = nullptr;
+  void* d_res = nullptr;  // the error flag (16 bytes), then d_out: read back in one copy
   double* d_out = nullptr;
+  unsigned char* h_res = nullptr;  // pinned host copy of d_res
   int* d_shells = nullptr;
   double* d_Nk = nullptr;
   int16_t* d_lut = nullptr;
@@ -137,7 +139,9 @@ struct sigw_plan_s {
   void* d_sigma[2] = {nullptr, nullptr};
   void* d_tw = nullptr;
   void* d_amp = nullptr;            // [max_batch][msq_max + 1] synthesis amplitudes
+  unsigned char* d_gen = nullptr;   // one upload per sigw_generate: the next three arrays
   sigw::MapArgs* d_maps = nullptr;  // [max_batch] map parameters
+  sigw::PzArgs* d_pz = nullptr;     // [max_batch]
   double* d_sq = nullptr;
   double* d_mean = nullptr;
   unsigned long long* d_hits = nullptr;
@@ -295,8 +299,7 @@ std::vector<double> count_shell_modes(int N) {
   for (int a = -H + 1; a <= H; ++a)
     for (int b = -H + 1; b <= H; ++b) {
       const int base = a * a + b * b;
-      for (int v = 0; v <= H * H; ++v)
-        if (c2[v]) hist[base + v] += c2[v];
+      for (int n = 0; n <= H; ++n) hist[base + n * n] += c2[n * n];
     }
   std::vector<double> nk(H + 1, 0.0);
   for (int nc = 1; nc <= H; ++nc) {
@@ -479,7 +482,9 @@ sigw_status sigw_plan_create(int N, double L, const sigw_opts* opts, void* cuda_
   ALLOC(p->d_F, p->sz.F);
   ALLOC(p->d_F2, p->sz.F2);
   ALLOC(p->d_partial, p->sz.partial);
-  ALLOC(p->d_out, mb * H * 4 * sizeof(double));
+  ALLOC(p->d_res, 16 + mb * H * 4 * sizeof(double));
+  p->d_err = (int*)p->d_res;
+  p->d_out = (double*)((char*)p->d_res + 16);
   ALLOC(p->d_shells, H * sizeof(int));
   ALLOC(p->d_Nk, H * sizeof(double));
   ALLOC(p->d_lut, p->sz.lut);
@@ -489,17 +494,23 @@ sigw_status sigw_plan_create(int N, double L, const sigw_opts* opts, void* cuda_
   }
   ALLOC(p->d_tw, (size_t)N * cel);
   ALLOC(p->d_amp, mb * (p->msq_max + 1) * rel);
-  ALLOC(p->d_maps, mb * sizeof(sigw::MapArgs));
+  ALLOC(p->d_gen, mb * (sizeof(sigw::MapArgs) + sizeof(sigw::PzArgs) + sizeof(uint64_t)));
+  p->d_maps = (sigw::MapArgs*)p->d_gen;
+  p->d_pz = (sigw::PzArgs*)(p->d_maps + mb);
+  p->d_seeds = (uint64_t*)(p->d_pz + mb);
   const int rb = OPS(p, rows_blocks, N);
   ALLOC(p->d_sq, mb * rb * sizeof(double));
   ALLOC(p->d_mean, mb * sizeof(double));
   ALLOC(p->d_hits, mb * sizeof(unsigned long long));
-  ALLOC(p->d_seeds, mb * sizeof(uint64_t));
-  ALLOC(p->d_err, sizeof(int));
   ALLOC(p->d_shells_all, H * sizeof(int));
   ALLOC(p->d_Nk_all, H * sizeof(double));
 #undef ALLOC
   if (cudaMemset(p->d_err, 0, sizeof(int)) != cudaSuccess) return bail(SIGW_ECUDA);
+  if (cudaMallocHost((void**)&p->h_res, 16 + mb * H * 4 * sizeof(double)) != cudaSuccess) {
+    (void)cudaGetLastError();
+    p->h_res = nullptr;
+    return bail(SIGW_ENOMEM);
+  }
   // tables
   std::vector<unsigned char> buf;
   {
@@ -551,6 +562,7 @@ sigw_status sigw_plan_destroy(sigw_plan p) {
   if (p->st) cudaStreamSynchronize(p->st);
   if (p->graph) cudaGraphExecDestroy(p->graph);
   for (void* q : p->allocs) cudaFree(q);
+  if (p->h_res) cudaFreeHost(p->h_res);
   prof_reset(p);
   for (cudaEvent_t e : p->pool) cudaEventDestroy(e);
   if (p->own_stream && p->st) cudaStreamDestroy(p->st);
@@ -577,8 +589,12 @@ sigw_status sigw_synchronize(sigw_plan p) {
   return check_err_flag(p);
 }
 
-sigw_status sigw_generate_batch(sigw_plan p, const sigw_pzeta* pz, const sigw_ngmap* maps, const uint64_t* seeds,
-                                int batch, int64_t* usr_hits) {
+}  // extern "C" (a helper of the entry points follows)
+
+// sigw_generate_batch; without `wait` the work is only queued (for calls that follow on the plan's stream), and floor
+// hits are neither read back nor checked.
+static sigw_status generate_impl(sigw_plan p, const sigw_pzeta* pz, const sigw_ngmap* maps, const uint64_t* seeds,
+                                 int batch, int64_t* usr_hits, bool wait) {
   if (!p) return SIGW_EINVAL;
   if (!pz || !maps || !seeds || batch < 1 || batch > p->opts.max_batch)
     return fail(p, SIGW_EINVAL, "sigw_generate: bad arguments");
@@ -597,37 +613,30 @@ sigw_status sigw_generate_batch(sigw_plan p, const sigw_pzeta* pz, const sigw_ng
   const double L = p->L, dx = L / N, kf = 2.0 * kPi / L;
   const size_t NN = (size_t)N * N;
   const size_t msq1 = p->msq_max + 1;
-  // synthesis amplitude sqrt(P_zeta(k) dx^3) per integer |n|^2, P = 2 pi^2 Delta^2 / k^3 (Eq. eq_lognormal)
-  std::vector<double> amp(batch * msq1, 0.0);
-  std::vector<sigw::MapArgs> margs(batch);
+  cudaStream_t st = p->st;
+  // parameters of every realisation in one upload: maps, P_zeta, seeds (in the places of a full batch)
+  const size_t mb = p->opts.max_batch;
+  std::vector<unsigned char> buf(mb * (sizeof(sigw::MapArgs) + sizeof(sigw::PzArgs) + sizeof(uint64_t)));
+  sigw::MapArgs* margs = (sigw::MapArgs*)buf.data();
+  sigw::PzArgs* pargs = (sigw::PzArgs*)(margs + mb);
+  std::memcpy(pargs + mb, seeds, sizeof(uint64_t) * batch);
   for (int b = 0; b < batch; ++b) {
-    for (size_t msq = 1; msq <= p->msq_max; ++msq) {
-      const double k = kf * std::sqrt((double)msq);
-      const double lk = std::log(k / pz[b].kstar);
-      const double sg = pz[b].sigma;
-      const double d2 = pz[b].A / std::sqrt(2.0 * kPi * sg * sg) * std::exp(-lk * lk / (2.0 * sg * sg));
-      const double P = 2.0 * kPi * kPi * d2 / (k * k * k);
-      amp[b * msq1 + msq] = std::sqrt(P * dx * dx * dx);
-    }
+    pargs[b] = sigw::PzArgs{pz[b].A, pz[b].sigma, pz[b].kstar};
     const double ks2 = pz[b].kstar * pz[b].kstar;
     margs[b] = maps[b].kind == SIGW_MAP_NONLOCAL
                    ? sigw::MapArgs{maps[b].kind, maps[b].alpha_NL / ks2, maps[b].beta_NL / ks2, 1e-6}
                    : sigw::MapArgs{maps[b].kind, maps[b].F_NL, maps[b].G_NL,
                                    maps[b].usr_floor > 0 ? maps[b].usr_floor : 1e-6};
   }
-  std::vector<unsigned char> buf;
-  convert(amp, p->opts.precision, buf);
-  CKP(p, cudaMemcpyAsync(p->d_amp, buf.data(), buf.size(), cudaMemcpyHostToDevice, p->st), "upload amp");
-  CKP(p, cudaMemcpyAsync(p->d_maps, margs.data(), sizeof(sigw::MapArgs) * batch, cudaMemcpyHostToDevice, p->st),
-      "upload maps");
-  CKP(p, cudaMemcpyAsync(p->d_seeds, seeds, sizeof(uint64_t) * batch, cudaMemcpyHostToDevice, p->st), "upload seeds");
-  p->h2d += buf.size() + sizeof(uint64_t) * batch + sizeof(sigw::MapArgs) * batch;
+  CKP(p, cudaMemcpyAsync(p->d_gen, buf.data(), buf.size(), cudaMemcpyHostToDevice, st), "upload parameters");
+  p->h2d += buf.size();
+  RUN(p, 0, (double)batch * msq1 * p->relem(), "amplitudes",
+      sigw::launch_amp(p->d_pz, p->d_amp, (long)msq1, L, N, p->opts.precision, batch, st));
   const size_t cel = p->celem();
   char* work = (char*)p->d_work;
   void* Y = work;
   void* X = work + (size_t)p->opts.max_batch * NN * H * cel;
   void* R = (char*)X + (size_t)p->opts.max_batch * NN * (H + 1) * cel;
-  cudaStream_t st = p->st;
   const double Yb = (double)batch * NN * H * cel, Xb = (double)batch * NN * (H + 1) * cel;
   const double Rb = (double)batch * NN * N * p->relem();
   RUN(p, 0, Yb, "noise + rows R2C", OPS(p, rows_r2c_noise, N, Y, p->d_seeds, batch, p->d_tw, st));
@@ -673,6 +682,9 @@ sigw_status sigw_generate_batch(sigw_plan p, const sigw_pzeta* pz, const sigw_ng
     RUN(p, 0, Yb + Xb, "unpack (Phi)",
         OPS(p, unpack, N, Y, p->d_phi, batch, nullptr, 0L, (2.0 / 3.0) * dx * dx * dx, 1, st));
   }
+  p->generated = batch;
+  if (!wait) return SIGW_OK;
+  p->generated = 0;
   std::vector<unsigned long long> hits(batch, 0);
   if (any_usr) {
     CKP(p, cudaMemcpyAsync(hits.data(), p->d_hits, sizeof(unsigned long long) * batch, cudaMemcpyDeviceToHost, st),
@@ -688,6 +700,13 @@ sigw_status sigw_generate_batch(sigw_plan p, const sigw_pzeta* pz, const sigw_ng
   }
   if (any && p->opts.strict_domain) return fail(p, SIGW_EDOMAIN, "USR floor hits in strict mode");
   return SIGW_OK;
+}
+
+extern "C" {
+
+sigw_status sigw_generate_batch(sigw_plan p, const sigw_pzeta* pz, const sigw_ngmap* maps, const uint64_t* seeds,
+                                int batch, int64_t* usr_hits) {
+  return generate_impl(p, pz, maps, seeds, batch, usr_hits, true);
 }
 
 sigw_status sigw_generate(sigw_plan p, const sigw_pzeta* pz, const sigw_ngmap* map, const uint64_t* seeds, int batch,
@@ -821,6 +840,16 @@ static bool capture_all_shells(sigw_plan p, const std::vector<int>& sh) {
   }
   p->graph_batch = p->generated;
   return true;
+}
+
+// Wait for the stream and bring the error flag and the first n results (4 doubles each) to p->h_res.
+static sigw_status download_results(sigw_plan p, size_t n) {
+  CKP(p, cudaMemcpyAsync(p->h_res, p->d_res, 16 + n * 4 * sizeof(double), cudaMemcpyDeviceToHost, p->st),
+      "download results");
+  p->d2h += n * 4 * sizeof(double);
+  CKP(p, cudaStreamSynchronize(p->st), "spectrum");
+  if (*(const int*)p->h_res) return check_err_flag(p);
+  return SIGW_OK;
 }
 
 sigw_status sigw_spectrum_async(sigw_plan p, const int* shells, int n_shells, double* dev_out) {
@@ -978,15 +1007,8 @@ sigw_status sigw_spectrum(sigw_plan p, const int* shells, int n_shells, double* 
   if (s != SIGW_OK) return s;
   const int ns = shells ? n_shells : p->N / 2;
   const int batch = p->generated;
-  std::vector<double> host((size_t)batch * ns * 4);
-  CKP(p, cudaMemcpyAsync(host.data(), p->d_out, host.size() * sizeof(double), cudaMemcpyDeviceToHost, p->st),
-      "download results");
-  p->d2h += host.size() * sizeof(double);
-  CKP(p, cudaStreamSynchronize(p->st), "spectrum");
-  {
-    sigw_status fs = check_err_flag(p);
-    if (fs != SIGW_OK) return fs;
-  }
+  if ((s = download_results(p, (size_t)batch * ns)) != SIGW_OK) return s;
+  const double* host = (const double*)(p->h_res + 16);
   for (int i = 0; i < batch * ns; ++i) {
     if (PA) PA[i] = host[4 * i + 0];
     if (PB) PB[i] = host[4 * i + 1];
@@ -1213,20 +1235,50 @@ sigw_status sigw_target_scan(sigw_plan p, const sigw_pzeta* pz, const sigw_ngmap
                              const double* k, int n_k, double eps, double* omega, double* L_out, int* nc_out) {
   if (!p) return SIGW_EINVAL;
   if (!pz || !map || !k || n_k < 1) return fail(p, SIGW_EINVAL, "sigw_target_scan: bad arguments");
-  for (int i = 0; i < n_k; ++i) {
+  std::vector<double> box;
+  std::vector<int> nc;
+  while ((int)box.size() < n_k) {
     double L = 0.0;
-    int nc = 0;
-    if (sigw_target_box(p->N, k[i], pz, eps, &L, &nc) != SIGW_OK)
-      return fail(p, SIGW_EINVAL, "sigw_target_scan: bad target or P_zeta");
-    sigw_status s = sigw_plan_set_box(p, L);
-    if (s == SIGW_OK) s = sigw_generate(p, pz, map, &seed, 1, nullptr);
-    double om = 0.0;
-    if (s == SIGW_OK) s = sigw_spectrum(p, &nc, 1, &om, nullptr, nullptr, nullptr);
-    if (s != SIGW_OK) return s;
-    if (omega) omega[i] = om;
-    if (L_out) L_out[i] = L;
-    if (nc_out) nc_out[i] = nc;
+    int c = 0;
+    if (sigw_target_box(p->N, k[box.size()], pz, eps, &L, &c) != SIGW_OK || !std::isfinite(L)) break;
+    box.push_back(L);
+    nc.push_back(c);
   }
+  // Targets are queued one behind the other, each writing its own place of the results, and read back together (at
+  // most a plan's worth of results at a time).  Strict-domain plans wait for each realisation's floor hits.
+  const bool strict = p->opts.strict_domain && map->kind == SIGW_MAP_USR;
+  const int n_ok = (int)box.size(), most = p->N / 2;
+  if (n_ok) {
+    sigw_status s = sigw_plan_set_box(p, box[0]);
+    if (s != SIGW_OK) return s;
+  }
+  for (int i0 = 0; i0 < n_ok; i0 += most) {
+    const int n = std::min(most, n_ok - i0);
+    int queued = 0;
+    sigw_status s = SIGW_OK;
+    for (; queued < n; ++queued) {
+      const int i = i0 + queued;
+      p->L = box[i];
+      p->generated = 0;
+      if ((s = generate_impl(p, pz, map, &seed, 1, nullptr, strict)) != SIGW_OK) break;
+      if ((s = enqueue_spectrum(p, {nc[i]}, p->d_shells_all + nc[i] - 1, p->d_Nk_all + nc[i] - 1,
+                                p->d_out + 4 * queued)) != SIGW_OK)
+        break;
+    }
+    if (queued) {
+      const std::string msg = p->err;
+      const sigw_status d = download_results(p, queued);
+      if (d != SIGW_OK) return d;
+      p->err = msg;
+    }
+    for (int q = 0; q < queued; ++q) {
+      if (omega) omega[i0 + q] = ((const double*)(p->h_res + 16))[4 * q + 3];
+      if (L_out) L_out[i0 + q] = box[i0 + q];
+      if (nc_out) nc_out[i0 + q] = nc[i0 + q];
+    }
+    if (s != SIGW_OK) return s;
+  }
+  if (n_ok < n_k) return fail(p, SIGW_EINVAL, "sigw_target_scan: bad target or P_zeta");
   return SIGW_OK;
 }
 

@@ -1945,33 +1945,56 @@ __global__ void __launch_bounds__(256) k_subvol(const T* __restrict__ R, int N, 
 }
 
 #ifdef SIGW_COMMON_KERNELS
+// Synthesis amplitude sqrt(P_zeta(k) dx^3) per integer |n|^2 (k = k_f |n|), P_zeta = 2 pi^2 Delta^2 / k^3 with the
+// log-normal Delta^2 of Eq. eq_lognormal: amp[b][msq], msq = 0..msq_max (zero at 0).  Evaluated in FP64; on the host it
+// took longer than the rest of a call's host work (4 realisations at 256^3: 197 k logarithms and exponentials, 3.6 ms).
+template <typename T>
+__global__ void k_amp(const PzArgs* __restrict__ pz, T* __restrict__ amp, long msq1, double L, int N) {
+  const long msq = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (msq >= msq1) return;
+  const int b = blockIdx.y;
+  double v = 0.0;
+  if (msq > 0) {
+    const double pi = 3.14159265358979323846;
+    const double dx = L / N, sg = pz[b].sigma;
+    const double k = 2.0 * pi / L * sqrt((double)msq);
+    const double lk = log(k / pz[b].kstar);
+    const double d2 = pz[b].A / sqrt(2.0 * pi * sg * sg) * exp(-lk * lk / (2.0 * sg * sg));
+    v = sqrt(2.0 * pi * pi * d2 / (k * k * k) * dx * dx * dx);
+  }
+  amp[b * msq1 + msq] = (T)v;
+}
+
 // Deterministic second-stage reduction and the Omega constants:
 //   P_X = C^2 sum / (V N_k), C = 4 dx^3 / (n_c^2 V^2), Omega = k_c^3 / (48 pi^2) (P_A + P_B).
-__global__ void k_fin(const double* __restrict__ partial, long pbstride, int maxblk, int n_shells,
-                      const int* __restrict__ shells, const double* __restrict__ Nk, int N, double L, int tc3,
-                      double* __restrict__ out, int batch) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= batch * n_shells) return;
-  const int b = i / n_shells, s = i % n_shells;
+// One CTA per (realisation, shell), two warps per kernel: 64 threads add strided partials, then a
+// fixed tree.  (One thread per pair walked up to 33 k partials: 0.52 ms at 256^3, 1.04 ms at 512^3.)
+__global__ void __launch_bounds__(128) k_fin(const double* __restrict__ partial, long pbstride, int maxblk, int n_shells,
+                                             const int* __restrict__ shells, const double* __restrict__ Nk, int N,
+                                             double L, int tc3, double* __restrict__ out) {
+  __shared__ double red[4];
+  const int b = blockIdx.x / n_shells, s = blockIdx.x % n_shells;
   const int n_c = shells[s];
   const int H = N / 2;
   const int n1lo = max(-n_c, -H + 1), n1hi = min(n_c, H);
   const int nk1 = n1hi - n1lo + 1;
   const int nblk = ((n_c + 1 + tc3 - 1) / tc3) * nk1;
-  double sum[2];
-  for (int m = 0; m < 2; ++m) {
-    const double* p = partial + (long)b * pbstride + ((long)s * 2 + m) * maxblk;
-    double t = 0.0;
-    for (int k = 0; k < nblk; ++k) t += p[k];
-    sum[m] = t;
-  }
+  const int m = threadIdx.x >> 6;
+  const double* p = partial + (long)b * pbstride + ((long)s * 2 + m) * maxblk;
+  double t = 0.0;
+#pragma unroll 4
+  for (int k = threadIdx.x & 63; k < nblk; k += 64) t += p[k];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x) return;
   const double pi = 3.14159265358979323846;
   const double V = L * L * L, dx = L / N;
   const double C = 4.0 * dx * dx * dx / ((double)n_c * n_c * V * V);
   const double nk = Nk[s];
-  const double PA = C * C * sum[0] / (V * nk), PB = C * C * sum[1] / (V * nk);
+  const double PA = C * C * (red[0] + red[1]) / (V * nk), PB = C * C * (red[2] + red[3]) / (V * nk);
   const double kc = n_c * 2.0 * pi / L;
-  double* o = out + (long)i * 4;
+  double* o = out + (long)blockIdx.x * 4;
   o[0] = PA;
   o[1] = PB;
   o[2] = nk;

@@ -21,6 +21,10 @@ struct MapArgs {
   double F, G, floor;
 };
 
+struct PzArgs {  // P_zeta of one realisation (Eq. eq_lognormal)
+  double A, sigma, kstar;
+};
+
 template <typename T>
 struct OpsRT {
   // ---- synthesis chain (packed layout [b][a0][a1][N/2], standard layout [b][k0][k1][N/2+1])
@@ -87,5 +91,9 @@ extern template struct OpsRT<double>;
 cudaError_t launch_reduce_mean(const double* part, int nblk, double* mean, int batch, double inv, cudaStream_t st);
 cudaError_t launch_fin(const double* partial, long pbstride, int maxblk, int n_shells, const int* shells,
                        const double* Nk, int N, double L, int tc3, double* out, int batch, cudaStream_t st);
+
+// synthesis amplitudes amp[batch][msq1] in the plan precision
+cudaError_t launch_amp(const PzArgs* pz, void* amp, long msq1, double L, int N, int precision, int batch,
+                       cudaStream_t st);
 
 }  // namespace sigw

@@ -11,8 +11,15 @@ cudaError_t launch_reduce_mean(const double* part, int nblk, double* mean, int b
 
 cudaError_t launch_fin(const double* partial, long pbstride, int maxblk, int n_shells, const int* shells,
                        const double* Nk, int N, double L, int tc3, double* out, int batch, cudaStream_t st) {
-  const int n = batch * n_shells;
-  k_fin<<<(n + 127) / 128, 128, 0, st>>>(partial, pbstride, maxblk, n_shells, shells, Nk, N, L, tc3, out, batch);
+  k_fin<<<batch * n_shells, 128, 0, st>>>(partial, pbstride, maxblk, n_shells, shells, Nk, N, L, tc3, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_amp(const PzArgs* pz, void* amp, long msq1, double L, int N, int precision, int batch,
+                       cudaStream_t st) {
+  const dim3 grid((unsigned)((msq1 + 127) / 128), batch);
+  if (precision == 64) k_amp<double><<<grid, 128, 0, st>>>(pz, (double*)amp, msq1, L, N);
+  else k_amp<float><<<grid, 128, 0, st>>>(pz, (float*)amp, msq1, L, N);
   return cudaGetLastError();
 }
 }  // namespace sigw

@@ -57,3 +57,18 @@ def test_fused_pass_matches_three_passes(lib):
         p.set_tuning(16, 8)
         assert np.array_equal(p.spectrum()["omega"][0], fused)
     np.testing.assert_allclose(fused, three, rtol=2e-5)  # two FP32 evaluations of the same sums
+
+
+def test_scan_of_more_targets_than_shells(lib):
+    """A scan whose targets do not fit one read-back (N = 8 holds four results): the values of one-target scans, and a
+    bad target in the middle is refused after the ones before it were written."""
+    k = np.geomspace(0.3, 2.5, 11)
+    with lib.Plan(8, 1.0, precision=64, n_alpha=5) as p:
+        scan = p.target_scan(k, 1e-2, 0.5, 1.0, "local", 2.0, seed=3)
+        one = [p.target_scan([x], 1e-2, 0.5, 1.0, "local", 2.0, seed=3) for x in k]
+        assert p.L == one[-1]["L"][0]
+        with pytest.raises(lib.SigwError) as e:
+            p.target_scan([0.5, -1.0, 2.0], 1e-2, 0.5, 1.0)
+        assert e.value.status == lib.EINVAL
+    for key in ("omega", "L", "n_c"):
+        assert np.array_equal(scan[key], np.concatenate([o[key] for o in one]))
