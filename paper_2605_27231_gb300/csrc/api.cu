@@ -37,15 +37,26 @@ sigw::DecompParams params_of(const sigw_opts& o) {
   return p;
 }
 
-int auto_alpha_batch(int N, const sigw_opts& o) {
-  if (o.alpha_batch > 0) return std::min(o.alpha_batch, o.n_alpha);
-  return std::min(o.n_alpha, N <= 64 ? 16 : 10);
-}
-
-// Largest terms-per-launch the first-pass output buffer holds (the autotuner's largest candidate).
+// Terms per launch of the first and second pass: what the options fix, else at most 16 (the autotuner's largest
+// candidate and the untuned choice).
 int max_alpha_batch(const sigw_opts& o) {
   if (o.alpha_batch > 0) return std::min(o.alpha_batch, o.n_alpha);
   return std::min(o.n_alpha, 16);
+}
+
+// Terms the first-pass output buffer holds.  At N = 128 the largest choice, 16, stands for 25: a launch of 16 terms of
+// one realisation leaves the last of its few waves short (first pass, 50 terms: 253 us in fours of 16, 205 us in two
+// of 25; second pass 325 and 316 us).
+int buffer_terms(int N, const sigw_opts& o) {
+  const int b = max_alpha_batch(o);
+  return N == 128 && o.alpha_batch == 0 && b == 16 ? std::min(o.n_alpha, 25) : b;
+}
+
+// Terms per launch for the choice B: equal parts of at most B (N = 128: see buffer_terms).
+int launch_terms(int N, const sigw_opts& o, int B) {
+  const int most = B == max_alpha_batch(o) ? buffer_terms(N, o) : B;
+  const int launches = (o.n_alpha + most - 1) / most;
+  return (o.n_alpha + launches - 1) / launches;
 }
 
 // Process-wide autotuning results: (N, precision, realisations, n_alpha) -> (terms per launch, variant).
@@ -72,7 +83,7 @@ Sizes sizes_of(int N, const sigw_opts& o) {
   const size_t H = N / 2, NH = H + 1, NN = (size_t)N * N;
   const size_t rel = o.precision == 64 ? 8 : 4, cel = 2 * rel;
   const size_t mb = (size_t)o.max_batch;
-  const int B = max_alpha_batch(o);
+  const int B = buffer_terms(N, o);
   sigw::LaunchShape sh = o.precision == 64 ? sigw::OpsRT<double>::shape(N) : sigw::OpsRT<float>::shape(N);
   s.maxblk = sh.maxblk_f3;
   s.phi = mb * NN * NH * cel;
@@ -436,11 +447,11 @@ sigw_status sigw_plan_create(int N, double L, const sigw_opts* opts, void* cuda_
   p->N = N;
   p->L = L;
   p->opts = o;
-  p->B = auto_alpha_batch(N, o);
+  p->B = max_alpha_batch(o);
   // Untuned default: the choices measured fastest on GB300 (at 128^3 and 256^3 the first and the radix-16 last pass
   // with their per-thread state in tensor memory; at 512^3 the 512-specific strided passes and the tensor-memory
   // last pass).  sigw_plan_autotune or the table may override it.
-  p->variant = o.precision == 32 ? (N == 512 ? 15 : (N >= 128 ? 26 : (N == 64 ? 8 : 0))) : 0;
+  p->variant = o.precision == 32 ? (N == 512 ? 15 : (N == 256 ? 26 : (N == 128 ? 30 : (N == 64 ? 8 : 0)))) : 0;
   std::string e;
   if (!sigw::build_decomposition(params_of(o), &p->dec, &e)) {
     delete p;
@@ -742,8 +753,9 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, con
   const int var = p->variant;
   // the fused second and last pass takes the first pass's output of all terms, kept in W's place (it needs no W)
   const bool fused = OPS(p, fused, N, var);
+  const int B = launch_terms(N, p->opts, p->B);
   void* Ta = fused ? p->d_work : p->d_T;
-  void* Tb = (char*)Ta + (size_t)batch * (fused ? n_alpha : p->B) * NN * H * cel;
+  void* Tb = (char*)Ta + (size_t)batch * (fused ? n_alpha : B) * NN * H * cel;
   const int groups = OPS(p, last_groups, N, var, n_alpha);
   const long pbs = (long)ns * 2 * p->sz.maxblk;
   const double fieldb = (double)batch * NN * H * cel;  // one packed complex field per realisation batch
@@ -765,8 +777,8 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, con
             OPS(p, p23, N, Ta, Tb, p->d_sigma[m], n_alpha, p->d_F, groups, n_c, batch, p->d_tw, p->d_err, p->wait_limit,
                 st));
       }
-      for (int a0 = 0; a0 < n_alpha && !fused; a0 += p->B) {
-        const int nb = std::min(p->B, n_alpha - a0);
+      for (int a0 = 0; a0 < n_alpha && !fused; a0 += B) {
+        const int nb = std::min(B, n_alpha - a0);
         RUN(p, 1, phib + 2.0 * nb * fieldb, "P1",
             OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[m], nm1, a0, nb, batch, p->d_tw, var, st));
         RUN(p, 2, 5.0 * nb * fieldb, "P2",
@@ -1072,7 +1084,8 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
   sigw_status status = SIGW_OK;
   // For each terms-per-launch candidate the two strided passes are timed separately (each with both radix
   // variants, bit 0 for the first pass and bit 2 for the second), so the best pair is found in 2 x nvar runs.
-  auto time_pass = [&](int which, int B, int v, float* ms) -> sigw_status {
+  auto time_pass = [&](int which, int choice, int v, float* ms) -> sigw_status {
+    const int B = launch_terms(N, p->opts, choice);
     void* Ta = p->d_T;
     void* Tb = (char*)p->d_T + (size_t)batch * B * NN * H * cel;
     for (int rep = 0; rep < 2; ++rep) {  // first pass warms the variant; the second is timed
@@ -1122,10 +1135,11 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
   const bool has_fused = OPS(p, fused, N, 8);
   if (status == SIGW_OK && (OPS(p, p3_variants, N) > 1 || has_fused)) {
     {
+      const int B = launch_terms(N, p->opts, bestB);
       void* Ta = p->d_T;
-      void* Tb = (char*)p->d_T + (size_t)batch * bestB * NN * H * cel;
-      for (int a0 = 0; a0 < n_alpha && status == SIGW_OK; a0 += bestB) {
-        const int nb = std::min(bestB, n_alpha - a0);
+      void* Tb = (char*)p->d_T + (size_t)batch * B * NN * H * cel;
+      for (int a0 = 0; a0 < n_alpha && status == SIGW_OK; a0 += B) {
+        const int nb = std::min(B, n_alpha - a0);
         cudaError_t e = OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, a0, nb, batch, p->d_tw, bestV, st);
         if (e == cudaSuccess) e = OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, bestV, st);
         if (e != cudaSuccess) status = cuda_fail(p, e, "autotune launch");
@@ -1145,7 +1159,7 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
     const int p3bits[3] = {0, 2, 8};
     float t3[3] = {1e30f, 1e30f, 1e30f};
     for (int v3 = 0; v3 < np3; ++v3) {
-      const int bits = p3bits[v3], groups = has_fused ? OPS(p, last_groups, N, 0, n_alpha) : 1;
+      const int bits = p3bits[v3], groups = OPS(p, last_groups, N, bits, n_alpha);
       time_last(&t3[v3], [&]() {
         return OPS(p, p3, N, p->d_work, p->d_sigma[0], n_alpha, p->d_F, groups, n_c, batch, p->d_tw, p->d_err,
                    sigw::kDefaultWaitLimit, bits, st);

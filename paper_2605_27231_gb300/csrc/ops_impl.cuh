@@ -67,14 +67,24 @@ struct OpsT {
     return cudaGetLastError();
   }
   // ------------------------------------------------------------ hot path
-  // CTAs that share the nb terms of one first-pass tile: enough for about four waves of the 456 CTAs that fit the SMs
-  // (three a SM), at least four terms each, so that the tile's set-up (Phi~, cells, twiddles) stays small against its
-  // transforms.  One realisation at N = 64 has 64 tiles: 50 terms took 114 us on 64 SMs (five launches), 37 us in 768
-  // CTAs; FP64 N = 32 (32 tiles of 64 threads) 119 us for 10 terms, 45 us for 16.  From 256^3 on there is one group.
+  // CTAs that share the nb terms of one first-pass tile: the number for which the waves of the 456 CTAs that fit the
+  // SMs (three a SM) times a CTA's terms is least; half a term stands for a CTA's set-up (Phi~, cells, twiddles).  One
+  // realisation at N = 64 has 64 tiles: 50 terms took 114 us on 64 SMs (five launches), 37 us in 768 CTAs; FP64 N = 32
+  // (32 tiles of 64 threads) 119 us for 10 terms, 45 us for 16.  With many tiles (four realisations at 256^3: 8192) the
+  // waves are nearly full as they are and there is one group.
   static int p1_groups(long tiles, int nb) {
-    const long want = (1700 + tiles - 1) / tiles;
-    const int most = nb / 4 < 1 ? 1 : nb / 4;
-    return (int)(want < most ? want : most);
+    const long slots = 456;
+    int best = 1;
+    double least = 1e30;
+    for (int g = 1; g <= nb; ++g) {
+      const long waves = (tiles * g + slots - 1) / slots;
+      const double cost = (double)waves * ((nb + g - 1) / g + 0.5);
+      if (cost < 0.97 * least) {  // more groups only for a clear gain
+        least = cost;
+        best = g;
+      }
+    }
+    return best;
   }
   template <int N, int E, int TC>
   static cudaError_t p1_v(const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* phitab, int nm1,
