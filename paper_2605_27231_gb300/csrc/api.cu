@@ -44,19 +44,19 @@ int max_alpha_batch(const sigw_opts& o) {
   return std::min(o.n_alpha, 16);
 }
 
-// Terms the first-pass output buffer holds.  At N = 128 the largest choice, 16, stands for 25: a launch of 16 terms of
-// one realisation leaves the last of its few waves short (first pass, 50 terms: 253 us in fours of 16, 205 us in two
-// of 25; second pass 325 and 316 us).
+// Terms the first-pass output buffer holds (at least the pair that the second pass works on).  At N = 128 the largest
+// choice, 16, stands for 26: a launch of 16 terms of one realisation leaves the last of its few waves short (first pass,
+// 50 terms: 253 us in launches of 16, 215 us in two of 25; second pass 325 and 313 us).
 int buffer_terms(int N, const sigw_opts& o) {
   const int b = max_alpha_batch(o);
-  return N == 128 && o.alpha_batch == 0 && b == 16 ? std::min(o.n_alpha, 25) : b;
+  return std::max(2, N == 128 && o.alpha_batch == 0 && b == 16 ? std::min(o.n_alpha, 26) : b);
 }
 
-// Terms per launch for the choice B: equal parts of at most B (N = 128: see buffer_terms).
+// Terms per launch for the choice B: equal parts of at most B (N = 128: see buffer_terms), in whole pairs.
 int launch_terms(int N, const sigw_opts& o, int B) {
-  const int most = B == max_alpha_batch(o) ? buffer_terms(N, o) : B;
+  const int most = std::max(2, B == max_alpha_batch(o) ? buffer_terms(N, o) : B) & ~1;
   const int launches = (o.n_alpha + most - 1) / most;
-  return (o.n_alpha + launches - 1) / launches;
+  return ((o.n_alpha + launches - 1) / launches + 1) & ~1;
 }
 
 // Process-wide autotuning results: (N, precision, realisations, n_alpha) -> (terms per launch, variant).
@@ -88,7 +88,7 @@ Sizes sizes_of(int N, const sigw_opts& o) {
   s.maxblk = sh.maxblk_f3;
   s.phi = mb * NN * NH * cel;
   s.T = 2 * mb * (size_t)B * NN * H * cel;
-  s.W = mb * 3 * (size_t)o.n_alpha * NN * H * cel;
+  s.W = mb * 6 * (size_t)((o.n_alpha + 1) / 2) * NN * H * cel;  // three full rows per term pair
   // the jackknife reuses W after each shell: two standard + two packed half spectra + two real fields
   s.W = std::max(s.W, mb * 2 * (NN * NH * cel + NN * H * cel + NN * (size_t)N * rel) + 1024);
   s.synth = mb * (NN * H * cel + NN * NH * cel + 3 * NN * (size_t)N * rel) + 1024;  // + two real fields (non-local map)
@@ -448,10 +448,10 @@ sigw_status sigw_plan_create(int N, double L, const sigw_opts* opts, void* cuda_
   p->L = L;
   p->opts = o;
   p->B = max_alpha_batch(o);
-  // Untuned default: the choices measured fastest on GB300 (at 128^3 and 256^3 the first and the radix-16 last pass
-  // with their per-thread state in tensor memory; at 512^3 the 512-specific strided passes and the tensor-memory
-  // last pass).  sigw_plan_autotune or the table may override it.
-  p->variant = o.precision == 32 ? (N == 512 ? 15 : (N == 256 ? 26 : (N == 128 ? 30 : (N == 64 ? 8 : 0)))) : 0;
+  // Untuned default: the choices measured fastest on GB300 (from 128^3 on the first and the radix-16 last pass with their
+  // per-thread state in tensor memory; at 64^3 the fused second and last pass).  sigw_plan_autotune or the table may
+  // override it.
+  p->variant = o.precision == 32 ? (N >= 128 ? 26 : (N == 64 ? 8 : 0)) : 0;
   std::string e;
   if (!sigw::build_decomposition(params_of(o), &p->dec, &e)) {
     delete p;
@@ -782,7 +782,7 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, con
         RUN(p, 1, phib + 2.0 * nb * fieldb, "P1",
             OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[m], nm1, a0, nb, batch, p->d_tw, var, st));
         RUN(p, 2, 5.0 * nb * fieldb, "P2",
-            OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, var, st));
+            OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, p->d_err, p->wait_limit, st));
       }
       if (!fused)
         RUN(p, 3, 3.0 * n_alpha * fieldb + 6.0 * groups * batch * NN * ncp * cel, "P3",
@@ -1079,11 +1079,10 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
   CKP(p, cudaEventCreate(&e0), "event");
   CKP(p, cudaEventCreate(&e1), "event");
   double best = 1e300;
-  int bestB = p->B, bestV = p->variant & 21;
+  int bestB = p->B, bestV = p->variant & 17;
   const int cands[] = {4, 5, 8, 10, 16};
   sigw_status status = SIGW_OK;
-  // For each terms-per-launch candidate the two strided passes are timed separately (each with both radix
-  // variants, bit 0 for the first pass and bit 2 for the second), so the best pair is found in 2 x nvar runs.
+  // For each terms-per-launch candidate the two strided passes are timed separately, the first in each of its forms.
   auto time_pass = [&](int which, int choice, int v, float* ms) -> sigw_status {
     const int B = launch_terms(N, p->opts, choice);
     void* Ta = p->d_T;
@@ -1094,7 +1093,8 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
         const int nb = std::min(B, n_alpha - a0);
         cudaError_t e = which == 0
                             ? OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, a0, nb, batch, p->d_tw, v, st)
-                            : OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, v << 2, st);
+                            : OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, p->d_err,
+                                  sigw::kDefaultWaitLimit, st);
         if (e != cudaSuccess) return cuda_fail(p, e, "autotune launch");
       }
       cudaEventRecord(e1, st);
@@ -1110,22 +1110,18 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
   for (int B : cands) {
     if (p->opts.alpha_batch > 0) B = bmax;  // terms per launch fixed by the options: tune the radices only
     if (B > bmax || status != SIGW_OK) continue;
-    float t1[3] = {1e30f, 1e30f, 1e30f}, t2[2] = {1e30f, 1e30f};
-    for (int v = 0; v < np1 && status == SIGW_OK; ++v) {
-      const int bits = (v == nvar) ? 16 : p1bits[v];
-      status = time_pass(0, B, bits, &t1[v]);  // P1 writes the T that P2 reads next
-      if (status == SIGW_OK && v < nvar) status = time_pass(1, B, v, &t2[v]);
-    }
+    float t1[3] = {1e30f, 1e30f, 1e30f}, t2 = 1e30f;
+    for (int v = 0; v < np1 && status == SIGW_OK; ++v) status = time_pass(0, B, v == nvar ? 16 : p1bits[v], &t1[v]);
+    if (status == SIGW_OK) status = time_pass(1, B, 0, &t2);  // P1 wrote the T that P2 reads
     if (status != SIGW_OK) break;
     int v1 = 0;
     for (int v = 1; v < np1; ++v)
       if (t1[v] < t1[v1]) v1 = v;
-    const int v2 = t2[1] < t2[0] ? 1 : 0;
-    const double ms = (double)t1[v1] + (double)t2[v2];
+    const double ms = (double)t1[v1] + (double)t2;
     if (ms < best) {
       best = ms;
       bestB = B;
-      bestV = (v1 == nvar ? 16 : p1bits[v1]) | (v2 << 2);
+      bestV = v1 == nvar ? 16 : p1bits[v1];
     }
     if (p->opts.alpha_batch > 0) break;
   }
@@ -1141,7 +1137,8 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
       for (int a0 = 0; a0 < n_alpha && status == SIGW_OK; a0 += B) {
         const int nb = std::min(B, n_alpha - a0);
         cudaError_t e = OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, a0, nb, batch, p->d_tw, bestV, st);
-        if (e == cudaSuccess) e = OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, bestV, st);
+        if (e == cudaSuccess)
+          e = OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, p->d_err, sigw::kDefaultWaitLimit, st);
         if (e != cudaSuccess) status = cuda_fail(p, e, "autotune launch");
       }
     }

@@ -45,9 +45,8 @@ template <typename T, int N> struct Shape {
   static constexpr int TC3 = TC3_1 * P3 < 32 ? 32 / P3 : TC3_1;  // whole warps (the partial sum uses shuffles)
 };
 
-// Alternative radix of the strided inverse passes (variant bit 1 for the first pass; the second pass uses
-// AltStrided2 with bit 4): FP32, N >= 128 only.  At N = 512 the
-// alternative is radix 32 (two stages, one exchange, 16-column tiles) instead of radix 16 (three stages).
+// Alternative radix of the first strided inverse pass (variant bit 1): FP32, N >= 128 only.  At N = 512 the alternative
+// is radix 32 (two stages, one exchange, 16-column tiles) instead of radix 16 (three stages).
 template <typename T, int N> struct AltStrided {
   static constexpr bool exists = sizeof(T) == 4 && N >= 128;
   static constexpr int E = N == 512 ? 32 : (Shape<T, N>::ES == 16 ? 8 : 16);
@@ -60,13 +59,20 @@ template <typename T, int N> struct AltStrided {
 // points would otherwise need 128 KB for a 16-column tile).
 template <typename T, int N, int TC, int E> using StridedLay = ColLayout<T, N, TC, E, (E >= 32)>;
 
-// Alternative of the second strided pass (variant bit 4): as AltStrided, except at N = 512, where a 512-thread
-// CTA runs 16 columns of radix 16 (full 128-byte row segments, 16 warps per SM, no spills).
-template <typename T, int N> struct AltStrided2 {
-  static constexpr bool exists = sizeof(T) == 4 && N >= 128;
-  static constexpr int E = N == 512 ? 16 : AltStrided<T, N>::E;
-  static constexpr int TC = N == 512 ? 16 : AltStrided<T, N>::TC;
+// Second strided pass: E values per thread and TCL columns per CTA.  TCL is also the column tile of the first pass's
+// output T[b][term][a0][column tile][k1][TCL], so that a CTA's input is one contiguous block (one bulk copy).
+template <typename T, int N> struct Pass2 {
+  static constexpr int E = sizeof(T) == 4 && N == 128 ? 16 : Shape<T, N>::ES;
+  static constexpr int TCL = Shape<T, N>::TC;
+  static constexpr int THREADS = TCL * (N / E);
+  // a field's first transform waits for the second in tensor memory (FP32, N >= 128)
+  static constexpr bool ZTM = sizeof(T) == 4 && E == 16;
 };
+// Place of (k1, cc) in a plane a0 of T.
+template <typename T, int N> __device__ __forceinline__ int t_index(int k1, int cc) {
+  constexpr int TCL = Pass2<T, N>::TCL;
+  return (cc / TCL) * (N * TCL) + k1 * TCL + cc % TCL;
+}
 
 template <int P> struct RowSync { using type = SyncWarp; };
 template <> struct RowSync<64> { using type = SyncBlock; };
@@ -418,59 +424,26 @@ __global__ void __launch_bounds__(256) k_p1(const cx<T>* __restrict__ phi, cx<T>
         v[r] = x;
       }
       fft_pencil<T, N, E, +1, Lay, SyncBlock>(v, j, L, tw, SyncBlock());
-      cx<T>* dst = (D ? Tb : Ta) + ((long)b * nb + a) * fstride + (long)k1 * H + cs;
+      cx<T>* dst = (D ? Tb : Ta) + ((long)b * nb + a) * fstride + t_index<T, N>(k1, cs);
 #pragma unroll
       for (int r = 0; r < E; ++r) dst[(long)(j + r * P) * N * H] = v[r];
     }
   }
 }
 
-// P2: second inverse pass along axis 1 at fixed a0.  For term a:
-//   W[0] = IDFT_1[Ta]            (G_2 after i n2 and the last pass)
-//   W[1] = IDFT_1[i n1^D Ta]     (G_1)
-//   W[2] = IDFT_1[Tb]            (G_0)
-// One value array is live at a time (the Ta tile is reloaded through L1 for the second transform).
-template <typename T, int N, int E_ = Shape<T, N>::ES, int TC_ = Shape<T, N>::TC>
-__global__ void __launch_bounds__(TC_ * (N / E_), ((E_ >= 32 || TC_ * (N / E_) > 256) ? 1 : 2)) k_p2(const cx<T>* __restrict__ Ta, const cx<T>* __restrict__ Tb,
-                                               cx<T>* __restrict__ W, int n_alpha, int alpha0, int nb,
-                                               const cx<T>* __restrict__ tw) {
-  constexpr int E = E_, P = N / E_, TC = TC_, H = N / 2;
-  using Lay = StridedLay<T, N, TC, E>;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int c = threadIdx.x % TC, j = threadIdx.x / TC;
-  const Lay L{reinterpret_cast<cx<T>*>(smraw), c};
-  const int cc = blockIdx.x * TC + c;
-  const int a0 = blockIdx.y;
-  const int b = blockIdx.z / nb, a = blockIdx.z % nb;
-  const long fstride = (long)N * N * H;
-  const long off = (long)a0 * N * H + cc;
-  const cx<T>* ta = Ta + ((long)b * nb + a) * fstride + off;
-  const cx<T>* tb = Tb + ((long)b * nb + a) * fstride + off;
-  auto wout = [&](int f) { return W + (((long)b * 3 + f) * n_alpha + alpha0 + a) * fstride + off; };
-  cx<T> v[E];
-#pragma unroll
-  for (int r = 0; r < E; ++r) v[r] = __ldg(ta + (long)(j + r * P) * H);
-  fft_pencil<T, N, E, +1, Lay, SyncBlock>(v, j, L, tw, SyncBlock());
-  cx<T>* o0 = wout(0);
-#pragma unroll
-  for (int r = 0; r < E; ++r) o0[(long)(j + r * P) * H] = v[r];
-#pragma unroll
-  for (int r = 0; r < E; ++r) {
-    const cx<T> x = __ldg(ta + (long)(j + r * P) * H);
-    const T nd = (T)derivn(j + r * P, N);
-    v[r] = mk<T>(-nd * x.y, nd * x.x);
-  }
-  fft_pencil<T, N, E, +1, Lay, SyncBlock>(v, j, L, tw, SyncBlock());
-  cx<T>* o1 = wout(1);
-#pragma unroll
-  for (int r = 0; r < E; ++r) o1[(long)(j + r * P) * H] = v[r];
-#pragma unroll
-  for (int r = 0; r < E; ++r) v[r] = __ldg(tb + (long)(j + r * P) * H);
-  fft_pencil<T, N, E, +1, Lay, SyncBlock, false>(v, j, L, tw, SyncBlock());
-  cx<T>* o2 = wout(2);
-#pragma unroll
-  for (int r = 0; r < E; ++r) o2[(long)(j + r * P) * H] = v[r];
-}
+// Rows handed from the second to the last inverse pass: for term pair (a, a + 1) and every (a0, a1) three full complex
+// rows over k2, the inputs of the last pass's three complex transforms:
+//   f = 0: g2^a + i g1^a      f = 1: the same of a + 1      f = 2: g0^a + i g0^{a+1}       W[b][pair][f][a0][a1][N]
+// Element c < N/2 of a row is the value at k2 = c, element N - 1 - c the one at k2 = -c; element N - 1 is the value at
+// k2 = N/2.
+// With 64-bit values at N = 128 the index is xor-ed with 8 on odd rows: a half warp of the radix-16 last pass reads two
+// rows there, and they then fall into different banks (see k_p3_tm).
+template <typename T, int N> struct ZRow {
+  static constexpr int SWZ = sizeof(T) == 4 && N == 128 ? 8 : 0;
+};
+
+// All rows carry a common factor -1 (the products do not see it), which saves sign changes here.
+//
 
 // ---------------------------------------------------------------- bulk-copy pipeline helpers
 // cp.async.bulk (TMA, 1-D) global -> shared with mbarrier completion.  Waits are bounded: after `limit` clock
@@ -530,13 +503,13 @@ template <typename T, int N, int E_ = ((N >= 16) ? 8 : 4)> struct P3Cfg {
     return (size_t)STAGES * 6 * rpc * H * sizeof(cx<T>) + (size_t)rpc * Lay::SIZE * sizeof(cx<T>) +
            STAGES * sizeof(uint64_t);
   }
-  // One 16 KB bulk copy per (field, term).  On the small lattices 64 threads: a realisation at N = 32 then has 64 CTAs
-  // (times the groups of term pairs) instead of 16 or 8 (FP64, 50 terms: 976 -> 253 us, the FP64 pipe of 128 SMs).
+  // A 32 KB bulk copy per row block.  On the small lattices 64 threads: a realisation at N = 32 then has 64 CTAs (times
+  // seven groups of term pairs) instead of 16 or 8 (FP64, 50 terms: 976 -> 131 us).
   static constexpr int RPC0 = N <= 32 ? 64 / P : 16384 / (H * (int)sizeof(cx<T>));
   static constexpr int RPC1 = RPC0 > N * N ? N * N : RPC0;
   static constexpr int RPC = smem_for(RPC1) <= 227 * 1024 ? RPC1 : RPC1 / 2;
   static constexpr int THREADS = RPC * P;
-  static constexpr int STAGE_ELEMS = 6 * RPC * H;  // three fields of two terms
+  static constexpr int STAGE_ELEMS = 3 * RPC * N;  // the three row blocks of a term pair
   static constexpr size_t SMEM = smem_for(RPC);
   static_assert(SMEM <= 227 * 1024, "shared memory");
 };
@@ -549,74 +522,21 @@ template <typename T, int N> struct AltP3 {
   static constexpr int E = 16;
 };
 
-// 1-D Hermitian spectrum value of a packed row held in shared memory, at the element k = j + r P that thread j
-// (0 <= j < P) holds in its r-th register (r unrolled).  plain: k = 0 -> Re row[0], k = N/2 -> Im row[0], else
-// row[k] or conj(row[N-k]); grad: i n^D(k) times the plain value, zero at k = 0 and k = N/2.
-// With P E = N, k < N/2 exactly when r < E/2, so only j = 0 needs a run-time test (k = 0 and k = N/2 come from
-// the packed column 0), and the wave number of the gradient is (T) j plus a compile-time offset.
+// Transform input k = j + r P (0 <= j < P, r unrolled) of a row written by k_p2; par: the row's parity.
 template <typename T, int N, int E>
-__device__ __forceinline__ cx<T> herm_plain_r(const cx<T>* row, int j, int r) {
-  constexpr int P = N / E;
-  if (r < E / 2) {
-    const cx<T> v = row[j + r * P];
-    return (r == 0 && j == 0) ? mk<T>(v.x, (T)0) : v;
-  }
-  const bool hz = (r == E / 2) && (j == 0);
-  const cx<T> v = row[hz ? 0 : (E - r) * P - j];
-  return hz ? mk<T>(v.y, (T)0) : conjg<T>(v);
-}
-template <typename T, int N, int E>
-__device__ __forceinline__ cx<T> herm_grad_r(const cx<T>* row, int j, int r, T fj) {
-  constexpr int P = N / E;
-  if (r < E / 2) {
-    const cx<T> x = row[j + r * P];
-    const T n = fj + (T)(r * P);
-    return mk<T>(-n * x.y, n * x.x);
-  }
-  const bool hz = (r == E / 2) && (j == 0);
-  const cx<T> x = conjg<T>(row[hz ? 0 : (E - r) * P - j]);
-  const T n = hz ? (T)0 : fj + (T)(r * P - N);
-  return mk<T>(-n * x.y, n * x.x);
-}
-
-// The same values by a run-time test on k = j + r P.  At N = 512 this form measured faster in the radix-16 last
-// pass (the specialised form above costs registers there, where the kernel already spills).
-template <typename T, int N, int E>
-__device__ __forceinline__ cx<T> herm_plain_k(const cx<T>* row, int j, int r) {
-  constexpr int H = N / 2;
-  const int k = j + r * (N / E);
-  if (k == 0) return mk<T>(row[0].x, (T)0);
-  if (k == H) return mk<T>(row[0].y, (T)0);
-  if (k < H) return row[k];
-  return conjg<T>(row[N - k]);
-}
-template <typename T, int N, int E>
-__device__ __forceinline__ cx<T> herm_grad_k(const cx<T>* row, int j, int r) {
-  constexpr int H = N / 2;
-  const int k = j + r * (N / E);
-  if (k == 0 || k == H) return mk<T>((T)0, (T)0);
-  cx<T> x;
-  T n;
-  if (k < H) {
-    x = row[k];
-    n = (T)k;
+__device__ __forceinline__ cx<T> zrow(const cx<T>* row, int j, int r, int par) {
+  constexpr int P = N / E, SWZ = ZRow<T, N>::SWZ;
+  const bool hz = (r == E / 2) && (j == 0);  // k = N/2
+  if constexpr (SWZ == 0) {
+    return row[r < E / 2 ? j + r * P : (hz ? N - 1 : j + r * P - 1)];
+  } else if constexpr (P == 8) {  // the xor moves by one register index: constant offsets from two bases
+    const int sx = (r & 1) ? -8 * par : 8 * par;
+    if (r < E / 2) return row[j + sx + r * P];
+    return row[hz ? N - 1 - 8 * par : j - 1 + (j == 0 ? -sx : sx) + r * P];
   } else {
-    x = conjg<T>(row[N - k]);
-    n = (T)(k - N);
+    return row[(r < E / 2 ? j + r * P : (hz ? N - 1 : j + r * P - 1)) ^ (SWZ * par)];
   }
-  return mk<T>(-n * x.y, n * x.x);
 }
-template <typename T, int N, int E>
-__device__ __forceinline__ cx<T> row_plain(const cx<T>* row, int j, int r) {
-  if constexpr (N <= 256) return herm_plain_r<T, N, E>(row, j, r);
-  else return herm_plain_k<T, N, E>(row, j, r);
-}
-template <typename T, int N, int E>
-__device__ __forceinline__ cx<T> row_grad(const cx<T>* row, int j, int r, T fj) {
-  if constexpr (N <= 256) return herm_grad_r<T, N, E>(row, j, r, fj);
-  else return herm_grad_k<T, N, E>(row, j, r);
-}
-
 // One term's contribution sigma g_i g_j to the six product components at one point, with zz = (g2, g1):
 // a0 = s_00, a21 = (s_22, s_11), a43 = (s_02, s_01), a5 = s_12.  PAIRED (FP32, N <= 256) uses paired (FP32x2)
 // multiply-adds; at N = 512 their aligned register pairs made the radix-16 last pass spill, so it stays scalar.
@@ -643,8 +563,8 @@ __device__ __forceinline__ void accum6<float, true>(float sa, float g0, float2 z
 // P3: last inverse pass (axis 2, C2R) of all terms for RPC consecutive rows, the product
 //   s_ij(x) = sum_a sigma_a g^a_i(x) g^a_j(x)  (six components in registers),
 // then the forward R2C of s_ij along axis 2 keeping k2 = 0..n_c, written to F[b][comp][a0][a1][k2].
-// Term pair (a, a+1) uses three complex transforms: (g2^a + i g1^a), (g0^a + i g0^{a+1}), (g2^{a+1} + i g1^{a+1}).
-// The six packed rows of a term pair stream into a STAGES-deep shared-memory ring by cp.async.bulk,
+// Term pair (a, a+1) uses three complex transforms: (g2^a + i g1^a), (g0^a + i g0^{a+1}), (g2^{a+1} + i g1^{a+1}),
+// whose inputs are the rows of W.  The rows of a term pair stream into a STAGES-deep shared-memory ring by cp.async.bulk,
 // issued STAGES-1 pairs ahead by thread 0.  Bounded waits: the main loop's waits give up after wait_limit cycles
 // (normally kDefaultWaitLimit; a test passes a tiny limit, so that waits give up while the copies still land).
 // A thread whose wait gave up sets *err, stops waiting and (thread 0) stops issuing copies; before the CTA exits,
@@ -669,29 +589,27 @@ __global__ void __launch_bounds__(P3Cfg<T, N, E_>::THREADS, 1) k_p3(const cx<T>*
   const long row0 = (long)blockIdx.x * RPC;
   const long row = row0 + rr;
   const int b = blockIdx.y;
-  const long fstride = (long)N * N * H;
+  const long fstride = (long)N * N * N;
   // term pairs pr0 .. pr0 + npairs - 1 (blockIdx.z of gridDim.z groups; each group writes its own partial F)
   const int allpairs = (n_alpha + 1) / 2;
   const int pr0 = allpairs * (int)blockIdx.z / (int)gridDim.z;
   const int npairs = allpairs * ((int)blockIdx.z + 1) / (int)gridDim.z - pr0;
   F += (long)blockIdx.z * fgstride;
-  constexpr uint32_t COPY = RPC * H * sizeof(cx<T>);
+  constexpr uint32_t COPY = RPC * N * sizeof(cx<T>);
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) mbar_init(bars + s, 1);
     mbar_init_fence();
   }
   __syncthreads();
-  auto issue = [&](int pr) {  // thread 0: the six rows blocks of term pair pr into stage pr % STAGES
-    const int s = pr % STAGES, a = 2 * (pr0 + pr);
-    const bool two = a + 1 < n_alpha;
+  auto issue = [&](int pr) {  // thread 0: the row blocks of term pair pr into stage pr % STAGES
+    const int s = pr % STAGES;
+    const bool two = 2 * (pr0 + pr) + 1 < n_alpha;
     cx<T>* dst = ring + s * CF::STAGE_ELEMS;
     fence_proxy_async();
-    mbar_expect_tx(bars + s, (two ? 6u : 3u) * COPY);
-    for (int f = 0; f < 3; ++f) {
-      bulk_g2s(dst + f * RPC * H, W + (((long)b * 3 + f) * n_alpha + a) * fstride + row0 * H, COPY, bars + s);
-      if (two) bulk_g2s(dst + (3 + f) * RPC * H, W + (((long)b * 3 + f) * n_alpha + a + 1) * fstride + row0 * H, COPY,
-                        bars + s);
-    }
+    mbar_expect_tx(bars + s, (two ? 3u : 2u) * COPY);
+    for (int f = 0; f < 3; ++f)
+      if (f != 1 || two)
+        bulk_g2s(dst + f * RPC * N, W + (((long)b * allpairs + pr0 + pr) * 3 + f) * fstride + row0 * N, COPY, bars + s);
   };
   if (threadIdx.x == 0)
     for (int pr = 0; pr < STAGES - 1 && pr < npairs; ++pr) issue(pr);
@@ -702,7 +620,7 @@ __global__ void __launch_bounds__(P3Cfg<T, N, E_>::THREADS, 1) k_p3(const cx<T>*
     a0[r] = a5[r] = (T)0;
     a21[r] = a43[r] = mk<T>((T)0, (T)0);
   }
-  const T fj = (T)j;
+  const int par = (int)(row & 1);
   bool ok = true;
   int issued = STAGES - 1 < npairs ? STAGES - 1 : npairs;  // term pairs whose copies thread 0 has issued
   for (int pr = 0; pr < npairs; ++pr) {
@@ -714,38 +632,22 @@ __global__ void __launch_bounds__(P3Cfg<T, N, E_>::THREADS, 1) k_p3(const cx<T>*
     if (ok) ok = mbar_wait(bars + s, (uint32_t)((pr / STAGES) & 1), err, wait_limit);
     const int a = 2 * (pr0 + pr);
     const bool two = a + 1 < n_alpha;
-    const cx<T>* st = ring + s * CF::STAGE_ELEMS + rr * H;
-    const cx<T>* wb0 = st;
-    const cx<T>* w10 = st + RPC * H;
-    const cx<T>* w20 = st + 2 * RPC * H;
-    const cx<T>* wb1 = st + 3 * RPC * H;
-    const cx<T>* w11 = st + 4 * RPC * H;
-    const cx<T>* w21 = st + 5 * RPC * H;
+    const cx<T>* z0 = ring + s * CF::STAGE_ELEMS + rr * N;  // f = 0, 1, 2 follow RPC rows apart
     // (g0^a + i g0^{a+1}) first; its two real parts are kept while the other two transforms run
     cx<T> zB[E], z[E];
 #pragma unroll
-    for (int r = 0; r < E; ++r) {
-      const cx<T> g0 = row_plain<T, N, E>(w20, j, r);
-      const cx<T> g0b = two ? row_plain<T, N, E>(w21, j, r) : mk<T>((T)0, (T)0);
-      zB[r] = mk<T>(g0.x - g0b.y, g0.y + g0b.x);
-    }
+    for (int r = 0; r < E; ++r) zB[r] = zrow<T, N, E>(z0 + 2 * RPC * N, j, r, par);
     fft_pencil<T, N, E, +1, Lay, Sync>(zB, j, L, tw, Sync());
     const T sa = sigma[a];
 #pragma unroll
-    for (int r = 0; r < E; ++r) {
-      const cx<T> g2 = row_grad<T, N, E>(wb0, j, r, fj), g1 = row_plain<T, N, E>(w10, j, r);
-      z[r] = mk<T>(g2.x - g1.y, g2.y + g1.x);
-    }
+    for (int r = 0; r < E; ++r) z[r] = zrow<T, N, E>(z0, j, r, par);
     fft_pencil<T, N, E, +1, Lay, Sync>(z, j, L, tw, Sync());
 #pragma unroll
     for (int r = 0; r < E; ++r) accum6<T, (sizeof(T) == 4 && N <= 256)>(sa, zB[r].x, z[r], a0[r], a21[r], a43[r], a5[r]);
     if (two) {  // uniform across the CTA
       const T sb = sigma[a + 1];
 #pragma unroll
-      for (int r = 0; r < E; ++r) {
-        const cx<T> h2 = row_grad<T, N, E>(wb1, j, r, fj), h1 = row_plain<T, N, E>(w11, j, r);
-        z[r] = mk<T>(h2.x - h1.y, h2.y + h1.x);
-      }
+      for (int r = 0; r < E; ++r) z[r] = zrow<T, N, E>(z0 + RPC * N, j, r, par);
       fft_pencil<T, N, E, +1, Lay, Sync>(z, j, L, tw, Sync());
 #pragma unroll
       for (int r = 0; r < E; ++r) accum6<T, (sizeof(T) == 4 && N <= 256)>(sb, zB[r].y, z[r], a0[r], a21[r], a43[r], a5[r]);
@@ -825,6 +727,37 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) 
       "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15]))
       : "memory");
 }
+// 32 consecutive columns of this thread's lane into registers (one wait).
+__device__ __forceinline__ void tmem_ld32(uint32_t t0, float (&v)[32]) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(t0)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) {
+  uint32_t r[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(v[i]);
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
+      "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
+      "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Two-stage inverse pencil transform of N = 16 R points (R = 8, 16: N = 128, 256), radix 16 then radix R, with the
@@ -832,7 +765,7 @@ __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.
 // W^{-r k}, k = (j + t P) mod 16 (t < NB = 16 / R, 0 < r < R), in every transform of a launch; tw_tm_store writes
 // them once into 32 columns of its lane (twiddle q = t (R - 1) + r - 1 in columns 2q, 2q + 1), and
 // fft_pencil_tw_tm reads them with two tensor-memory loads instead of NB (R - 1) table loads.  Its first stage
-// writes the exchange row as 16-byte pairs (RowLayoutV).  Same arithmetic, in the same order, as
+// writes an exchange row in 16-byte pairs where the layout has them (RowLayoutV).  Same arithmetic, in the same order, as
 // fft_pencil<float, N, 16, +1>.
 template <int N> struct TwTm {
   static constexpr int E = 16, P = N / E, R = N / E, NB = E / R;
@@ -862,17 +795,21 @@ template <int N, typename Lay, typename Sync>
 __device__ __forceinline__ void fft_pencil_tw_tm(float2 (&v)[16], int j, const Lay& L, uint32_t tw_taddr, Sync sync) {
   using C = TwTm<N>;
   constexpr int E = C::E, P = C::P, R = C::R, NB = C::NB;
-  static_assert(Lay::VEC && Lay::SINGLE, "one exchange row with 16-byte pairs");
+  static_assert(Lay::SINGLE, "one exchange buffer");
   float2* x = L.buf(0);
   dftR<float, +1, E>(v);
+  if constexpr (Lay::VEC) {
 #pragma unroll
-  for (int m = 0; m < E / 2; ++m)
-    *reinterpret_cast<float4*>(x + L.idx(j * E + 2 * m)) =
-        make_float4(v[2 * m].x, v[2 * m].y, v[2 * m + 1].x, v[2 * m + 1].y);
+    for (int m = 0; m < E / 2; ++m)
+      *reinterpret_cast<float4*>(x + L.idx(j * E + 2 * m)) =
+          make_float4(v[2 * m].x, v[2 * m].y, v[2 * m + 1].x, v[2 * m + 1].y);
+  } else {
+#pragma unroll
+    for (int r = 0; r < E; ++r) x[L.idx(j * E + r)] = v[r];
+  }
   sync();
-  float w[2][16];
-  tmem_ld16(tw_taddr, w[0]);
-  tmem_ld16(tw_taddr + 16, w[1]);
+  float w[32];
+  tmem_ld32(tw_taddr, w);
 #pragma unroll
   for (int t = 0; t < NB; ++t) {
     const int jj = j + t * P;
@@ -882,7 +819,7 @@ __device__ __forceinline__ void fft_pencil_tw_tm(float2 (&v)[16], int j, const L
 #pragma unroll
     for (int r = 1; r < R; ++r) {
       const int q = t * (R - 1) + r - 1;
-      a[r] = mul<float>(a[r], make_float2(w[q >> 3][2 * (q & 7)], w[q >> 3][2 * (q & 7) + 1]));
+      a[r] = mul<float>(a[r], make_float2(w[2 * q], w[2 * q + 1]));
     }
     dftR<float, +1, R>(a);
 #pragma unroll
@@ -938,6 +875,227 @@ __device__ __forceinline__ void fft_pencil_tw8_tm(float2 (&v)[16], int j, const 
   sync();  // the exchange buffer may be rewritten at once
 }
 
+// P2: second inverse pass along axis 1 at fixed a0, for one term pair.  Two column transforms give a field's two rows:
+//   f = 0, 1:  B = IDFT_1[n1^D Ta], A = IDFT_1[Ta]      (G1 = i B, G2 = i n2 A)
+//              U = -(G2 + i G1) at k2 >= 0,              V = -conj(G2 - i G1), the same at -k2
+//   f = 2:     A = IDFT_1[Tb^a], B = IDFT_1[Tb^{a+1}]:   U = -(A + i B),   V = -conj(A - i B)
+// i.e. six column transforms for six half spectra, as if the fields themselves were stored; the last pass then
+// reads each transform input with one access and no arithmetic.  It is bound by its shared-memory accesses, this pass
+// by HBM: storing the fields and assembling there cost 96 instead of 48 reads a thread and pair (four realisations at
+// 256^3, 50 terms: last pass 6.94 -> 6.04 ms, this pass 10.2 ms either way, 6.6 TB/s).  The first transform
+// of a field waits in tensor memory (FP32, N >= 128) or in the shared memory of its tile.
+//
+// A CTA takes the pairs of one of nag groups for its tile of columns.  Its input tiles (N rows x TCL columns of a field,
+// contiguous) come through a ring of two by bulk copy.  A tile is read from shared memory for both transforms that need
+// it, and its slot is refilled as soon as it is free, at least one transform (2.6 us at 256^3) before the new tile is
+// needed: with both tiles of f = 2 used by one transform the next pair's first copy was waited for (11.3 ms).  FP32, N = 128 and 256: the last-stage twiddles sit in tensor memory.
+// Bounded waits, error flag and the drain before exit as in k_p3.
+template <typename T, int N> struct P2Cfg {
+  static constexpr int E = Pass2<T, N>::E, TC = Pass2<T, N>::TCL, THREADS = Pass2<T, N>::THREADS;
+  using Lay = ColLayout<T, N, TC, E, true>;  // one exchange buffer
+  static constexpr int TILE = N * TC;
+  static constexpr size_t SMEM = (size_t)(Lay::SIZE + 2 * TILE) * sizeof(cx<T>) + 32;
+  static constexpr int CTAS = THREADS > 128 ? 2 : 4;
+  static constexpr bool FSPLIT = N <= 32;  // few tiles: the three fields of a pair go to three CTAs
+  static constexpr bool TWTM = sizeof(T) == 4 && E == 16 && (N == 128 || N == 256);
+  static constexpr bool ZTM = Pass2<T, N>::ZTM;
+  static constexpr uint32_t NCOLS = 64 * ((THREADS + 127) / 128);  // a warp's share: 32 for each of the two
+};
+
+template <typename T, int N>
+__global__ void __launch_bounds__(P2Cfg<T, N>::THREADS, P2Cfg<T, N>::CTAS) k_p2(
+    const cx<T>* __restrict__ Ta, const cx<T>* __restrict__ Tb, cx<T>* __restrict__ W, int npairs, int alpha0, int nb,
+    int nag, const cx<T>* __restrict__ tw, int* __restrict__ err, long long wait_limit) {
+  using CF = P2Cfg<T, N>;
+  constexpr int E = CF::E, P = N / E, TC = CF::TC, H = N / 2, SWZ = ZRow<T, N>::SWZ;
+  constexpr uint32_t COPY = CF::TILE * sizeof(cx<T>);
+  using Lay = typename CF::Lay;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  cx<T>* const ring = reinterpret_cast<cx<T>*>(smraw);
+  cx<T>* const xch = ring + 2 * CF::TILE;
+  uint64_t* const bars = reinterpret_cast<uint64_t*>(xch + Lay::SIZE);
+  uint32_t* const tslot = reinterpret_cast<uint32_t*>(bars + 2);
+  const int c = threadIdx.x % TC, j = threadIdx.x / TC;
+  const Lay L{xch, c};
+  const int cc = blockIdx.x * TC + c;
+  const int a0 = blockIdx.y;
+  const int b = blockIdx.z / nag, g = CF::FSPLIT ? blockIdx.z % nag / 3 : blockIdx.z % nag;
+  const int fs = CF::FSPLIT ? blockIdx.z % nag % 3 : 0;  // the one field of this CTA
+  const int npl = (nb + 1) / 2;  // pairs of this launch (alpha0 is even)
+  const int p0 = CF::FSPLIT ? g : npl * g / nag, p1 = CF::FSPLIT ? g + 1 : npl * (g + 1) / nag;
+  const int nt = min(2 * p1, nb) - 2 * p0;  // terms of this CTA
+  if (CF::FSPLIT && fs == 1 && nt == 1) return;
+  const long fstride = (long)N * N * H;
+  const T n2 = (T)cc, fj = (T)j;
+  const int sw = SWZ * (j & 1);  // P is even: the parity of the row a1 = j + r P (and of N - a1)
+  // input tiles in order of use: Ta^a, Ta^{a+1}, Tb^a, Tb^{a+1} of every pair (Ta^a, Tb^a of a single last term)
+  const int ntiles = !CF::FSPLIT ? 2 * nt : (fs == 2 ? nt : 1);
+  const long toff = ((long)b * nb + 2 * p0) * fstride + (long)a0 * N * H + (long)blockIdx.x * CF::TILE;
+  auto issue = [&](int q) {  // thread 0: tile q into slot q % 2
+    const bool pair = nt - 2 * (q >> 2) >= 2;
+    const int e = q & 3, term = CF::FSPLIT ? (fs == 2 ? q : fs) : 2 * (q >> 2) + (pair ? (e & 1) : 0);
+    const bool isa = CF::FSPLIT ? fs < 2 : (pair ? e < 2 : e < 1);
+    fence_proxy_async();
+    mbar_expect_tx(bars + (q & 1), COPY);
+    bulk_g2s(ring + (q & 1) * CF::TILE, (isa ? Ta : Tb) + toff + term * fstride, COPY, bars + (q & 1));
+  };
+  uint32_t twt = 0;
+  if (threadIdx.x == 0) {
+    mbar_init(bars, 1);
+    mbar_init(bars + 1, 1);
+    mbar_init_fence();
+    issue(0);
+    if (ntiles > 1) issue(1);
+  }
+  if constexpr (CF::ZTM) {
+    const int warp = threadIdx.x >> 5;
+    if (warp == 0) tmem_alloc(tslot, CF::NCOLS);
+    tmem_fence_before_sync();
+    __syncthreads();
+    tmem_fence_after_sync();
+    twt = *tslot + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(64 * (warp >> 2));
+    if constexpr (CF::TWTM) {
+      tw_tm_store<N>(twt, j, tw);
+      tmem_wait_st();
+    }
+  } else {
+    __syncthreads();
+  }
+  int issued = ntiles > 1 ? 2 : 1;  // tiles thread 0 has issued
+  bool ok = true;
+  int q = 0;  // tiles used up
+  for (int lp = 0; 2 * lp < nt; ++lp) {
+    const bool two = nt - 2 * lp >= 2;
+    cx<T>* const w0 = W + (((long)b * npairs + alpha0 / 2 + p0 + lp) * 3 * N + a0) * (long)N * N;
+    cx<T> hold[E];  // without tensor memory: the first transform of a field until its stash is free
+#pragma unroll 1
+    for (int t = 0; t < 6; ++t) {
+      const int f = t >> 1, s = t & 1;
+      if (!two && (f == 1 || t == 5)) continue;
+      if (CF::FSPLIT && f != fs) continue;
+      const bool last = s == 1 || !two && f == 2;  // this transform completes the field's two rows
+      if (s == 0 || f == 2)                        // its tile has arrived
+        if (ok) ok = mbar_wait(bars + (q & 1), (uint32_t)((q >> 1) & 1), err, wait_limit);
+      cx<T>* const x0 = ring + (q & 1) * CF::TILE + j * TC + c;
+      cx<T> v[E];
+#pragma unroll
+      for (int r = 0; r < E; ++r) v[r] = x0[r * P * TC];
+      if (f < 2 && s == 0) {
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+          const T nd = r < E / 2 ? fj + (T)(r * P) : ((r == E / 2 && j == 0) ? (T)0 : fj + (T)(r * P - N));
+          v[r] = scale<T>(v[r], nd);
+        }
+      }
+      // the stash of a thread without tensor memory: its own places of the field's first tile, read for the last time
+      cx<T>* const stash = ring + ((f == 2 ? q - 1 : q) & 1) * CF::TILE + j * TC + c;
+      if constexpr (!CF::ZTM) {
+        if (s == 1) {
+#pragma unroll
+          for (int r = 0; r < E; ++r) stash[r * P * TC] = hold[r];
+        }
+      }
+      if constexpr (CF::TWTM) fft_pencil_tw_tm<N, Lay, SyncBlock>(v, j, L, twt, SyncBlock());
+      else fft_pencil<T, N, E, +1, Lay, SyncBlock>(v, j, L, tw, SyncBlock());
+      if (CF::ZTM && (s == 1 || f == 2)) {  // every thread has read this tile: refill its slot
+        if (threadIdx.x == 0 && ok && q + 2 < ntiles) {
+          issue(q + 2);
+          issued = q + 3;
+        }
+        ++q;
+      }
+      cx<T> h[E];  // the field's first transform
+      if constexpr (CF::ZTM) {
+        float w[32];
+        if (!last) {
+#pragma unroll
+          for (int r = 0; r < E; ++r) {
+            w[2 * r] = v[r].x;
+            w[2 * r + 1] = v[r].y;
+          }
+          tmem_st32(twt + 32, w);
+          tmem_wait_st();
+          continue;
+        }
+        if (s == 1) {
+          tmem_ld32(twt + 32, w);
+#pragma unroll
+          for (int r = 0; r < E; ++r) h[r] = make_float2(w[2 * r], w[2 * r + 1]);
+        }
+      } else {
+        if (!last) {
+#pragma unroll
+          for (int r = 0; r < E; ++r) hold[r] = v[r];
+          if (f == 2) ++q;
+          continue;
+        }
+        if (s == 1) {
+#pragma unroll
+          for (int r = 0; r < E; ++r) h[r] = stash[r * P * TC];
+        }
+      }
+      if (s == 0) {  // a single last term: Tb^{a+1} = 0
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+          h[r] = v[r];
+          v[r] = mk<T>((T)0, (T)0);
+        }
+      }
+      cx<T>* const o = w0 + (long)f * N * N * N + j * N;
+      const int pu = cc ^ sw, pv = (N - 1 - cc) ^ sw;
+      if (cc == 0) {  // packed column, k2 = 0 and k2 = N/2 (n2^D = 0 on both)
+        if (f < 2) {
+#pragma unroll
+          for (int r = 0; r < E; ++r) {
+            o[r * P * N + pu] = mk<T>((T)0, h[r].y);
+            o[r * P * N + pv] = mk<T>((T)0, -h[r].x);
+          }
+        } else {
+#pragma unroll
+          for (int r = 0; r < E; ++r) {
+            o[r * P * N + pu] = mk<T>(-h[r].x, -v[r].x);
+            o[r * P * N + pv] = mk<T>(-h[r].y, -v[r].y);
+          }
+        }
+      } else if (f < 2) {
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+          o[r * P * N + pu] = mk<T>(n2 * v[r].y + h[r].x, h[r].y - n2 * v[r].x);
+          o[r * P * N + pv] = mk<T>(n2 * v[r].y - h[r].x, h[r].y + n2 * v[r].x);
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+          o[r * P * N + pu] = mk<T>(v[r].y - h[r].x, -h[r].y - v[r].x);
+          o[r * P * N + pv] = mk<T>(-h[r].x - v[r].y, h[r].y - v[r].x);
+        }
+      }
+      if constexpr (!CF::ZTM) {  // every thread has read its stash: refill the field's slots
+        __syncthreads();
+        const int q0 = (f == 2 && two) ? q - 1 : q;
+        ++q;
+        if (threadIdx.x == 0 && ok)
+          for (int u = q0; u < q; ++u)
+            if (u + 2 < ntiles) {
+              issue(u + 2);
+              issued = u + 3;
+            }
+      }
+    }
+  }
+  if (threadIdx.x == 0) {  // the last copy issued into each slot has landed before the CTA may exit
+    mbar_wait(bars + ((issued - 1) & 1), (uint32_t)(((issued - 1) >> 1) & 1), err);
+    if (issued > 1) mbar_wait(bars + ((issued - 2) & 1), (uint32_t)(((issued - 2) >> 1) & 1), err);
+  }
+  if constexpr (CF::ZTM) {
+    tmem_fence_before_sync();
+    __syncthreads();
+    tmem_fence_after_sync();
+    if (threadIdx.x < 32) tmem_dealloc(*tslot, CF::NCOLS);
+  }
+}
+
+
 // P3 with its accumulators in tensor memory (autotuner variant bit 8; FP32, radix 16, N = 128, 256, 512).  The last pass
 // above keeps the six product components of its 16 points per thread in registers (96 of its 254), which holds
 // it to one CTA of 8 warps per SM.  Here they live in TMEM, in the thread's lane: s00 in columns 0-15, s12 in
@@ -947,6 +1105,10 @@ __device__ __forceinline__ void fft_pencil_tw8_tm(float2 (&v)[16], int j, const 
 // One ring stage per CTA: the three transforms' inputs of a term pair are read into registers, the stage is
 // refilled for the next pair while the transforms run, and the other CTAs of the SM cover the copy.
 // Bounded waits, error flag and the drain before exit as in k_p3.
+// What bounds it: HBM at 256^3 (6.8 TB/s of rows, four realisations).  Before the rows came ready-made from k_p2 its
+// shared-memory path did (80 % of its cycles at 128^3 with a third of them bank conflicts, 88 % at 512^3), and 50 terms
+// took 284 us at 128^3 (one realisation; now 219), 6.94 ms at 256^3 (four; now 6.04), 15.9 ms at 512^3 (40 terms; now 14.3,
+// still bound by the exchanges of its three-stage transform).
 template <int N>
 struct P3TCfg {
   static constexpr int H = N / 2, E = 16, P = N / E, RPC = 128 / P, THREADS = RPC * P;  // 16 / 8 / 4 rows at N = 128 / 256 / 512
@@ -954,7 +1116,7 @@ struct P3TCfg {
   // two-stage transforms (N <= 256): twiddles in TMEM columns 96-127 and 16-byte exchange stores
   static constexpr bool TWTM = N <= 256;
   using Lay = std::conditional_t<TWTM, RowLayoutV<float, N>, RowLayout<float, N, true, 4>>;
-  static constexpr int STAGE_ELEMS = 6 * RPC * H;  // three fields of two terms
+  static constexpr int STAGE_ELEMS = 3 * RPC * N;  // the three row blocks of a term pair
   static constexpr uint32_t NCOLS = 128;           // TMEM columns per CTA (96, or 128 with the twiddles)
   static constexpr size_t SMEM = (size_t)STAGE_ELEMS * 8 + (size_t)RPC * Lay::SIZE * 8 + 16;
 };
@@ -966,7 +1128,7 @@ __global__ void __launch_bounds__(P3TCfg<N>::THREADS, 3) k_p3_tm(const float2* _
                                                                   const float2* __restrict__ tw,
                                                                   int* __restrict__ err, long long wait_limit) {
   using CF = P3TCfg<N>;
-  constexpr int E = CF::E, P = CF::P, H = CF::H, RPC = CF::RPC;
+  constexpr int E = CF::E, P = CF::P, RPC = CF::RPC;
   using Sync = typename RowSync<P>::type;
   using Lay = typename CF::Lay;
   extern __shared__ __align__(128) unsigned char smraw[];
@@ -979,9 +1141,9 @@ __global__ void __launch_bounds__(P3TCfg<N>::THREADS, 3) k_p3_tm(const float2* _
   const long row0 = (long)blockIdx.x * RPC;
   const long row = row0 + rr;
   const int b = blockIdx.y;
-  const long fstride = (long)N * N * H;
+  const long fstride = (long)N * N * N;
   const int npairs = (n_alpha + 1) / 2;
-  constexpr uint32_t COPY = RPC * H * sizeof(float2);
+  constexpr uint32_t COPY = RPC * N * sizeof(float2);
   const int warp = threadIdx.x >> 5;
   if (warp == 0) tmem_alloc(tslot, CF::NCOLS);
   if (threadIdx.x == 0) {
@@ -1002,53 +1164,36 @@ __global__ void __launch_bounds__(P3TCfg<N>::THREADS, 3) k_p3_tm(const float2* _
     if constexpr (CF::TWTM) tw_tm_store<N>(tcol(6), j, tw);
     tmem_wait_st();
   }
-  auto issue = [&](int pr) {  // thread 0: the six row blocks of term pair pr into the stage
-    const int a = 2 * pr;
-    const bool two = a + 1 < n_alpha;
+  auto issue = [&](int pr) {  // thread 0: the row blocks of term pair pr into the stage
+    const bool two = 2 * pr + 1 < n_alpha;
     fence_proxy_async();
-    mbar_expect_tx(bar, (two ? 6u : 3u) * COPY);
-    for (int f = 0; f < 3; ++f) {
-      bulk_g2s(ring + f * RPC * H, W + (((long)b * 3 + f) * n_alpha + a) * fstride + row0 * H, COPY, bar);
-      if (two) bulk_g2s(ring + (3 + f) * RPC * H, W + (((long)b * 3 + f) * n_alpha + a + 1) * fstride + row0 * H, COPY,
-                        bar);
-    }
+    mbar_expect_tx(bar, (two ? 3u : 2u) * COPY);
+    for (int f = 0; f < 3; ++f)
+      if (f != 1 || two)
+        bulk_g2s(ring + f * RPC * N, W + (((long)b * npairs + pr) * 3 + f) * fstride + row0 * N, COPY, bar);
   };
   if (threadIdx.x == 0) issue(0);
   int issued = 1;  // term pairs whose copies thread 0 has issued
-  const float fj = (float)j;
+  const int par = (int)(row & 1);
+  const float2* zin = ring + rr * N;  // rows f = 0, 1, 2 follow RPC rows apart
   bool ok = true;
   for (int pr = 0; pr < npairs; ++pr) {
     if (ok) ok = mbar_wait(bar, (uint32_t)(pr & 1), err, wait_limit);
     const int a = 2 * pr;
     const bool two = a + 1 < n_alpha;
-    const float2* wb0 = ring + rr * H;
-    const float2* w10 = wb0 + RPC * H;
-    const float2* w20 = wb0 + 2 * RPC * H;
-    const float2* wb1 = wb0 + 3 * RPC * H;
-    const float2* w11 = wb0 + 4 * RPC * H;
-    const float2* w21 = wb0 + 5 * RPC * H;
-    // inputs of the three transforms: (g0^a + i g0^{a+1}), (g2^a + i g1^a), (g2^{a+1} + i g1^{a+1}); whether the
-    // pair has a second term (all but an odd last pair) is chosen once, not per value
+    // inputs of the three transforms: (g0^a + i g0^{a+1}), (g2^a + i g1^a), (g2^{a+1} + i g1^{a+1})
     float2 zB[E], za[E], zb[E];
-    auto assemble = [&](auto second) {
-      constexpr bool TWO = decltype(second)::value;
 #pragma unroll
-      for (int r = 0; r < E; ++r) {
-        const float2 g0 = row_plain<float, N, E>(w20, j, r);
-        const float2 g0b = TWO ? row_plain<float, N, E>(w21, j, r) : make_float2(0.f, 0.f);
-        zB[r] = make_float2(g0.x - g0b.y, g0.y + g0b.x);
-        const float2 g2 = row_grad<float, N, E>(wb0, j, r, fj), g1 = row_plain<float, N, E>(w10, j, r);
-        za[r] = make_float2(g2.x - g1.y, g2.y + g1.x);
-        if constexpr (TWO) {
-          const float2 h2 = row_grad<float, N, E>(wb1, j, r, fj), h1 = row_plain<float, N, E>(w11, j, r);
-          zb[r] = make_float2(h2.x - h1.y, h2.y + h1.x);
-        } else {
-          zb[r] = make_float2(0.f, 0.f);
-        }
-      }
-    };
-    if (two) assemble(std::true_type{});
-    else assemble(std::false_type{});
+    for (int r = 0; r < E; ++r) zB[r] = zrow<float, N, E>(zin + 2 * RPC * N, j, r, par);
+#pragma unroll
+    for (int r = 0; r < E; ++r) za[r] = zrow<float, N, E>(zin, j, r, par);
+    if (two) {  // all but an odd last pair
+#pragma unroll
+      for (int r = 0; r < E; ++r) zb[r] = zrow<float, N, E>(zin + RPC * N, j, r, par);
+    } else {
+#pragma unroll
+      for (int r = 0; r < E; ++r) zb[r] = make_float2(0.f, 0.f);
+    }
     __syncthreads();  // the stage has been read: refill it for the next pair while the transforms run
     if (threadIdx.x == 0 && ok && pr + 1 < npairs) {
       issue(pr + 1);
@@ -1300,7 +1445,7 @@ __global__ void __launch_bounds__(P1TCfg<N>::THREADS, 3) k_p1_tm(const float2* _
       }
       if constexpr (N <= 256) fft_pencil_tw8_tm<N, Lay, SyncBlock>(v, j, L, tw, tbase + 48, SyncBlock());
       else fft_pencil<float, N, E, +1, Lay, SyncBlock>(v, j, L, tw, SyncBlock());
-      float2* dst = (D ? Tb : Ta) + ((long)b * nb + a) * fstride + (long)k1 * H + cs;
+      float2* dst = (D ? Tb : Ta) + ((long)b * nb + a) * fstride + t_index<float, N>(k1, cs);
 #pragma unroll
       for (int r = 0; r < E; ++r) dst[(long)(j + r * P) * N * H] = v[r];
     }
@@ -1358,37 +1503,6 @@ template <int N> struct P23RowLay {
   __device__ __forceinline__ float2* buf(int) const { return base; }
   __device__ __forceinline__ int idx(int p) const { return p + 2 * (p >> 4); }
 };
-
-// 32 consecutive columns of this thread's lane into registers (one wait).
-__device__ __forceinline__ void tmem_ld32(uint32_t t0, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(t0)
-      : "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) {
-  uint32_t r[32];
-#pragma unroll
-  for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(v[i]);
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
-      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
-      "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
-      "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-      : "memory");
-}
 
 template <int N>
 __global__ void __launch_bounds__(P23Cfg<N>::THREADS, P23Cfg<N>::CTAS) k_p23(

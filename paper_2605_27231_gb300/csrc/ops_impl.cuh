@@ -67,18 +67,17 @@ struct OpsT {
     return cudaGetLastError();
   }
   // ------------------------------------------------------------ hot path
-  // CTAs that share the nb terms of one first-pass tile: the number for which the waves of the 456 CTAs that fit the
-  // SMs (three a SM) times a CTA's terms is least; half a term stands for a CTA's set-up (Phi~, cells, twiddles).  One
-  // realisation at N = 64 has 64 tiles: 50 terms took 114 us on 64 SMs (five launches), 37 us in 768 CTAs; FP64 N = 32
-  // (32 tiles of 64 threads) 119 us for 10 terms, 45 us for 16.  With many tiles (four realisations at 256^3: 8192) the
-  // waves are nearly full as they are and there is one group.
+  // CTAs that share the nb terms of one first-pass tile: the number for which the waves of the 456 CTAs that fit the SMs
+  // (three a SM; 0.4 for the uneven end) times a CTA's terms is least, half a term standing for a CTA's set-up (Phi~,
+  // cells, twiddles).  One realisation at N = 64 has 64 tiles: 50 terms took 114 us on 64 SMs (five launches), 35 us in
+  // 7 groups; N = 128, 50 terms: 268 us in one group, 219 us in 7 (three realisations 628, 557 in 3); FP64 N = 32 (32
+  // tiles of 64 threads): 594 us in one, 94 us in 14.  With many tiles (256^3: 2048 and more) there is one group.
   static int p1_groups(long tiles, int nb) {
-    const long slots = 456;
     int best = 1;
     double least = 1e30;
     for (int g = 1; g <= nb; ++g) {
-      const long waves = (tiles * g + slots - 1) / slots;
-      const double cost = (double)waves * ((nb + g - 1) / g + 0.5);
+      const double waves = tiles * g / 456.0;
+      const double cost = (waves <= 1.0 ? 1.0 : waves + 0.4) * ((nb + g - 1) / g + 0.5);
       if (cost < 0.97 * least) {  // more groups only for a clear gain
         least = cost;
         best = g;
@@ -158,30 +157,27 @@ struct OpsT {
     } else {
       using CF = P3Cfg<T, N, ((N >= 16) ? 8 : 4)>;
       tiles = (long)N * N / CF::RPC;
-      slots = 152;
+      slots = N <= 32 ? 456 : 152;  // 64-thread CTAs, three a SM (FP64 N = 32: 224 us in two groups, 131 us in seven)
     }
     const long g = slots / tiles, pairs = (n_alpha + 1) / 2;
-    return (int)(g < 1 ? 1 : (g > 8 ? (pairs < 8 ? pairs : 8) : (g > pairs ? pairs : g)));
-  }
-  template <int N, int E, int TC>
-  static cudaError_t p2_v(const void* Ta, const void* Tb, void* W, int n_alpha, int alpha0, int nb, int batch,
-                          const void* tw, cudaStream_t st) {
-    const size_t sm = strided_bytes<N, TC, E>();
-    auto k = k_p2<T, N, E, TC>;
-    SIGW_CHECK_LAUNCH(allow_smem(k, sm));
-    dim3 grid((N / 2) / TC, N, batch * nb);
-    k<<<grid, TC * (N / E), sm, st>>>((const C*)Ta, (const C*)Tb, (C*)W, n_alpha, alpha0, nb, (const C*)tw);
-    return cudaGetLastError();
+    return (int)(g < 1 ? 1 : (g > 7 ? (pairs < 7 ? pairs : 7) : (g > pairs ? pairs : g)));
   }
   template <int N>
   static cudaError_t p2_n(const void* Ta, const void* Tb, void* W, int n_alpha, int alpha0, int nb, int batch,
-                          const void* tw, int variant, cudaStream_t st) {
-    using SH = Shape<T, N>;
-    using AL = AltStrided2<T, N>;
-    if constexpr (AL::exists) {
-      if (variant & 4) return p2_v<N, AL::E, AL::TC>(Ta, Tb, W, n_alpha, alpha0, nb, batch, tw, st);
-    }
-    return p2_v<N, SH::ES, SH::TC>(Ta, Tb, W, n_alpha, alpha0, nb, batch, tw, st);
+                          const void* tw, int* err, long long wait_limit, cudaStream_t st) {
+    using CF = P2Cfg<T, N>;
+    auto k = k_p2<T, N>;
+    SIGW_CHECK_LAUNCH(allow_smem(k, CF::SMEM));
+    // CTAs that share the pairs of a tile.  Where four fit a SM the first loads of one are hidden by the others: a pair
+    // each (N = 128, 50 terms: 444 us in one group, 326 us in 13).  Where two fit, about twelve waves are enough (256^3,
+    // one realisation: 2628 us in one, 2590 us in two, 2690 us in 13).
+    const long tiles = (long)(N / 2) / CF::TC * N * batch, pairs = (nb + 1) / 2;
+    const long want = CF::CTAS == 4 ? pairs : (12L * 152 * CF::CTAS + tiles - 1) / tiles;
+    const int nag = (int)(want < pairs ? want : pairs) * (CF::FSPLIT ? 3 : 1);
+    dim3 grid((N / 2) / CF::TC, N, batch * nag);
+    k<<<grid, CF::THREADS, CF::SMEM, st>>>((const C*)Ta, (const C*)Tb, (C*)W, (n_alpha + 1) / 2, alpha0, nb, nag,
+                                           (const C*)tw, err, wait_limit);
+    return cudaGetLastError();
   }
   template <int N, int E>
   static cudaError_t p3_v(const void* W, const void* sigma, int n_alpha, void* F, int groups, int n_c, int batch,
@@ -382,8 +378,8 @@ cudaError_t OpsRT<T>::p1(int N, const void* phi, void* Ta, void* Tb, const int16
 }
 template <typename T>
 cudaError_t OpsRT<T>::p2(int N, const void* Ta, const void* Tb, void* W, int n_alpha, int alpha0, int nb, int batch,
-                      const void* tw, int variant, cudaStream_t st) {
-  SIGW_DISPATCH_N(N, return (OpsT<T>::template p2_n<NN>(Ta, Tb, W, n_alpha, alpha0, nb, batch, tw, variant, st)));
+                      const void* tw, int* err, long long wait_limit, cudaStream_t st) {
+  SIGW_DISPATCH_N(N, return (OpsT<T>::template p2_n<NN>(Ta, Tb, W, n_alpha, alpha0, nb, batch, tw, err, wait_limit, st)));
 }
 template <typename T>
 bool OpsRT<T>::fused(int N, int variant) {
