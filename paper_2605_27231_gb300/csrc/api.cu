@@ -451,7 +451,7 @@ sigw_status sigw_plan_create(int N, double L, const sigw_opts* opts, void* cuda_
   // Untuned default: the choices measured fastest on GB300 (from 128^3 on the first and the radix-16 last pass with their
   // per-thread state in tensor memory; at 64^3 the fused second and last pass).  sigw_plan_autotune or the table may
   // override it.
-  p->variant = o.precision == 32 ? (N >= 128 ? 26 : (N == 64 ? 8 : 0)) : 0;
+  p->variant = o.precision == 32 ? (N >= 128 ? 26 : (N == 64 ? 24 : 0)) : 0;
   std::string e;
   if (!sigw::build_decomposition(params_of(o), &p->dec, &e)) {
     delete p;
@@ -1104,7 +1104,7 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
     return SIGW_OK;
   };
   // first-pass candidates: the two radix forms and, where it exists, the radix-16 form with its tile in TMEM
-  const bool p1tm = p->opts.precision == 32 && (N == 128 || N == 256 || N == 512);
+  const bool p1tm = p->opts.precision == 32 && N >= 64;
   const int p1bits[3] = {0, 1, 16};
   const int np1 = nvar + (p1tm ? 1 : 0);
   for (int B : cands) {

@@ -1308,17 +1308,264 @@ __global__ void __launch_bounds__(P3TCfg<N>::THREADS, 3) k_p3_tm(const float2* _
   if (warp == 0) tmem_dealloc(*tslot, CF::NCOLS);
 }
 
-// P1 with its Phi~ tile and cell indices in tensor memory (autotuner variant bit 16; FP32, radix 16, 256 threads
-// per CTA: 32, 16 or 8 columns at N = 128, 256, 512).  k_p1 keeps each thread's 16 Phi~ values and cells in registers for all the terms of a launch
+// ---------------------------------------------------------------- two transforms side by side
+// c2 holds one point of two transforms A and B that use the same roots: r = (Re A, Re B), i = (Im A, Im B).  Every complex
+// operation is then two or four paired (FP32x2) instructions for both, and a multiplication by i costs nothing.  SC:
+// the outputs of a last butterfly layer come from scalar instructions, so that (Re A, Im A) and (Re B, Im B) can be
+// stored as they are without moves.
+struct c2 {
+  float2 r, i;
+};
+template <bool SC> __device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  if constexpr (SC) return make_float2(a.x + b.x, a.y + b.y);
+  else return __fadd2_rn(a, b);
+}
+template <bool SC> __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  if constexpr (SC) return make_float2(a.x - b.x, a.y - b.y);
+  else return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+}
+template <bool SC> __device__ __forceinline__ float2 fma2(float s, float2 u, float2 a) {  // s u + a
+  if constexpr (SC) return make_float2(fmaf(s, u.x, a.x), fmaf(s, u.y, a.y));
+  else return __ffma2_rn(u, make_float2(s, s), a);
+}
+// inverse DFTs (roots e^{+2 pi i / R})
+template <bool SC> __device__ __forceinline__ void idft2c(c2& a, c2& b) {
+  const c2 t = a;
+  a = {add2<SC>(t.r, b.r), add2<SC>(t.i, b.i)};
+  b = {sub2<SC>(t.r, b.r), sub2<SC>(t.i, b.i)};
+}
+// (e + i o, e - i o)
+template <bool SC> __device__ __forceinline__ void bfly_i(const c2& e, const c2& o, c2& p, c2& m) {
+  p = {sub2<SC>(e.r, o.i), add2<SC>(e.i, o.r)};
+  m = {add2<SC>(e.r, o.i), sub2<SC>(e.i, o.r)};
+}
+// (e + s u, e - s u) with separate signs of the real and imaginary parts
+template <bool SC> __device__ __forceinline__ void bfly_s(const c2& e, const c2& u, float sr, float si, c2& p, c2& m) {
+  p = {fma2<SC>(sr, u.r, e.r), fma2<SC>(si, u.i, e.i)};
+  m = {fma2<SC>(-sr, u.r, e.r), fma2<SC>(-si, u.i, e.i)};
+}
+template <bool SC> __device__ __forceinline__ void idft4c(c2* v) {
+  c2 s0 = v[0], d0 = v[2], s1 = v[1], d1 = v[3];
+  idft2c<false>(s0, d0);
+  idft2c<false>(s1, d1);
+  idft2c<SC>(s0, s1);
+  v[0] = s0;
+  v[2] = s1;
+  bfly_i<SC>(d0, d1, v[1], v[3]);
+}
+template <bool SC> __device__ __forceinline__ void idft8c(c2* v) {
+  const float h = 0.70710678118654752440f;
+  c2 e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+  idft4c<false>(e);
+  idft4c<false>(o);
+  idft2c<SC>(e[0], o[0]);
+  v[0] = e[0];
+  v[4] = o[0];
+  c2 u = {sub2<false>(o[1].r, o[1].i), add2<false>(o[1].r, o[1].i)};  // o1 (1 + i)
+  bfly_s<SC>(e[1], u, h, h, v[1], v[5]);
+  bfly_i<SC>(e[2], o[2], v[2], v[6]);
+  u = {add2<false>(o[3].r, o[3].i), sub2<false>(o[3].r, o[3].i)};  // o3 (-1 + i) = (-(r + i), r - i)
+  bfly_s<SC>(e[3], u, -h, h, v[3], v[7]);
+}
+__device__ __forceinline__ void idft16c(c2* v) {
+  const float h = 0.70710678118654752440f, c = 0.92387953251128675613f, t = 0.41421356237309504880f;  // cos, tan (pi/8)
+  c2 e[8], o[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) { e[k] = v[2 * k]; o[k] = v[2 * k + 1]; }
+  idft8c<false>(e);
+  idft8c<false>(o);
+  idft2c<false>(e[0], o[0]);
+  v[0] = e[0];
+  v[8] = o[0];
+  // o_k times e^{i k pi / 8}, the cosine of the octant taken out
+  c2 u = {fma2<false>(-t, o[1].i, o[1].r), fma2<false>(t, o[1].r, o[1].i)};
+  bfly_s<false>(e[1], u, c, c, v[1], v[9]);
+  u = {sub2<false>(o[2].r, o[2].i), add2<false>(o[2].r, o[2].i)};
+  bfly_s<false>(e[2], u, h, h, v[2], v[10]);
+  u = {fma2<false>(-t, o[3].r, o[3].i), fma2<false>(t, o[3].i, o[3].r)};
+  bfly_s<false>(e[3], u, -c, c, v[3], v[11]);
+  bfly_i<false>(e[4], o[4], v[4], v[12]);
+  u = {fma2<false>(t, o[5].r, o[5].i), fma2<false>(-t, o[5].i, o[5].r)};
+  bfly_s<false>(e[5], u, -c, c, v[5], v[13]);
+  u = {add2<false>(o[6].r, o[6].i), sub2<false>(o[6].r, o[6].i)};
+  bfly_s<false>(e[6], u, -h, h, v[6], v[14]);
+  u = {fma2<false>(t, o[7].i, o[7].r), fma2<false>(-t, o[7].r, o[7].i)};
+  bfly_s<false>(e[7], u, -c, -c, v[7], v[15]);
+}
+template <int R, bool SC> __device__ __forceinline__ void idftc(c2* v) {
+  if constexpr (R == 4) idft4c<SC>(v);
+  else idft8c<SC>(v);
+}
+// Times a root given to both transforms as w = (wx, wx, wy, wy), n = (-wy, -wy).
+__device__ __forceinline__ c2 mulc(const c2& z, const float4& w, const float2& n) {
+  return {__ffma2_rn(z.i, n, __fmul2_rn(z.r, make_float2(w.x, w.y))),
+          __ffma2_rn(z.i, make_float2(w.x, w.y), __fmul2_rn(z.r, make_float2(w.z, w.w)))};
+}
+
+// P1 with its two transforms side by side (autotuner variant bit 16; FP32, N = 64 and 128): Ta and Tb of a term are the
+// transforms of f Phi~ and i n0 f Phi~ with the same roots, so they run as one c2 transform.  Against one after the other
+// that is one filter lookup and Phi~ read instead of two, one exchange (16-byte elements) and about 0.6 of the
+// instructions.  A thread's 16 Phi~ values and cells sit in its tensor-memory lane for all the terms of a launch (columns
+// 0-31: Phi~ as (re, im) pairs, 32-47: cells); the roots of the last stage are in shared memory in the form mulc wants.
+// Four CTAs of 128 threads share an SM (with two of 256 threads the barriers of a CTA left it idle: 128^3, 50 terms of one
+// realisation 207 us, now 173; the transforms one after the other 219).  Eight realisations at 64^3: 198 -> 161 us.  From
+// 256^3 on k_p1_tm is faster: rows of 128 bytes need 256 threads here, and 16 warps a SM then leave more latency open
+// than its 24 (50 terms of four realisations 5.80 ms against 5.33).
+template <int N>
+struct P1ACfg {
+  static constexpr int H = N / 2, E = 16, P = N / E;
+  static constexpr int THREADS = 128, CTAS = 4, TC = THREADS / P;  // 32 and 16 columns
+  static constexpr int RL = N / 16, NB = 16 / RL;                  // last stage: radix, butterflies per thread
+  static constexpr int ROOTS = NB * (RL - 1) * P;                  // its roots [t][r - 1][j]
+  static constexpr uint32_t NCOLS = 64;
+  static size_t smem(int nb, int nm1) {
+    return (size_t)N * TC * 16 + (size_t)ROOTS * 24 + (size_t)N * 8 + (size_t)N * 4 + (size_t)nb * nm1 * 4 + 16;
+  }
+};
+
+template <int N>
+__global__ void __launch_bounds__(P1ACfg<N>::THREADS, P1ACfg<N>::CTAS) k_p1_ab(
+    const float2* __restrict__ phi, float2* __restrict__ Ta, float2* __restrict__ Tb, const int16_t* __restrict__ lut,
+    const float* __restrict__ phitab, int nm1, int alpha0, int nb, int nag, int swz, const float2* __restrict__ tw) {
+  using CF = P1ACfg<N>;
+  constexpr int E = CF::E, P = CF::P, TC = CF::TC, H = CF::H, NH = H + 1, RL = CF::RL, NB = CF::NB;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float4* const xch = reinterpret_cast<float4*>(smraw);           // [N][TC]
+  float4* const rw = xch + N * TC;                                // roots
+  float2* const rn = reinterpret_cast<float2*>(rw + CF::ROOTS);
+  float2* const sm_nyq = rn + CF::ROOTS;                          // N values (column 0 only)
+  int* const sm_cn = reinterpret_cast<int*>(sm_nyq + N);          // N cells
+  float* const sm_tab = reinterpret_cast<float*>(sm_cn + N);      // (terms of this CTA) * nm1
+  const int b = blockIdx.z / nag, ag = blockIdx.z % nag;
+  const int alo = (int)((long)nb * ag / nag), ahi = (int)((long)nb * (ag + 1) / nag);  // terms of this CTA
+  uint32_t* const tslot = reinterpret_cast<uint32_t*>(sm_tab + (ahi - alo) * nm1);
+  const int c = threadIdx.x % TC, j = threadIdx.x / TC;
+  const int cc = blockIdx.x * TC + c;
+  const int k1 = blockIdx.y;
+  const int n1 = wrapn(k1, N);
+  const int warp = threadIdx.x >> 5;
+  if (warp == 0) tmem_alloc(tslot, CF::NCOLS);
+  for (int i = threadIdx.x; i < (ahi - alo) * nm1; i += CF::THREADS) sm_tab[i] = phitab[(long)(alpha0 + alo) * nm1 + i];
+  for (int i = threadIdx.x; i < CF::ROOTS; i += CF::THREADS) {
+    const int jj = i % P, q = i / P, t = q / (RL - 1), r = q % (RL - 1) + 1;
+    const int e = r * ((jj + t * P) & 15);  // exponent of e^{+2 pi i / N}
+    const float2 w = __ldg(tw + e);  // e^{-2 pi i e / N}
+    rw[i] = make_float4(w.x, w.x, -w.y, -w.y);
+    rn[i] = make_float2(w.y, w.y);
+  }
+  const float2* pb = phi + ((long)b * N * N + k1) * NH;  // + k0 * N * NH + k2
+  if (blockIdx.x == 0) {
+    for (int k0 = threadIdx.x; k0 < N; k0 += CF::THREADS) {
+      const int n0 = wrapn(k0, N);
+      sm_nyq[k0] = pb[(long)k0 * N * NH + H];
+      sm_cn[k0] = lut[n0 * n0 + n1 * n1 + H * H];
+    }
+  }
+  tmem_fence_before_sync();
+  __syncthreads();
+  tmem_fence_after_sync();
+  const uint32_t tbase = *tslot + ((uint32_t)(32 * warp) << 16);
+  {
+    float u[16];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float2 v = pb[(long)(j + (8 * h + i) * P) * N * NH + cc];
+        u[2 * i] = v.x;
+        u[2 * i + 1] = v.y;
+      }
+      tmem_st16(tbase + 16 * h, u);
+    }
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+      const int n0 = wrapn(j + r * P, N);
+      u[r] = __int_as_float((int)lut[n0 * n0 + n1 * n1 + cc * cc]);
+    }
+    tmem_st16(tbase + 32, u);
+    tmem_wait_st();
+  }
+  const long fstride = (long)N * N * H;  // one field
+  const float fj = (float)j;
+  const int cs = cc ^ ((k1 & 1) * swz);
+  const long toff = ((long)b * nb) * fstride + t_index<float, N>(k1, cs) + (long)j * N * H;
+  float4* const xw = xch + 16 * j * TC + c;  // first-stage outputs 16 j + r
+  float4* const xr = xch + j * TC + c;       // points j + ...
+  auto put = [](const c2& z) { return make_float4(z.r.x, z.r.y, z.i.x, z.i.y); };
+  auto get = [](const float4& x) { return c2{make_float2(x.x, x.y), make_float2(x.z, x.w)}; };
+#pragma unroll 1
+  for (int a = alo; a < ahi; ++a) {
+    const float* tab = sm_tab + (a - alo) * nm1;
+    c2 v[E];
+    {
+      float fl[16], u[32];
+      tmem_ld16(tbase + 32, fl);
+#pragma unroll
+      for (int r = 0; r < E; ++r) fl[r] = tab[__float_as_int(fl[r])];
+      tmem_ld32(tbase, u);
+      // the pair (V, i n0^D V): n0^D of k0 = j + r P (k0 < N/2 exactly when r < E/2; zero on the Nyquist index r = E/2,
+      // j = 0).  NYQ: the CTA holds packed column 0, whose thread c = 0 adds i V(k2 = N/2) with its own cell.
+      auto fill = [&](auto nyq) {
+#pragma unroll
+        for (int r = 0; r < E; ++r) {
+          const float nd = r < E / 2 ? fj + (float)(r * P) : ((r == E / 2 && j == 0) ? 0.f : fj + (float)(r * P - N));
+          float x = fl[r] * u[2 * r], y = fl[r] * u[2 * r + 1];
+          if (decltype(nyq)::value && cc == 0) {
+            const float fn = tab[sm_cn[j + r * P]];
+            const float2 yn = sm_nyq[j + r * P];
+            x = x - fn * yn.y;
+            y = y + fn * yn.x;
+          }
+          v[r] = {make_float2(x, -nd * y), make_float2(y, nd * x)};
+        }
+      };
+      if (blockIdx.x == 0) fill(std::true_type{});
+      else fill(std::false_type{});
+    }
+    idft16c(v);
+    __syncthreads();  // the exchange of the term before has been read
+#pragma unroll
+    for (int r = 0; r < E; ++r) xw[r * TC] = put(v[r]);
+    __syncthreads();
+    float2* const da = Ta + toff + a * fstride;
+    float2* const db = Tb + toff + a * fstride;
+#pragma unroll
+    for (int t = 0; t < NB; ++t) {
+      c2 z[RL];
+#pragma unroll
+      for (int r = 0; r < RL; ++r) {
+        z[r] = get(xr[(t * P + r * (N / RL)) * TC]);
+        if (r) {
+          const int i = (t * (RL - 1) + r - 1) * P + j;
+          z[r] = mulc(z[r], rw[i], rn[i]);
+        }
+      }
+      idftc<RL, true>(z);
+#pragma unroll
+      for (int r = 0; r < RL; ++r) {  // point j + t P + r N / RL
+        da[(long)(t * P + r * (N / RL)) * N * H] = make_float2(z[r].r.x, z[r].i.x);
+        db[(long)(t * P + r * (N / RL)) * N * H] = make_float2(z[r].r.y, z[r].i.y);
+      }
+    }
+  }
+  tmem_fence_before_sync();
+  __syncthreads();
+  tmem_fence_after_sync();
+  if (warp == 0) tmem_dealloc(*tslot, CF::NCOLS);
+}
+
+// P1 with its Phi~ tile and cell indices in tensor memory (autotuner variant bit 16; FP32, N = 256 and 512, radix 16,
+// 256 threads per CTA: 16 or 8 columns).  k_p1 keeps each thread's 16 Phi~ values and cells in registers for all the terms of a launch
 // (125 registers: two CTAs of 8 warps per SM, latency-bound).  Here they sit in the thread's TMEM lane (columns
 // 0-31: Phi~ as (re, im) pairs, 32-47: cells; warps w and w + 4 share a lane quarter, the latter at column 64) and are read back for every transform;
 // with a single exchange buffer (free for a two-stage transform; a three-stage
 // one syncs between a stage's reads and writes) three CTAs share an SM at 80 registers (measured faster than four at
-// 64).  At N <= 256, 8 of each thread's 15 last-stage twiddles also sit in its lane (columns 48-63).  Same arithmetic
+// 64).  At N = 256, 8 of each thread's 15 last-stage twiddles also sit in its lane (columns 48-63).  Same arithmetic
 // as k_p1.
 template <int N>
 struct P1TCfg {
-  static constexpr int H = N / 2, E = 16, P = N / E, TC = 256 / P, THREADS = TC * P;  // 32 / 16 / 8 columns
+  static constexpr int H = N / 2, E = 16, P = N / E, TC = 256 / P, THREADS = TC * P;  // 16 / 8 columns
+  static constexpr int CTAS = 3;
   static_assert(THREADS == 256, "two warps per TMEM lane quarter");
   using Lay = ColLayout<float, N, TC, E, true>;
   static constexpr uint32_t NCOLS = 128;  // per warp group: Phi~ 0-31, cells 32-47, 8 twiddles 48-63 (N <= 256)

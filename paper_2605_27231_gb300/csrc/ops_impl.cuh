@@ -67,18 +67,20 @@ struct OpsT {
     return cudaGetLastError();
   }
   // ------------------------------------------------------------ hot path
-  // CTAs that share the nb terms of one first-pass tile: the number for which the waves of the 456 CTAs that fit the SMs
-  // (three a SM; 0.4 for the uneven end) times a CTA's terms is least, half a term standing for a CTA's set-up (Phi~,
-  // cells, twiddles).  One realisation at N = 64 has 64 tiles: 50 terms took 114 us on 64 SMs (five launches), 35 us in
-  // 7 groups; N = 128, 50 terms: 268 us in one group, 219 us in 7 (three realisations 628, 557 in 3); FP64 N = 32 (32
-  // tiles of 64 threads): 594 us in one, 94 us in 14.  With many tiles (256^3: 2048 and more) there is one group.
-  static int p1_groups(long tiles, int nb) {
+  // CTAs that share the nb terms of one first-pass tile: the number for which the waves of the `slots` CTAs that fit the
+  // SMs (a quarter more for the uneven end) times a CTA's terms is least, half a term standing for a CTA's set-up (Phi~,
+  // cells, roots).  One realisation at N = 64 has 64 tiles: 50 terms took 114 us on 64 SMs (five launches), 32 us in 9
+  // groups; N = 128, 50 terms: 201 us in one group, 173 us in two; FP64 N = 32 (32 tiles of 64 threads): 594 us in one,
+  // 94 us in 14.  With many tiles (256^3: 2048 and more) there is one group.
+  static int p1_groups(long tiles, int nb, int nm1, int slots) {
     int best = 1;
     double least = 1e30;
     for (int g = 1; g <= nb; ++g) {
-      const double waves = tiles * g / 456.0;
-      const double cost = (waves <= 1.0 ? 1.0 : waves + 0.4) * ((nb + g - 1) / g + 0.5);
-      if (cost < 0.97 * least) {  // more groups only for a clear gain
+      // the filter tables of a CTA's terms stay within 64 KB of its shared memory where the terms can be split further
+      if ((long)((nb + g - 1) / g) * nm1 * (long)sizeof(T) > 64 * 1024 && g < nb) continue;
+      const double waves = (double)tiles * g / slots;
+      const double cost = (waves <= 1.0 ? 1.0 : waves + 0.25) * ((nb + g - 1) / g + 0.5);
+      if (cost < 0.99 * least) {  // more groups only for a gain
         least = cost;
         best = g;
       }
@@ -88,7 +90,7 @@ struct OpsT {
   template <int N, int E, int TC>
   static cudaError_t p1_v(const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* phitab, int nm1,
                           int alpha0, int nb, int batch, const void* tw, int swz, cudaStream_t st) {
-    const int nag = p1_groups((long)(N / 2) / TC * N * batch, nb), per = (nb + nag - 1) / nag;
+    const int nag = p1_groups((long)(N / 2) / TC * N * batch, nb, nm1, 456), per = (nb + nag - 1) / nag;
     const size_t sm = strided_bytes<N, TC, E>() + N * sizeof(C) + N * sizeof(int) + (size_t)per * nm1 * sizeof(T);
     auto k = k_p1<T, N, E, TC>;
     SIGW_CHECK_LAUNCH(allow_smem(k, 227 * 1024));
@@ -100,10 +102,13 @@ struct OpsT {
   template <int N>
   static cudaError_t p1_tm_v(const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* phitab, int nm1,
                              int alpha0, int nb, int batch, const void* tw, int swz, cudaStream_t st) {
-    using CF = P1TCfg<N>;
-    const int nag = p1_groups((long)(N / 2) / CF::TC * N * batch, nb), per = (nb + nag - 1) / nag;
+    using CF = std::conditional_t<(N <= 128), P1ACfg<(N <= 128 ? N : 128)>, P1TCfg<N>>;
+    const int nag = p1_groups((long)(N / 2) / CF::TC * N * batch, nb, nm1, 152 * CF::CTAS), per = (nb + nag - 1) / nag;
     const size_t sm = CF::smem(per, nm1);
-    auto k = k_p1_tm<N>;
+    auto k = [] {
+      if constexpr (N <= 128) return k_p1_ab<N>;
+      else return k_p1_tm<N>;
+    }();
     SIGW_CHECK_LAUNCH(allow_smem(k, 227 * 1024));
     dim3 grid((N / 2) / CF::TC, N, batch * nag);
     k<<<grid, CF::THREADS, sm, st>>>((const float2*)phi, (float2*)Ta, (float2*)Tb, lut, (const float*)phitab, nm1,
@@ -116,7 +121,7 @@ struct OpsT {
     using SH = Shape<T, N>;
     using AL = AltStrided<T, N>;
     const int swz = fused_n<N>(variant) ? 8 : 0;  // the fused second and last pass reads swizzled columns
-    if constexpr (sizeof(T) == 4 && (N == 128 || N == 256 || N == 512)) {  // Phi~ tile and cells in tensor memory
+    if constexpr (sizeof(T) == 4 && N >= 64) {  // both transforms side by side, Phi~ tile and cells in tensor memory
       if (variant & 16) return p1_tm_v<N>(phi, Ta, Tb, lut, phitab, nm1, alpha0, nb, batch, tw, swz, st);
     }
     if constexpr (AL::exists) {

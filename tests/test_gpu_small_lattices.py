@@ -47,15 +47,19 @@ def test_split_terms_match_oracle(lib, N, precision, n_alpha):
 
 
 def test_fused_pass_matches_three_passes(lib):
-    """N = 64, FP32, all shells: the fused form (variant bit 8, the default) against the three passes (bit 0)."""
+    """N = 64, FP32, all shells: the untuned choice (bits 24: both transforms of the first pass side by side, second and
+    last pass fused), and each of its two parts alone, against the three passes (bits 0)."""
     spec = workloads.Spec(N=64, L=1.0, A=1e-2, sigma=0.5, kstar=8 * 2 * np.pi, kind="usr", seed=43)
     with lib.Plan(64, 1.0, precision=32, n_alpha=21) as p:
         p.generate_spec(spec)
         fused = p.spectrum()["omega"][0]
         p.set_tuning(16, 0)
         three = p.spectrum()["omega"][0]
-        p.set_tuning(16, 8)
+        p.set_tuning(16, 24)
         assert np.array_equal(p.spectrum()["omega"][0], fused)
+        for bits in (8, 16):
+            p.set_tuning(16, bits)
+            np.testing.assert_allclose(p.spectrum()["omega"][0], three, rtol=2e-5)
     np.testing.assert_allclose(fused, three, rtol=2e-5)  # two FP32 evaluations of the same sums
 
 
