@@ -69,6 +69,10 @@ struct TuneKey {
 std::mutex g_tune_mu;
 std::map<TuneKey, std::pair<int, int>> g_tune;
 
+// Kernels (I_s, I_c) of a shell whose forward passes, shell sums and jackknife share their launches.  Up to N = 128 these
+// are short (8 to 17 us each at 64^3 and 128^3, mostly latency), and the second kernel's run beside the first's.
+int kernels_at_once(int N) { return N <= 128 ? 2 : 1; }
+
 // Sizes (bytes) of every device buffer of a plan.
 struct Sizes {
   size_t phi, T, W, synth, F, F2, partial, out, lut, tab, tw, amp, rows_sq;
@@ -90,14 +94,15 @@ Sizes sizes_of(int N, const sigw_opts& o) {
   s.T = 2 * mb * (size_t)B * NN * H * cel;
   s.W = mb * 6 * (size_t)((o.n_alpha + 1) / 2) * NN * H * cel;  // three full rows per term pair
   // the jackknife reuses W after each shell: two standard + two packed half spectra + two real fields
-  s.W = std::max(s.W, mb * 2 * (NN * NH * cel + NN * H * cel + NN * (size_t)N * rel) + 1024);
+  s.W = std::max(s.W, kernels_at_once(N) * mb * 2 * (NN * NH * cel + NN * H * cel + NN * (size_t)N * rel) + 1024);
   s.synth = mb * (NN * H * cel + NN * NH * cel + 3 * NN * (size_t)N * rel) + 1024;  // + two real fields (non-local map)
   size_t parts = 1;  // partial fields of the last pass
   for (int v : {0, 8})
     parts = std::max(parts, (size_t)(o.precision == 64 ? sigw::OpsRT<double>::last_groups(N, v, o.n_alpha)
                                                        : sigw::OpsRT<float>::last_groups(N, v, o.n_alpha)));
-  s.F = parts * mb * 6 * NN * NH * cel;
-  s.F2 = mb * 6 * NN * NH * cel;
+  const size_t nm = kernels_at_once(N);
+  s.F = parts * nm * mb * 6 * NN * NH * cel;
+  s.F2 = nm * mb * 6 * NN * NH * cel;
   s.partial = mb * H * 2 * (size_t)s.maxblk * sizeof(double);
   s.out = mb * H * 4 * sizeof(double) + H * (sizeof(int) + sizeof(double));
   const size_t msq = 3 * H * H + 1;
@@ -729,8 +734,8 @@ sigw_status sigw_generate(sigw_plan p, const sigw_pzeta* pz, const sigw_ngmap* m
   return sigw_generate_batch(p, pzs.data(), ms.data(), seeds, batch, usr_hits);
 }
 
-// Jackknife scratch of one spectrum call (Sec. sec_envelope_obs): M^3 sub-volumes; per (shell, kernel) the TT
-// amplitudes go to Xj (standard half spectra, 2 per realisation), are packed into Yj, inverse-transformed into
+// Jackknife scratch of one spectrum call (Sec. sec_envelope_obs): M^3 sub-volumes; per (shell, kernel), or per shell where
+// kernels_at_once is 2, the TT amplitudes go to Xj (standard half spectra, 2 per kernel and realisation), are packed into Yj, inverse-transformed into
 // the real fields Rj, and reduced per sub-volume x0-plane into part[(si * 2 + m)][2 batch][M^3][N/M].
 struct Jackknife {
   int M = 4;
@@ -769,12 +774,15 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, con
     long disk = 0;
     for (int n1 = n1lo; n1 < n1lo + nk1; ++n1)
       for (int n2 = 0; n2 <= n_c; ++n2) disk += (n1 * n1 + n2 * n2 <= n_c * n_c + n_c);
+    const int nm = kernels_at_once(N);  // kernels per launch of the passes after the product
+    const long fvals = 6L * batch * (long)NN * ncp, fgs = fvals * nm;  // values of one kernel's F; between groups
     for (int m = 0; m < 2; ++m) {
+      void* F = (char*)p->d_F + (size_t)(m % nm) * fvals * cel;
       if (fused) {
         RUN(p, 1, phib + 2.0 * n_alpha * fieldb, "P1",
             OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[m], nm1, 0, n_alpha, batch, p->d_tw, var, st));
-        RUN(p, 3, 2.0 * n_alpha * fieldb + 6.0 * groups * batch * NN * ncp * cel, "P23",
-            OPS(p, p23, N, Ta, Tb, p->d_sigma[m], n_alpha, p->d_F, groups, n_c, batch, p->d_tw, p->d_err, p->wait_limit,
+        RUN(p, 3, 2.0 * n_alpha * fieldb + (double)groups * fvals * cel, "P23",
+            OPS(p, p23, N, Ta, Tb, p->d_sigma[m], n_alpha, F, groups, fgs, n_c, batch, p->d_tw, p->d_err, p->wait_limit,
                 st));
       }
       for (int a0 = 0; a0 < n_alpha && !fused; a0 += B) {
@@ -785,29 +793,28 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, con
             OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, p->d_err, p->wait_limit, st));
       }
       if (!fused)
-        RUN(p, 3, 3.0 * n_alpha * fieldb + 6.0 * groups * batch * NN * ncp * cel, "P3",
-            OPS(p, p3, N, p->d_work, p->d_sigma[m], n_alpha, p->d_F, groups, n_c, batch, p->d_tw, p->d_err,
+        RUN(p, 3, 3.0 * n_alpha * fieldb + (double)groups * fvals * cel, "P3",
+            OPS(p, p3, N, p->d_work, p->d_sigma[m], n_alpha, F, groups, fgs, n_c, batch, p->d_tw, p->d_err,
                 p->wait_limit, var, st));
-      RUN(p, 4, 6.0 * batch * (groups * (double)NN * ncp + (double)N * nk1 * ncp) * cel, "F2",
-          OPS(p, f2, N, p->d_F, groups, p->d_F2, n_c, batch, p->d_tw, st));
-      if (!jk) {
-        RUN(p, 5, 6.0 * batch * (double)N * disk * cel, "F3",
-            OPS(p, f3, N, p->d_F2, n_c, p->d_partial + ((long)si * 2 + m) * p->sz.maxblk, pbs, batch, p->d_tw, st));
-      } else {
-        const double xjb = 2.0 * batch * NN * (H + 1) * cel, yjb = 2.0 * batch * NN * H * cel;
-        const double rjb = 2.0 * batch * NN * N * p->relem();
-        CKP(p, cudaMemsetAsync(jk->Xj, 0, (size_t)xjb, st), "jackknife zero");
-        RUN(p, 5, 6.0 * batch * (double)N * disk * cel, "F3 + amplitudes",
-            OPS(p, f3, N, p->d_F2, n_c, p->d_partial + ((long)si * 2 + m) * p->sz.maxblk, pbs, batch, p->d_tw, st,
-                jk->Xj));
-        RUN(p, 0, xjb + yjb, "jackknife pack", OPS(p, pack, N, jk->Xj, jk->Yj, 2 * batch, st));
-        RUN(p, 0, 2 * yjb, "jackknife inverse axis 0", OPS(p, pass, N, jk->Yj, 0, +1, 2 * batch, p->d_tw, st));
-        RUN(p, 0, 2 * yjb, "jackknife inverse axis 1", OPS(p, pass, N, jk->Yj, 1, +1, 2 * batch, p->d_tw, st));
+      if (m % nm != nm - 1) continue;  // the forward passes take both kernels
+      const int nf = nm * batch;       // realisations times kernels
+      RUN(p, 4, (double)nm * (groups * (double)fvals + 6.0 * batch * N * nk1 * ncp) * cel, "F2",
+          OPS(p, f2, N, p->d_F, groups, fgs, p->d_F2, n_c, nf, p->d_tw, st));
+      double* part = p->d_partial + ((long)si * 2 + m + 1 - nm) * p->sz.maxblk;
+      if (jk) CKP(p, cudaMemsetAsync(jk->Xj, 0, (size_t)2 * nf * NN * (H + 1) * cel, st), "jackknife zero");
+      RUN(p, 5, 6.0 * nf * (double)N * disk * cel, jk ? "F3 + amplitudes" : "F3",
+          OPS(p, f3, N, p->d_F2, n_c, part, pbs, (long)p->sz.maxblk, nm, batch, p->d_tw, st, jk ? jk->Xj : nullptr));
+      if (jk) {
+        const double xjb = 2.0 * nf * NN * (H + 1) * cel, yjb = 2.0 * nf * NN * H * cel;
+        const double rjb = 2.0 * nf * NN * N * p->relem();
+        RUN(p, 0, xjb + yjb, "jackknife pack", OPS(p, pack, N, jk->Xj, jk->Yj, 2 * nf, st));
+        RUN(p, 0, 2 * yjb, "jackknife inverse axis 0", OPS(p, pass, N, jk->Yj, 0, +1, 2 * nf, p->d_tw, st));
+        RUN(p, 0, 2 * yjb, "jackknife inverse axis 1", OPS(p, pass, N, jk->Yj, 1, +1, 2 * nf, p->d_tw, st));
         RUN(p, 0, yjb + rjb, "jackknife rows C2R",
-            OPS(p, rows_c2r, N, jk->Yj, jk->Rj, 2 * batch, 1.0, nullptr, p->d_tw, st));
+            OPS(p, rows_c2r, N, jk->Yj, jk->Rj, 2 * nf, 1.0, nullptr, p->d_tw, st));
         const long per = 2L * batch * jk->M * jk->M * jk->M * (N / jk->M);
         RUN(p, 0, rjb, "jackknife sub-volumes",
-            OPS(p, subvol, N, jk->M, jk->Rj, 2 * batch, jk->part + ((long)si * 2 + m) * per, st));
+            OPS(p, subvol, N, jk->M, jk->Rj, 2 * nf, jk->part + ((long)si * 2 + m + 1 - nm) * per, st));
       }
     }
   }
@@ -932,8 +939,9 @@ sigw_status sigw_spectrum_jackknife(sigw_plan p, const int* shells, int n_shells
   Jackknife jk;
   jk.M = M;
   jk.Xj = p->d_work;
-  jk.Yj = (char*)jk.Xj + (size_t)2 * batch * NN * (H + 1) * cel;
-  jk.Rj = (char*)jk.Yj + (size_t)2 * batch * NN * H * cel;
+  const size_t nf = (size_t)kernels_at_once(N) * batch;
+  jk.Yj = (char*)jk.Xj + 2 * nf * NN * (H + 1) * cel;
+  jk.Rj = (char*)jk.Yj + 2 * nf * NN * H * cel;
   {
     void* q = nullptr;
     sigw_status s = dev_alloc(p, &q, sizeof(double) * per * 2 * ns);
@@ -1152,13 +1160,14 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
           status = cuda_fail(p, e != cudaSuccess ? e : cudaGetLastError(), "autotune last pass");
       }
     };
+    const long fgs = 6L * batch * (long)NN * (n_c + 1);
     const int np3 = OPS(p, p3_variants, N);  // 2: radix 8 / 16; 3: also radix 16 with TMEM accumulators
     const int p3bits[3] = {0, 2, 8};
     float t3[3] = {1e30f, 1e30f, 1e30f};
     for (int v3 = 0; v3 < np3; ++v3) {
       const int bits = p3bits[v3], groups = OPS(p, last_groups, N, bits, n_alpha);
       time_last(&t3[v3], [&]() {
-        return OPS(p, p3, N, p->d_work, p->d_sigma[0], n_alpha, p->d_F, groups, n_c, batch, p->d_tw, p->d_err,
+        return OPS(p, p3, N, p->d_work, p->d_sigma[0], n_alpha, p->d_F, groups, fgs, n_c, batch, p->d_tw, p->d_err,
                    sigw::kDefaultWaitLimit, bits, st);
       });
     }
@@ -1175,7 +1184,7 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
         cudaError_t e = OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, 0, n_alpha, batch, p->d_tw, bestV | 8,
                             st);
         if (e == cudaSuccess)
-          e = OPS(p, p23, N, Ta, Tb, p->d_sigma[0], n_alpha, p->d_F, OPS(p, last_groups, N, 8, n_alpha), n_c, batch,
+          e = OPS(p, p23, N, Ta, Tb, p->d_sigma[0], n_alpha, p->d_F, OPS(p, last_groups, N, 8, n_alpha), fgs, n_c, batch,
                   p->d_tw, p->d_err, sigw::kDefaultWaitLimit, st);
         return e;
       });

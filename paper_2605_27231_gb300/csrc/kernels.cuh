@@ -1906,16 +1906,23 @@ __global__ void __launch_bounds__(P23Cfg<N>::THREADS, P23Cfg<N>::CTAS) k_p23(
 #pragma unroll
       for (int r = 0; r < E; ++r) (r & 1 ? xw1 : xw0)[16 * (r >> 1)] = v[r];
       __syncwarp();
+      {
+        float w[32];  // the row transform's roots: the same length, and jj = j
+        tmem_ld32(tcol(6), w);
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        float2 a[4];
+        for (int t = 0; t < 4; ++t) {
+          float2 a[4];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) a[r] = (r & 1 ? xr1 : xr0)[8 * (4 * t + 16 * r)];
+          for (int r = 0; r < 4; ++r) a[r] = (r & 1 ? xr1 : xr0)[8 * (4 * t + 16 * r)];
 #pragma unroll
-        for (int r = 1; r < 4; ++r) a[r] = mul<float>(a[r], twN[r * j + 4 * r * t]);
-        dftR<float, +1, 4>(a);
+          for (int r = 1; r < 4; ++r) {
+            const int i = 3 * t + r - 1;
+            a[r] = mul<float>(a[r], make_float2(w[2 * i], w[2 * i + 1]));
+          }
+          dftR<float, +1, 4>(a);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) v[t + 4 * r] = a[r];
+          for (int r = 0; r < 4; ++r) v[t + 4 * r] = a[r];
+        }
       }
       __syncthreads();  // every exchange and every plane read is over
       if (threadIdx.x == 0 && ok) {
@@ -2110,35 +2117,33 @@ __global__ void __launch_bounds__(256) k_f2(const cx<T>* __restrict__ F, int par
 
 // The two TT amplitudes e^+_ij(k_hat) S_ij and e^x_ij(k_hat) S_ij (Sec. sec_sigw basis: u = k x e0 / |k x e0|,
 // e1 in place of e0 when k is parallel to e0, v = k x u; e^+ = (uu - vv)/sqrt2, e^x = (uv + vu)/sqrt2).
-// S = (00, 11, 22, 01, 02, 12).
+// S = (00, 11, 22, 01, 02, 12).  With the integer vector n, m2 = n1^2 + n2^2 and U = (0, n2, -n1), V = (-m2, n0 n1, n0 n2):
+// u = U / sqrt(m2), v = V / (|n| sqrt(m2)), so one root and one division serve all (FP64; six divisions and two roots made
+// this the larger part of a jackknife's last forward pass).
 __device__ __forceinline__ void tt_amp(int n0, int n1, int n2, const double2* S, double2& ap, double2& ax) {
-  const double nn = sqrt((double)(n0 * n0 + n1 * n1 + n2 * n2));
-  const double k0 = n0 / nn, k1 = n1 / nn, k2 = n2 / nn;
-  double u0 = 0.0, u1 = k2, u2 = -k1;  // k x e0
-  double un = sqrt(u1 * u1 + u2 * u2);
-  if (un < 1e-12) {  // k x e1
-    u0 = -k2;
-    u1 = 0.0;
-    u2 = k0;
-    un = sqrt(u0 * u0 + u2 * u2);
-  }
-  u0 /= un;
-  u1 /= un;
-  u2 /= un;
-  const double v0 = k1 * u2 - k2 * u1, v1 = k2 * u0 - k0 * u2, v2 = k0 * u1 - k1 * u0;
-  // S u and S v
   const double2 s00 = S[0], s11 = S[1], s22 = S[2], s01 = S[3], s02 = S[4], s12 = S[5];
-  auto sdot = [&](double a0, double a1, double a2, double c0, double c1, double c2) {
-    // a . S . c
-    double re = a0 * (s00.x * c0 + s01.x * c1 + s02.x * c2) + a1 * (s01.x * c0 + s11.x * c1 + s12.x * c2) +
-                a2 * (s02.x * c0 + s12.x * c1 + s22.x * c2);
-    double im = a0 * (s00.y * c0 + s01.y * c1 + s02.y * c2) + a1 * (s01.y * c0 + s11.y * c1 + s12.y * c2) +
-                a2 * (s02.y * c0 + s12.y * c1 + s22.y * c2);
-    return make_double2(re, im);
+  const double h = 0.70710678118654752440, q = 1.41421356237309504880;
+  const int m2 = n1 * n1 + n2 * n2;
+  if (m2 == 0) {  // k along e0: u = (0, 0, sign n0), v = (0, -1, 0)
+    const double sg = n0 < 0 ? q : -q;
+    ap = make_double2((s22.x - s11.x) * h, (s22.y - s11.y) * h);
+    ax = make_double2(sg * s12.x, sg * s12.y);
+    return;
+  }
+  const double a0 = n0, a1 = n1, a2 = n2, m = m2, nn2 = (double)(n0 * n0 + m2);
+  const double inv = 1.0 / (nn2 * m);  // 1 / (|n|^2 m2)
+  const double iu = nn2 * inv, iw = sqrt(nn2) * inv;
+  auto part = [&](double p00, double p11, double p22, double p01, double p02, double p12, double& plus, double& cross) {
+    const double uu = a2 * a2 * p11 + a1 * a1 * p22 - 2.0 * a1 * a2 * p12;
+    const double x1 = a1 * p01 + a2 * p02;                                   // (0, n1, n2) . S . e0
+    const double x2 = a1 * a1 * p11 + a2 * a2 * p22 + 2.0 * a1 * a2 * p12;   // (0, n1, n2) . S . (0, n1, n2)
+    const double vv = m * m * p00 - 2.0 * m * a0 * x1 + a0 * a0 * x2;
+    const double uv = -m * (a2 * p01 - a1 * p02) + a0 * (a1 * a2 * (p11 - p22) + (a2 * a2 - a1 * a1) * p12);
+    plus = (uu * iu - vv * inv) * h;
+    cross = uv * iw * q;
   };
-  const double2 uu = sdot(u0, u1, u2, u0, u1, u2), vv = sdot(v0, v1, v2, v0, v1, v2), uv = sdot(u0, u1, u2, v0, v1, v2);
-  ap = make_double2((uu.x - vv.x) * 0.70710678118654752440, (uu.y - vv.y) * 0.70710678118654752440);
-  ax = make_double2(uv.x * 1.41421356237309504880, uv.y * 1.41421356237309504880);
+  part(s00.x, s11.x, s22.x, s01.x, s02.x, s12.x, ap.x, ax.x);
+  part(s00.y, s11.y, s22.y, s01.y, s02.y, s12.y, ap.y, ax.y);
 }
 // Sum over the two polarisations of |e^l_ij(k_hat) S_ij|^2, written with the TT projector instead of the basis:
 // sum_l e^l_ij e^l_lm = (P_il P_jm + P_im P_jl - P_ij P_lm) / 2 with P = I - n n^T / |n|^2, which annihilates the
@@ -2193,10 +2198,12 @@ __device__ __forceinline__ double tt_power_f32(int n0, int n1, int n2, const flo
 // With Xj (jackknife), the amplitudes of the stored shell modes are also written to the standard half spectra
 // Xj[b][0] = e^+ : S and Xj[b][1] = -i e^x : S (both Hermitian in this basis away from the Nyquist shell),
 // [b][f][k0][k1][k2], k2 = 0..N/2; every other entry is left as it is (zero).
+// blockIdx.z = m * batch + b: the fields of kernel m follow those of the one before (F2 and Xj), and its partial sums are
+// mstride further.
 template <typename T, int N>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_f3(const cx<T>* __restrict__ F2, int n_c, int n1lo, int nk1,
-                                            double* __restrict__ partial, long pbstride,
-                                            const cx<T>* __restrict__ tw, cx<T>* __restrict__ Xj) {
+                                            double* __restrict__ partial, long pbstride, long mstride,
+                                            int batch, const cx<T>* __restrict__ tw, cx<T>* __restrict__ Xj) {
   using SH = Shape<T, N>;
   constexpr int E = SH::E3, P = SH::P3, TC = SH::TC3, H = N / 2;
   using Lay = ColLayout<T, N, TC, E>;
@@ -2207,13 +2214,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_f3(const cx<T>*
   const int ncp = n_c + 1;
   const int k1i = blockIdx.y;
   const int n1 = n1lo + k1i;
-  const int b = blockIdx.z;
+  const int b = blockIdx.z;  // m * batch + realisation
+  partial += (long)(b % batch) * pbstride + (long)(b / batch) * mstride;
   const long blk = (long)blockIdx.y * gridDim.x + blockIdx.x;
   const int cc0 = blockIdx.x * TC;
   const int rmax = n_c * n_c + n_c;  // |n|^2 < (n_c + 1/2)^2
   const int rmin = n_c * n_c - n_c + 1;  // |n|^2 >= (n_c - 1/2)^2
   if (!(cc0 < ncp && n1 * n1 + cc0 * cc0 <= rmax)) {  // no column of this tile reaches the shell
-    if (threadIdx.x == 0) partial[(long)b * pbstride + blk] = 0.0;
+    if (threadIdx.x == 0) partial[blk] = 0.0;
     return;
   }
   const int cc = cc0 + c;
@@ -2274,7 +2282,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_f3(const cx<T>*
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) t += red[w];
-    partial[(long)b * pbstride + blk] = t;
+    partial[blk] = t;
   }
 }
 

@@ -63,24 +63,28 @@ struct OpsRT {
   // cycles after which a wait of the main loop gives up (kDefaultWaitLimit unless a test shrinks it).
   // variant bit 2 selects the radix-16 form where p3_variants(N) >= 2; bit 8 the radix-16 form with its
   // accumulators in tensor memory where p3_variants(N) == 3 (FP32, N = 128, 256, 512).
-  // groups: the term pairs are split into that many groups, each writing its own F (6 batch N^2 (n_c + 1) values).
+  // groups: the term pairs are split into that many groups, each writing its own F (6 batch N^2 (n_c + 1) values),
+  // fgstride values apart.
   static int p3_variants(int N);
-  static cudaError_t p3(int N, const void* W, const void* sigma, int n_alpha, void* F, int groups, int n_c, int batch,
-                        const void* tw, int* err, long long wait_limit, int variant, cudaStream_t st);
+  static cudaError_t p3(int N, const void* W, const void* sigma, int n_alpha, void* F, int groups, long fgstride,
+                        int n_c, int batch, const void* tw, int* err, long long wait_limit, int variant,
+                        cudaStream_t st);
   // FP32, N = 64 with variant bit 8: one kernel for the second and the last inverse pass, from the first
   // pass's output for all terms (Ta, Tb [batch][n_alpha], columns swizzled by p1 for that variant); W is not used.
   static bool fused(int N, int variant);
   static cudaError_t p23(int N, const void* Ta, const void* Tb, const void* sigma, int n_alpha, void* F, int groups,
-                         int n_c, int batch, const void* tw, int* err, long long wait_limit, cudaStream_t st);
+                         long fgstride, int n_c, int batch, const void* tw, int* err, long long wait_limit,
+                         cudaStream_t st);
   // groups that fill the SMs for one realisation (1 for the tensor-memory last pass)
   static int last_groups(int N, int variant, int n_alpha);
   // forward pass along axis 1 keeping |n1| <= n_c, of the sum of the groups' fields
-  static cudaError_t f2(int N, const void* F, int groups, void* F2, int n_c, int batch, const void* tw,
+  static cudaError_t f2(int N, const void* F, int groups, long fgstride, void* F2, int n_c, int batch, const void* tw,
                         cudaStream_t st);
   // forward pass along axis 0 + TT projection + shell sum -> per-CTA FP64 partials; with Xj (nullable) also the
-  // two TT amplitudes of every stored shell mode into the zeroed standard half spectra Xj[batch][2]
-  static cudaError_t f3(int N, const void* F2, int n_c, double* partial, long pbstride, int batch, const void* tw,
-                        cudaStream_t st, void* Xj = nullptr);
+  // two TT amplitudes of every stored shell mode into the zeroed standard half spectra Xj[nm][batch][2].  nm: kernels
+  // in F2, one behind the other; the partial sums of the second are mstride further
+  static cudaError_t f3(int N, const void* F2, int n_c, double* partial, long pbstride, long mstride, int nm, int batch,
+                        const void* tw, cudaStream_t st, void* Xj = nullptr);
   // jackknife: sum of R^2 over each x0-plane of each of the M^3 sub-volumes, out[field][M^3][N/M]
   static cudaError_t subvol(int N, int M, const void* R, int nfields, double* out, cudaStream_t st);
 };

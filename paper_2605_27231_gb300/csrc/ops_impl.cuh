@@ -135,15 +135,15 @@ struct OpsT {
     return sizeof(T) == 4 && N == 64 && (variant & 8);
   }
   template <int N>
-  static cudaError_t p23_n(const void* Ta, const void* Tb, const void* sigma, int n_alpha, void* F, int groups, int n_c,
-                           int batch, const void* tw, int* err, long long wait_limit, cudaStream_t st) {
+  static cudaError_t p23_n(const void* Ta, const void* Tb, const void* sigma, int n_alpha, void* F, int groups,
+                           long fgstride, int n_c, int batch, const void* tw, int* err, long long wait_limit, cudaStream_t st) {
     if constexpr (sizeof(T) == 4 && N == 64) {
       using CF = P23Cfg<N>;
       auto k = k_p23<N>;
       SIGW_CHECK_LAUNCH(allow_smem(k, CF::SMEM));
       dim3 grid(N, batch, groups);
       k<<<grid, CF::THREADS, CF::SMEM, st>>>((const float2*)Ta, (const float2*)Tb, (const float*)sigma, n_alpha,
-                                             (float2*)F, 6L * batch * N * N * (n_c + 1), n_c, (const float2*)tw, err,
+                                             (float2*)F, fgstride, n_c, (const float2*)tw, err,
                                              wait_limit);
       return cudaGetLastError();
     } else {
@@ -185,14 +185,14 @@ struct OpsT {
     return cudaGetLastError();
   }
   template <int N, int E>
-  static cudaError_t p3_v(const void* W, const void* sigma, int n_alpha, void* F, int groups, int n_c, int batch,
-                          const void* tw, int* err, long long wait_limit, cudaStream_t st) {
+  static cudaError_t p3_v(const void* W, const void* sigma, int n_alpha, void* F, int groups, long fgstride, int n_c,
+                          int batch, const void* tw, int* err, long long wait_limit, cudaStream_t st) {
     using CF = P3Cfg<T, N, E>;
     auto k = k_p3<T, N, E>;
     SIGW_CHECK_LAUNCH(allow_smem(k, CF::SMEM));
     dim3 grid((N * N) / CF::RPC, batch, groups);
-    k<<<grid, CF::THREADS, CF::SMEM, st>>>((const C*)W, (const T*)sigma, n_alpha, (C*)F, 6L * batch * N * N * (n_c + 1),
-                                           n_c, (const C*)tw, err, wait_limit);
+    k<<<grid, CF::THREADS, CF::SMEM, st>>>((const C*)W, (const T*)sigma, n_alpha, (C*)F, fgstride, n_c,
+                                           (const C*)tw, err, wait_limit);
     return cudaGetLastError();
   }
   template <int N>
@@ -207,16 +207,16 @@ struct OpsT {
     return cudaGetLastError();
   }
   template <int N>
-  static cudaError_t p3_n(const void* W, const void* sigma, int n_alpha, void* F, int groups, int n_c, int batch,
-                          const void* tw, int* err, long long wait_limit, int variant, cudaStream_t st) {
+  static cudaError_t p3_n(const void* W, const void* sigma, int n_alpha, void* F, int groups, long fgstride, int n_c,
+                          int batch, const void* tw, int* err, long long wait_limit, int variant, cudaStream_t st) {
     if constexpr (sizeof(T) == 4 && (N == 128 || N == 256 || N == 512)) {  // accumulators in tensor memory
       if (variant & 8) return p3_tm_v<N>(W, sigma, n_alpha, F, n_c, batch, tw, err, wait_limit, st);
     }
     if constexpr (AltP3<T, N>::exists) {
       if (variant & 2)
-        return p3_v<N, AltP3<T, N>::E>(W, sigma, n_alpha, F, groups, n_c, batch, tw, err, wait_limit, st);
+        return p3_v<N, AltP3<T, N>::E>(W, sigma, n_alpha, F, groups, fgstride, n_c, batch, tw, err, wait_limit, st);
     }
-    return p3_v<N, ((N >= 16) ? 8 : 4)>(W, sigma, n_alpha, F, groups, n_c, batch, tw, err, wait_limit, st);
+    return p3_v<N, ((N >= 16) ? 8 : 4)>(W, sigma, n_alpha, F, groups, fgstride, n_c, batch, tw, err, wait_limit, st);
   }
   static void n1_range(int N, int n_c, int* lo, int* nk1) {
     const int H = N / 2;
@@ -226,7 +226,8 @@ struct OpsT {
     *nk1 = bhi - a + 1;
   }
   template <int N>
-  static cudaError_t f2_n(const void* F, int groups, void* F2, int n_c, int batch, const void* tw, cudaStream_t st) {
+  static cudaError_t f2_n(const void* F, int groups, long fgstride, void* F2, int n_c, int batch, const void* tw,
+                          cudaStream_t st) {
     using SH = Shape<T, N>;
     const size_t sm = (size_t)ColLayout<T, N, SH::TC, SH::ES, true>::SIZE * sizeof(C);  // single exchange buffer
     auto k = k_f2<T, N>;
@@ -234,21 +235,21 @@ struct OpsT {
     int lo, nk1;
     n1_range(N, n_c, &lo, &nk1);
     dim3 grid((n_c + 1 + SH::TC - 1) / SH::TC, N, batch * 6);
-    k<<<grid, SH::TC * SH::PS, sm, st>>>((const C*)F, groups, 6L * batch * N * N * (n_c + 1), (C*)F2, n_c, lo, nk1,
-                                         (const C*)tw);
+    k<<<grid, SH::TC * SH::PS, sm, st>>>((const C*)F, groups, fgstride, (C*)F2, n_c, lo, nk1, (const C*)tw);
     return cudaGetLastError();
   }
   template <int N>
-  static cudaError_t f3_n(const void* F2, int n_c, double* partial, long pbs, int batch, const void* tw,
-                          cudaStream_t st, void* Xj) {
+  static cudaError_t f3_n(const void* F2, int n_c, double* partial, long pbs, long mstride, int nm, int batch,
+                          const void* tw, cudaStream_t st, void* Xj) {
     using SH = Shape<T, N>;
     const size_t sm = col_bytes<N, SH::TC3, SH::E3>();
     auto k = k_f3<T, N>;
     SIGW_CHECK_LAUNCH(allow_smem(k, sm));
     int lo, nk1;
     n1_range(N, n_c, &lo, &nk1);
-    dim3 grid((n_c + 1 + SH::TC3 - 1) / SH::TC3, nk1, batch);
-    k<<<grid, SH::TC3 * SH::P3, sm, st>>>((const C*)F2, n_c, lo, nk1, partial, pbs, (const C*)tw, (C*)Xj);
+    dim3 grid((n_c + 1 + SH::TC3 - 1) / SH::TC3, nk1, nm * batch);
+    k<<<grid, SH::TC3 * SH::P3, sm, st>>>((const C*)F2, n_c, lo, nk1, partial, pbs, mstride, batch, (const C*)tw,
+                                           (C*)Xj);
     return cudaGetLastError();
   }
   template <int N>
@@ -403,25 +404,25 @@ int OpsRT<T>::last_groups(int N, int variant, int n_alpha) {
 }
 template <typename T>
 cudaError_t OpsRT<T>::p23(int N, const void* Ta, const void* Tb, const void* sigma, int n_alpha, void* F, int groups,
-                          int n_c, int batch, const void* tw, int* err, long long wait_limit, cudaStream_t st) {
+                          long fgstride, int n_c, int batch, const void* tw, int* err, long long wait_limit, cudaStream_t st) {
   if (N != 64) return cudaErrorInvalidValue;
-  return OpsT<T>::template p23_n<64>(Ta, Tb, sigma, n_alpha, F, groups, n_c, batch, tw, err, wait_limit, st);
+  return OpsT<T>::template p23_n<64>(Ta, Tb, sigma, n_alpha, F, groups, fgstride, n_c, batch, tw, err, wait_limit, st);
 }
 template <typename T>
-cudaError_t OpsRT<T>::p3(int N, const void* W, const void* sigma, int n_alpha, void* F, int groups, int n_c, int batch,
-                      const void* tw, int* err, long long wait_limit, int variant, cudaStream_t st) {
-  SIGW_DISPATCH_N(N, return (OpsT<T>::template p3_n<NN>(W, sigma, n_alpha, F, groups, n_c, batch, tw, err, wait_limit,
+cudaError_t OpsRT<T>::p3(int N, const void* W, const void* sigma, int n_alpha, void* F, int groups, long fgstride,
+                      int n_c, int batch, const void* tw, int* err, long long wait_limit, int variant, cudaStream_t st) {
+  SIGW_DISPATCH_N(N, return (OpsT<T>::template p3_n<NN>(W, sigma, n_alpha, F, groups, fgstride, n_c, batch, tw, err, wait_limit,
                                                        variant, st)));
 }
 template <typename T>
-cudaError_t OpsRT<T>::f2(int N, const void* F, int groups, void* F2, int n_c, int batch, const void* tw,
+cudaError_t OpsRT<T>::f2(int N, const void* F, int groups, long fgstride, void* F2, int n_c, int batch, const void* tw,
                          cudaStream_t st) {
-  SIGW_DISPATCH_N(N, return (OpsT<T>::template f2_n<NN>(F, groups, F2, n_c, batch, tw, st)));
+  SIGW_DISPATCH_N(N, return (OpsT<T>::template f2_n<NN>(F, groups, fgstride, F2, n_c, batch, tw, st)));
 }
 template <typename T>
-cudaError_t OpsRT<T>::f3(int N, const void* F2, int n_c, double* partial, long pbs, int batch, const void* tw,
-                      cudaStream_t st, void* Xj) {
-  SIGW_DISPATCH_N(N, return (OpsT<T>::template f3_n<NN>(F2, n_c, partial, pbs, batch, tw, st, Xj)));
+cudaError_t OpsRT<T>::f3(int N, const void* F2, int n_c, double* partial, long pbs, long mstride, int nm, int batch,
+                      const void* tw, cudaStream_t st, void* Xj) {
+  SIGW_DISPATCH_N(N, return (OpsT<T>::template f3_n<NN>(F2, n_c, partial, pbs, mstride, nm, batch, tw, st, Xj)));
 }
 template <typename T>
 cudaError_t OpsRT<T>::subvol(int N, int M, const void* R, int nfields, double* out, cudaStream_t st) {
