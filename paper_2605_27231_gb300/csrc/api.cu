@@ -93,6 +93,8 @@ Sizes sizes_of(int N, const sigw_opts& o) {
   s.phi = mb * NN * NH * cel;
   s.T = 2 * mb * (size_t)B * NN * H * cel;
   s.W = mb * 6 * (size_t)((o.n_alpha + 1) / 2) * NN * H * cel;  // three full rows per term pair
+  if (o.precision == 32 && N == 64)  // or the first pass's output of both kernels (fused second and last pass)
+    s.W = std::max(s.W, mb * 4 * (size_t)o.n_alpha * NN * H * cel);
   // the jackknife reuses W after each shell: two standard + two packed half spectra + two real fields
   s.W = std::max(s.W, kernels_at_once(N) * mb * 2 * (NN * NH * cel + NN * H * cel + NN * (size_t)N * rel) + 1024);
   s.synth = mb * (NN * H * cel + NN * NH * cel + 3 * NN * (size_t)N * rel) + 1024;  // + two real fields (non-local map)
@@ -504,10 +506,10 @@ sigw_status sigw_plan_create(int N, double L, const sigw_opts* opts, void* cuda_
   ALLOC(p->d_shells, H * sizeof(int));
   ALLOC(p->d_Nk, H * sizeof(double));
   ALLOC(p->d_lut, p->sz.lut);
-  for (int m = 0; m < 2; ++m) {
-    ALLOC(p->d_phitab[m], (size_t)o.n_alpha * (o.n_modes + 1) * rel);
-    ALLOC(p->d_sigma[m], (size_t)o.n_alpha * rel);
-  }
+  ALLOC(p->d_phitab[0], 2 * (size_t)o.n_alpha * (o.n_modes + 1) * rel);  // the kernels' tables one behind the other
+  ALLOC(p->d_sigma[0], 2 * (size_t)o.n_alpha * rel);
+  p->d_phitab[1] = (char*)p->d_phitab[0] + (size_t)o.n_alpha * (o.n_modes + 1) * rel;
+  p->d_sigma[1] = (char*)p->d_sigma[0] + (size_t)o.n_alpha * rel;
   ALLOC(p->d_tw, (size_t)N * cel);
   ALLOC(p->d_amp, mb * (p->msq_max + 1) * rel);
   ALLOC(p->d_gen, mb * (sizeof(sigw::MapArgs) + sizeof(sigw::PzArgs) + sizeof(uint64_t)));
@@ -756,11 +758,11 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, con
   const size_t NN = (size_t)N * N;
   const size_t cel = p->celem();
   const int var = p->variant;
-  // the fused second and last pass takes the first pass's output of all terms, kept in W's place (it needs no W)
+  // the fused second and last pass takes the first pass's output of all terms of both kernels, kept in W's place
   const bool fused = OPS(p, fused, N, var);
   const int B = launch_terms(N, p->opts, p->B);
   void* Ta = fused ? p->d_work : p->d_T;
-  void* Tb = (char*)Ta + (size_t)batch * (fused ? n_alpha : B) * NN * H * cel;
+  void* Tb = (char*)Ta + (size_t)batch * (fused ? 2 * n_alpha : B) * NN * H * cel;
   const int groups = OPS(p, last_groups, N, var, n_alpha);
   const long pbs = (long)ns * 2 * p->sz.maxblk;
   const double fieldb = (double)batch * NN * H * cel;  // one packed complex field per realisation batch
@@ -778,17 +780,18 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, con
     const long fvals = 6L * batch * (long)NN * ncp, fgs = fvals * nm;  // values of one kernel's F; between groups
     for (int m = 0; m < 2; ++m) {
       void* F = (char*)p->d_F + (size_t)(m % nm) * fvals * cel;
-      if (fused) {
-        RUN(p, 1, phib + 2.0 * n_alpha * fieldb, "P1",
-            OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[m], nm1, 0, n_alpha, batch, p->d_tw, var, st));
-        RUN(p, 3, 2.0 * n_alpha * fieldb + (double)groups * fvals * cel, "P23",
-            OPS(p, p23, N, Ta, Tb, p->d_sigma[m], n_alpha, F, groups, fgs, n_c, batch, p->d_tw, p->d_err, p->wait_limit,
+      if (fused && m == 0) {  // both kernels
+        RUN(p, 1, phib + 4.0 * n_alpha * fieldb, "P1",
+            OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, 2, (long)n_alpha * nm1, 0, n_alpha, batch, p->d_tw,
+                var, st));
+        RUN(p, 3, 4.0 * n_alpha * fieldb + (double)groups * fgs * cel, "P23",
+            OPS(p, p23, N, Ta, Tb, p->d_sigma[0], n_alpha, F, groups, fgs, n_c, batch, p->d_tw, p->d_err, p->wait_limit,
                 st));
       }
       for (int a0 = 0; a0 < n_alpha && !fused; a0 += B) {
         const int nb = std::min(B, n_alpha - a0);
         RUN(p, 1, phib + 2.0 * nb * fieldb, "P1",
-            OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[m], nm1, a0, nb, batch, p->d_tw, var, st));
+            OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[m], nm1, 1, 0L, a0, nb, batch, p->d_tw, var, st));
         RUN(p, 2, 5.0 * nb * fieldb, "P2",
             OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, p->d_err, p->wait_limit, st));
       }
@@ -1100,7 +1103,7 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
       for (int a0 = 0; a0 < n_alpha; a0 += B) {
         const int nb = std::min(B, n_alpha - a0);
         cudaError_t e = which == 0
-                            ? OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, a0, nb, batch, p->d_tw, v, st)
+                            ? OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, 1, 0L, a0, nb, batch, p->d_tw, v, st)
                             : OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, p->d_err,
                                   sigw::kDefaultWaitLimit, st);
         if (e != cudaSuccess) return cuda_fail(p, e, "autotune launch");
@@ -1144,7 +1147,7 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
       void* Tb = (char*)p->d_T + (size_t)batch * B * NN * H * cel;
       for (int a0 = 0; a0 < n_alpha && status == SIGW_OK; a0 += B) {
         const int nb = std::min(B, n_alpha - a0);
-        cudaError_t e = OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, a0, nb, batch, p->d_tw, bestV, st);
+        cudaError_t e = OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, 1, 0L, a0, nb, batch, p->d_tw, bestV, st);
         if (e == cudaSuccess)
           e = OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, p->d_err, sigw::kDefaultWaitLimit, st);
         if (e != cudaSuccess) status = cuda_fail(p, e, "autotune launch");
@@ -1160,7 +1163,7 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
           status = cuda_fail(p, e != cudaSuccess ? e : cudaGetLastError(), "autotune last pass");
       }
     };
-    const long fgs = 6L * batch * (long)NN * (n_c + 1);
+    const long fgs = 6L * batch * (long)NN * (n_c + 1) * kernels_at_once(N);
     const int np3 = OPS(p, p3_variants, N);  // 2: radix 8 / 16; 3: also radix 16 with TMEM accumulators
     const int p3bits[3] = {0, 2, 8};
     float t3[3] = {1e30f, 1e30f, 1e30f};
@@ -1179,15 +1182,16 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
     if (has_fused) {
       float tf = 1e30f;
       void* Ta = p->d_work;
-      void* Tb = (char*)p->d_work + (size_t)batch * n_alpha * NN * H * cel;
+      void* Tb = (char*)p->d_work + (size_t)batch * 2 * n_alpha * NN * H * cel;
       time_last(&tf, [&]() {
-        cudaError_t e = OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, 0, n_alpha, batch, p->d_tw, bestV | 8,
-                            st);
+        cudaError_t e = OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, 2, (long)n_alpha * nm1, 0,
+                            n_alpha, batch, p->d_tw, bestV | 8, st);
         if (e == cudaSuccess)
           e = OPS(p, p23, N, Ta, Tb, p->d_sigma[0], n_alpha, p->d_F, OPS(p, last_groups, N, 8, n_alpha), fgs, n_c, batch,
                   p->d_tw, p->d_err, sigw::kDefaultWaitLimit, st);
         return e;
       });
+      tf *= 0.5f;  // it does both kernels
       if (status == SIGW_OK && tf < best) {
         best = tf;
         bestP3 = 8;
