@@ -52,9 +52,9 @@ int buffer_terms(int N, const sigw_opts& o) {
   return std::max(2, N == 128 && o.alpha_batch == 0 && b == 16 ? std::min(o.n_alpha, 26) : b);
 }
 
-// Terms per launch for the choice B: equal parts of at most B (N = 128: see buffer_terms), in whole pairs.
+// Terms per launch for the choice B: equal parts of at most B (N = 128: see buffer_terms) and 256, in whole pairs.
 int launch_terms(int N, const sigw_opts& o, int B) {
-  const int most = std::max(2, B == max_alpha_batch(o) ? buffer_terms(N, o) : B) & ~1;
+  const int most = std::min(256, std::max(2, B == max_alpha_batch(o) ? buffer_terms(N, o) : B)) & ~1;
   const int launches = (o.n_alpha + most - 1) / most;
   return ((o.n_alpha + launches - 1) / launches + 1) & ~1;
 }
@@ -665,8 +665,7 @@ static sigw_status generate_impl(sigw_plan p, const sigw_pzeta* pz, const sigw_n
         OPS(p, unpack, N, Y, p->d_phi, batch, p->d_amp, (long)msq1, 2.0 / 3.0, 0, st));
   } else {  // Gaussian members of a mixed batch go through the identity map
     RUN(p, 0, Yb + Xb, "unpack (zeta_g)", OPS(p, unpack, N, Y, X, batch, p->d_amp, (long)msq1, 1.0, 0, st));
-    RUN(p, 0, Yb + Xb, "pack", OPS(p, pack, N, X, Y, batch, st));
-    RUN(p, 0, 2 * Yb, "inverse axis 0", OPS(p, pass, N, Y, 0, +1, batch, p->d_tw, st));
+    RUN(p, 0, Yb + Xb, "pack + inverse axis 0", OPS(p, pass_pack, N, X, Y, batch, p->d_tw, st));
     RUN(p, 0, 2 * Yb, "inverse axis 1", OPS(p, pass, N, Y, 1, +1, batch, p->d_tw, st));
     const double scale = 1.0 / ((double)NN * N * dx * dx * dx);
     RUN(p, 0, Yb + Rb, "rows C2R (zeta_g)", OPS(p, rows_c2r, N, Y, R, batch, scale, p->d_sq, p->d_tw, st));
@@ -679,16 +678,14 @@ static sigw_status generate_impl(sigw_plan p, const sigw_pzeta* pz, const sigw_n
       R2 = (char*)R + (size_t)p->opts.max_batch * NN * N * p->relem();
       R3 = (char*)R2 + (size_t)p->opts.max_batch * NN * N * p->relem();
       const double lap = kf * kf;
-      RUN(p, 0, Xb + Yb, "pack lap(zeta_g)", OPS(p, pack, N, X, Y, batch, st, lap));
-      RUN(p, 0, 2 * Yb, "inverse axis 0", OPS(p, pass, N, Y, 0, +1, batch, p->d_tw, st));
+      RUN(p, 0, Xb + Yb, "lap(zeta_g) inverse axis 0", OPS(p, pass_pack, N, X, Y, batch, p->d_tw, st, lap));
       RUN(p, 0, 2 * Yb, "inverse axis 1", OPS(p, pass, N, Y, 1, +1, batch, p->d_tw, st));
       RUN(p, 0, Yb + Rb, "rows C2R lap(zeta_g)", OPS(p, rows_c2r, N, Y, R2, batch, scale, nullptr, p->d_tw, st));
       RUN(p, 0, Rb + Yb, "zeta_g^2 rows R2C", OPS(p, rows_r2c_square, N, R, Y, batch, p->d_tw, st));
       RUN(p, 0, 2 * Yb, "forward axis 1", OPS(p, pass, N, Y, 1, -1, batch, p->d_tw, st));
       RUN(p, 0, 2 * Yb, "forward axis 0", OPS(p, pass, N, Y, 0, -1, batch, p->d_tw, st));
       RUN(p, 0, Yb + Xb, "unpack (zeta_g^2)", OPS(p, unpack, N, Y, X, batch, nullptr, 0L, dx * dx * dx, 1, st));
-      RUN(p, 0, Xb + Yb, "pack lap(zeta_g^2)", OPS(p, pack, N, X, Y, batch, st, lap));
-      RUN(p, 0, 2 * Yb, "inverse axis 0", OPS(p, pass, N, Y, 0, +1, batch, p->d_tw, st));
+      RUN(p, 0, Xb + Yb, "lap(zeta_g^2) inverse axis 0", OPS(p, pass_pack, N, X, Y, batch, p->d_tw, st, lap));
       RUN(p, 0, 2 * Yb, "inverse axis 1", OPS(p, pass, N, Y, 1, +1, batch, p->d_tw, st));
       RUN(p, 0, Yb + Rb, "rows C2R lap(zeta_g^2)", OPS(p, rows_c2r, N, Y, R3, batch, scale, nullptr, p->d_tw, st));
     }
@@ -810,8 +807,7 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, con
       if (jk) {
         const double xjb = 2.0 * nf * NN * (H + 1) * cel, yjb = 2.0 * nf * NN * H * cel;
         const double rjb = 2.0 * nf * NN * N * p->relem();
-        RUN(p, 0, xjb + yjb, "jackknife pack", OPS(p, pack, N, jk->Xj, jk->Yj, 2 * nf, st));
-        RUN(p, 0, 2 * yjb, "jackknife inverse axis 0", OPS(p, pass, N, jk->Yj, 0, +1, 2 * nf, p->d_tw, st));
+        RUN(p, 0, xjb + yjb, "jackknife inverse axis 0", OPS(p, pass_pack, N, jk->Xj, jk->Yj, 2 * nf, p->d_tw, st));
         RUN(p, 0, 2 * yjb, "jackknife inverse axis 1", OPS(p, pass, N, jk->Yj, 1, +1, 2 * nf, p->d_tw, st));
         RUN(p, 0, yjb + rjb, "jackknife rows C2R",
             OPS(p, rows_c2r, N, jk->Yj, jk->Rj, 2 * nf, 1.0, nullptr, p->d_tw, st));
@@ -1065,8 +1061,7 @@ sigw_status sigw_fft3d(sigw_plan p, int direction, const void* in_dev, void* out
     RUN(p, 0, 0, "forward axis 0", OPS(p, pass, N, Y, 0, -1, 1, p->d_tw, st));
     RUN(p, 0, 0, "unpack", OPS(p, unpack, N, Y, out_dev, 1, nullptr, 0L, 1.0, 1, st));
   } else {
-    RUN(p, 0, 0, "pack", OPS(p, pack, N, in_dev, Y, 1, st));
-    RUN(p, 0, 0, "inverse axis 0", OPS(p, pass, N, Y, 0, +1, 1, p->d_tw, st));
+    RUN(p, 0, 0, "pack + inverse axis 0", OPS(p, pass_pack, N, in_dev, Y, 1, p->d_tw, st));
     RUN(p, 0, 0, "inverse axis 1", OPS(p, pass, N, Y, 1, +1, 1, p->d_tw, st));
     RUN(p, 0, 0, "rows C2R", OPS(p, rows_c2r, N, Y, out_dev, 1, 1.0, nullptr, p->d_tw, st));
   }

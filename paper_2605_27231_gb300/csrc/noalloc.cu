@@ -96,8 +96,7 @@ cudaError_t run_fft(int N, int direction, const void* in, void* out, void* scrat
     if ((e = O::pass(N, scratch, 0, -1, 1, tw, st)) != cudaSuccess) return e;
     return O::unpack(N, scratch, out, 1, nullptr, 0, 1.0, 1, st);
   }
-  if ((e = O::pack(N, in, scratch, 1, st)) != cudaSuccess) return e;
-  if ((e = O::pass(N, scratch, 0, +1, 1, tw, st)) != cudaSuccess) return e;
+  if ((e = O::pass_pack(N, in, scratch, 1, tw, st)) != cudaSuccess) return e;
   if ((e = O::pass(N, scratch, 1, +1, 1, tw, st)) != cudaSuccess) return e;
   return O::rows_c2r(N, scratch, out, 1, 1.0, nullptr, tw, st);
 }

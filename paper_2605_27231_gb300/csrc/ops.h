@@ -43,8 +43,10 @@ struct OpsRT {
   // mode 1: times factor
   static cudaError_t unpack(int N, const void* Y, void* X, int batch, const void* amp, long amp_bstride, double factor,
                             int mode, cudaStream_t st);
-  // lap != 0: times -lap |n|^2 (spectral Laplacian for lap = k_f^2)
-  static cudaError_t pack(int N, const void* X, void* Y, int batch, cudaStream_t st, double lap = 0.0);
+  // inverse pass along axis 0 from the standard half spectrum X into the packed Y; lap != 0: times -lap |n|^2 (spectral
+  // Laplacian for lap = k_f^2)
+  static cudaError_t pass_pack(int N, const void* X, void* Y, int batch, const void* tw, cudaStream_t st,
+                               double lap = 0.0);
   static int rows_blocks(int N);  // CTAs per realisation of rows_c2r (entries of sq_partial per realisation)
   static LaunchShape shape(int N);
 

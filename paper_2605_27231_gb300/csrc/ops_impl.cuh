@@ -59,11 +59,21 @@ struct OpsT {
   template <int N, int DIR, int AX>
   static cudaError_t pass_n(void* Y, int batch, const void* tw, cudaStream_t st) {
     using SH = Shape<T, N>;
-    const size_t sm = col_bytes<N, SH::TC, SH::ES>();
+    const size_t sm = (size_t)ColLayout<T, N, SH::TC, SH::ES, true>::SIZE * sizeof(C);
     auto k = k_pass<T, N, DIR, AX>;
     SIGW_CHECK_LAUNCH(allow_smem(k, sm));
     dim3 grid((N / 2) / SH::TC, N, batch);
     k<<<grid, SH::TC * SH::PS, sm, st>>>((C*)Y, (const C*)tw);
+    return cudaGetLastError();
+  }
+  template <int N, bool LAP>
+  static cudaError_t pass_pack_n(const void* X, void* Y, int batch, double lap, const void* tw, cudaStream_t st) {
+    using SH = Shape<T, N>;
+    const size_t sm = (size_t)ColLayout<T, N, SH::TC, SH::ES, true>::SIZE * sizeof(C);
+    auto k = k_pass_pack<T, N, LAP>;
+    SIGW_CHECK_LAUNCH(allow_smem(k, sm));
+    dim3 grid((N / 2) / SH::TC, N, batch);
+    k<<<grid, SH::TC * SH::PS, sm, st>>>((const C*)X, (C*)Y, lap, (const C*)tw);
     return cudaGetLastError();
   }
   // ------------------------------------------------------------ hot path
@@ -75,9 +85,9 @@ struct OpsT {
   static int p1_groups(long tiles, int nb, int nm1, int slots) {
     int best = 1;
     double least = 1e30;
-    for (int g = 1; g <= nb; ++g) {
+    for (int g = 1; g <= nb && g <= 256; ++g) {
       // the filter tables of a CTA's terms stay within 64 KB of its shared memory where the terms can be split further
-      if ((long)((nb + g - 1) / g) * nm1 * (long)sizeof(T) > 64 * 1024 && g < nb) continue;
+      if ((long)((nb + g - 1) / g) * nm1 * (long)sizeof(T) > 64 * 1024 && g < nb && g < 256) continue;
       const double waves = (double)tiles * g / slots;
       const double cost = (waves <= 1.0 ? 1.0 : waves + 0.25) * ((nb + g - 1) / g + 0.5);
       if (cost < 0.99 * least) {  // more groups only for a gain
@@ -334,13 +344,9 @@ cudaError_t OpsRT<T>::unpack(int N, const void* Y, void* X, int batch, const voi
   return cudaGetLastError();
 }
 template <typename T>
-cudaError_t OpsRT<T>::pack(int N, const void* X, void* Y, int batch, cudaStream_t st, double lap) {
-  const long total = (long)batch * N * N * (N / 2);
-  const int thr = 256;
-  long blocks = (total + thr - 1) / thr;
-  if (blocks > 152 * 32) blocks = 152 * 32;
-  k_pack<T><<<(int)blocks, thr, 0, st>>>((const cx<T>*)X, (cx<T>*)Y, N, total, lap);
-  return cudaGetLastError();
+cudaError_t OpsRT<T>::pass_pack(int N, const void* X, void* Y, int batch, const void* tw, cudaStream_t st, double lap) {
+  if (lap != 0.0) { SIGW_DISPATCH_N(N, return (OpsT<T>::template pass_pack_n<NN, true>(X, Y, batch, lap, tw, st))); }
+  SIGW_DISPATCH_N(N, return (OpsT<T>::template pass_pack_n<NN, false>(X, Y, batch, lap, tw, st)));
 }
 template <typename T>
 int OpsRT<T>::rows_blocks(int N) {
