@@ -1739,11 +1739,12 @@ __global__ void __launch_bounds__(P1TCfg<N>::THREADS, 3) k_p1_tm(const float2* _
 //   - Rows: the transformed columns go to the row buffer (two block barriers a transform, the only ones), a warp owns
 //     8 rows, and the exchange of the row transform (radix 16 then 4) is in place.
 // Bounded waits, error flag and the drain before exit as in k_p3.
-// What bounds it: the shared-memory path (ncu, 50 terms of one realisation: 277 wavefronts a warp and transform, 62 % of
-// the path's cycles while active) with 16 warps a SM, issue 50 %; DRAM 17 %.  Both kernels of a shell run in one launch,
-// each with two groups of term pairs: 256 CTAs for one realisation, two a SM.  50 terms of both kernels of one realisation
-// take 146 us (with four groups and a launch per kernel 161; k_p2 and k_p3 before 432), of eight 915 us (976; 2044).  The same split at N = 128 (two residue classes of a1 per plane) was slower than the three
-// passes there (715 against 690 us): its shared-memory traffic grows while HBM already carries the passes.
+// What bounds it: the shared-memory path (ncu: 277 wavefronts a warp and transform, 62 % of the path's cycles while
+// active) with 16 warps a SM, issue 50 %; DRAM 17 %.  Both kernels of a shell run in one launch, each with two groups of
+// term pairs: 256 CTAs for one realisation, two a SM.  50 terms of both kernels of one realisation take 146 us (with four
+// groups and a launch per kernel 161; k_p2 and k_p3 before 432), of eight 915 us (976; 2044).  The same split at N = 128
+// (two residue classes of a1 per plane) was slower than the two passes there (715 against 690 us then, 545 now): its
+// shared-memory traffic grows while HBM already carries the passes.
 template <int N>
 struct P23Cfg {
   static_assert(N == 64, "one plane per CTA, two CTAs per SM");
