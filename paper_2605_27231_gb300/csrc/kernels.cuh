@@ -319,7 +319,7 @@ __global__ void k_unpack(const cx<T>* __restrict__ Y, cx<T>* __restrict__ X, int
 // Inverse C2C transforms along axis 0 from the standard half spectrum X into the packed array Y: column 0 takes
 // X(k2 = 0) + i X(k2 = H).  With LAP each value is first multiplied by -lap |n|^2 (the spectral Laplacian for
 // lap = k_f^2; a Nyquist index counts as n = +N/2, which is exact for the second derivative).  (A pass of its own for the
-// packing read and wrote the whole spectrum once more: inverse transform at 256^3 FP32 105 us, now 78.)
+// packing read and wrote the whole spectrum once more: inverse transform at 256^3 FP32 105 us, now 78 to 84.)
 template <typename T, int N, bool LAP>
 __global__ void __launch_bounds__(256) k_pass_pack(const cx<T>* __restrict__ X, cx<T>* __restrict__ Y, double lap,
                                                    const cx<T>* __restrict__ tw) {
