@@ -73,6 +73,9 @@ std::map<TuneKey, std::pair<int, int>> g_tune;
 // are short (8 to 17 us each at 64^3 and 128^3, mostly latency), and the second kernel's run beside the first's.
 int kernels_at_once(int N) { return N <= 128 ? 2 : 1; }
 
+// Parameters of one realisation in d_gen / h_gen.
+constexpr size_t kGenBytes = sizeof(sigw::MapArgs) + sizeof(sigw::PzArgs) + sizeof(uint64_t);
+
 // Sizes (bytes) of every device buffer of a plan.
 struct Sizes {
   size_t phi, T, W, synth, F, F2, partial, out, lut, tab, tw, amp, rows_sq;
@@ -106,7 +109,7 @@ Sizes sizes_of(int N, const sigw_opts& o) {
   s.F = parts * nm * mb * 6 * NN * NH * cel;
   s.F2 = nm * mb * 6 * NN * NH * cel;
   s.partial = mb * H * 2 * (size_t)s.maxblk * sizeof(double);
-  s.out = mb * H * 4 * sizeof(double) + H * (sizeof(int) + sizeof(double));
+  s.out = mb * H * 4 * sizeof(double) + H * sizeof(double);
   const size_t msq = 3 * H * H + 1;
   s.lut = H * msq * sizeof(int16_t);
   s.tab = 2 * ((size_t)o.n_alpha * (o.n_modes + 1) + o.n_alpha) * rel;
@@ -150,24 +153,19 @@ struct sigw_plan_s {
   void* d_res = nullptr;  // the error flag (16 bytes), then d_out: read back in one copy
   double* d_out = nullptr;
   unsigned char* h_res = nullptr;  // pinned host copy of d_res
-  int* d_shells = nullptr;
-  double* d_Nk = nullptr;
+  double* d_Nk = nullptr;  // modes of shell 1..N/2
   int16_t* d_lut = nullptr;
   void* d_phitab[2] = {nullptr, nullptr};
   void* d_sigma[2] = {nullptr, nullptr};
   void* d_tw = nullptr;
   void* d_amp = nullptr;            // [max_batch][msq_max + 1] synthesis amplitudes
-  unsigned char* d_gen = nullptr;   // one upload per sigw_generate: the next three arrays
-  sigw::MapArgs* d_maps = nullptr;  // [max_batch] map parameters
-  sigw::PzArgs* d_pz = nullptr;     // [max_batch]
+  unsigned char* d_gen = nullptr;   // parameters of sigw_generate's realisations: maps, P_zeta, seeds
+  unsigned char* h_gen = nullptr;   // pinned; the copy to d_gen is queued, so each target of a scan has its own place
   double* d_sq = nullptr;
   double* d_mean = nullptr;
   unsigned long long* d_hits = nullptr;
-  uint64_t* d_seeds = nullptr;
   int* d_err = nullptr;  // OR-ed by kernels whose bounded waits gave up
   long long wait_limit = sigw::kDefaultWaitLimit;  // cycles of P3's main-loop waits (sigw_plan_debug_wait_limit)
-  int* d_shells_all = nullptr;   // 1..N/2, for the all-shells call (no upload, so it can be captured)
-  double* d_Nk_all = nullptr;
   // CUDA graph of the all-shells spectrum loop, per realisation count
   cudaGraphExec_t graph = nullptr;
   int graph_batch = 0;
@@ -503,7 +501,6 @@ sigw_status sigw_plan_create(int N, double L, const sigw_opts* opts, void* cuda_
   ALLOC(p->d_res, 16 + mb * H * 4 * sizeof(double));
   p->d_err = (int*)p->d_res;
   p->d_out = (double*)((char*)p->d_res + 16);
-  ALLOC(p->d_shells, H * sizeof(int));
   ALLOC(p->d_Nk, H * sizeof(double));
   ALLOC(p->d_lut, p->sz.lut);
   ALLOC(p->d_phitab[0], 2 * (size_t)o.n_alpha * (o.n_modes + 1) * rel);  // the kernels' tables one behind the other
@@ -512,23 +509,20 @@ sigw_status sigw_plan_create(int N, double L, const sigw_opts* opts, void* cuda_
   p->d_sigma[1] = (char*)p->d_sigma[0] + (size_t)o.n_alpha * rel;
   ALLOC(p->d_tw, (size_t)N * cel);
   ALLOC(p->d_amp, mb * (p->msq_max + 1) * rel);
-  ALLOC(p->d_gen, mb * (sizeof(sigw::MapArgs) + sizeof(sigw::PzArgs) + sizeof(uint64_t)));
-  p->d_maps = (sigw::MapArgs*)p->d_gen;
-  p->d_pz = (sigw::PzArgs*)(p->d_maps + mb);
-  p->d_seeds = (uint64_t*)(p->d_pz + mb);
+  ALLOC(p->d_gen, mb * kGenBytes);
   const int rb = OPS(p, rows_blocks, N);
   ALLOC(p->d_sq, mb * rb * sizeof(double));
   ALLOC(p->d_mean, mb * sizeof(double));
   ALLOC(p->d_hits, mb * sizeof(unsigned long long));
-  ALLOC(p->d_shells_all, H * sizeof(int));
-  ALLOC(p->d_Nk_all, H * sizeof(double));
 #undef ALLOC
   if (cudaMemset(p->d_err, 0, sizeof(int)) != cudaSuccess) return bail(SIGW_ECUDA);
-  if (cudaMallocHost((void**)&p->h_res, 16 + mb * H * 4 * sizeof(double)) != cudaSuccess) {
-    (void)cudaGetLastError();
-    p->h_res = nullptr;
-    return bail(SIGW_ENOMEM);
-  }
+  for (auto [ptr, bytes] : {std::pair{&p->h_res, 16 + mb * H * 4 * sizeof(double)},
+                            std::pair{&p->h_gen, std::max(mb, (size_t)H) * kGenBytes}})
+    if (cudaMallocHost((void**)ptr, bytes) != cudaSuccess) {
+      (void)cudaGetLastError();
+      *ptr = nullptr;
+      return bail(SIGW_ENOMEM);
+    }
   // tables
   std::vector<unsigned char> buf;
   {
@@ -564,13 +558,8 @@ sigw_status sigw_plan_create(int N, double L, const sigw_opts* opts, void* cuda_
       p->tuned_from_table = true;
     }
   }
-  {
-    std::vector<int> sh(H);
-    for (int i = 0; i < H; ++i) sh[i] = i + 1;
-    if (cudaMemcpy(p->d_shells_all, sh.data(), sizeof(int) * H, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(p->d_Nk_all, p->Nk.data() + 1, sizeof(double) * H, cudaMemcpyHostToDevice) != cudaSuccess)
-      return bail(SIGW_ECUDA);
-  }
+  if (cudaMemcpy(p->d_Nk, p->Nk.data() + 1, sizeof(double) * H, cudaMemcpyHostToDevice) != cudaSuccess)
+    return bail(SIGW_ECUDA);
   *out = p;
   return SIGW_OK;
 }
@@ -581,6 +570,7 @@ sigw_status sigw_plan_destroy(sigw_plan p) {
   if (p->graph) cudaGraphExecDestroy(p->graph);
   for (void* q : p->allocs) cudaFree(q);
   if (p->h_res) cudaFreeHost(p->h_res);
+  if (p->h_gen) cudaFreeHost(p->h_gen);
   prof_reset(p);
   for (cudaEvent_t e : p->pool) cudaEventDestroy(e);
   if (p->own_stream && p->st) cudaStreamDestroy(p->st);
@@ -610,9 +600,10 @@ sigw_status sigw_synchronize(sigw_plan p) {
 }  // extern "C" (a helper of the entry points follows)
 
 // sigw_generate_batch; without `wait` the work is only queued (for calls that follow on the plan's stream), and floor
-// hits are neither read back nor checked.
+// hits are neither read back nor checked.  The parameters go through the places of h_gen from `place` on, which a call that
+// does not wait leaves to the queued copy until the stream has been waited for.
 static sigw_status generate_impl(sigw_plan p, const sigw_pzeta* pz, const sigw_ngmap* maps, const uint64_t* seeds,
-                                 int batch, int64_t* usr_hits, bool wait) {
+                                 int batch, int64_t* usr_hits, bool wait, int place = 0) {
   if (!p) return SIGW_EINVAL;
   if (!pz || !maps || !seeds || batch < 1 || batch > p->opts.max_batch)
     return fail(p, SIGW_EINVAL, "sigw_generate: bad arguments");
@@ -632,12 +623,13 @@ static sigw_status generate_impl(sigw_plan p, const sigw_pzeta* pz, const sigw_n
   const size_t NN = (size_t)N * N;
   const size_t msq1 = p->msq_max + 1;
   cudaStream_t st = p->st;
-  // parameters of every realisation in one upload: maps, P_zeta, seeds (in the places of a full batch)
-  const size_t mb = p->opts.max_batch;
-  std::vector<unsigned char> buf(mb * (sizeof(sigw::MapArgs) + sizeof(sigw::PzArgs) + sizeof(uint64_t)));
-  sigw::MapArgs* margs = (sigw::MapArgs*)buf.data();
-  sigw::PzArgs* pargs = (sigw::PzArgs*)(margs + mb);
-  std::memcpy(pargs + mb, seeds, sizeof(uint64_t) * batch);
+  // parameters of every realisation in one upload: maps, P_zeta, seeds
+  sigw::MapArgs* margs = (sigw::MapArgs*)(p->h_gen + place * kGenBytes);
+  sigw::PzArgs* pargs = (sigw::PzArgs*)(margs + batch);
+  std::memcpy(pargs + batch, seeds, sizeof(uint64_t) * batch);
+  const sigw::MapArgs* d_maps = (const sigw::MapArgs*)p->d_gen;
+  const sigw::PzArgs* d_pz = (const sigw::PzArgs*)(d_maps + batch);
+  const uint64_t* d_seeds = (const uint64_t*)(d_pz + batch);
   for (int b = 0; b < batch; ++b) {
     pargs[b] = sigw::PzArgs{pz[b].A, pz[b].sigma, pz[b].kstar};
     const double ks2 = pz[b].kstar * pz[b].kstar;
@@ -646,10 +638,10 @@ static sigw_status generate_impl(sigw_plan p, const sigw_pzeta* pz, const sigw_n
                    : sigw::MapArgs{maps[b].kind, maps[b].F_NL, maps[b].G_NL,
                                    maps[b].usr_floor > 0 ? maps[b].usr_floor : 1e-6};
   }
-  CKP(p, cudaMemcpyAsync(p->d_gen, buf.data(), buf.size(), cudaMemcpyHostToDevice, st), "upload parameters");
-  p->h2d += buf.size();
+  CKP(p, cudaMemcpyAsync(p->d_gen, margs, batch * kGenBytes, cudaMemcpyHostToDevice, st), "upload parameters");
+  p->h2d += batch * kGenBytes;
   RUN(p, 0, (double)batch * msq1 * p->relem(), "amplitudes",
-      sigw::launch_amp(p->d_pz, p->d_amp, (long)msq1, L, N, p->opts.precision, batch, st));
+      sigw::launch_amp(d_pz, p->d_amp, (long)msq1, L, N, p->opts.precision, batch, st));
   const size_t cel = p->celem();
   char* work = (char*)p->d_work;
   void* Y = work;
@@ -657,7 +649,7 @@ static sigw_status generate_impl(sigw_plan p, const sigw_pzeta* pz, const sigw_n
   void* R = (char*)X + (size_t)p->opts.max_batch * NN * (H + 1) * cel;
   const double Yb = (double)batch * NN * H * cel, Xb = (double)batch * NN * (H + 1) * cel;
   const double Rb = (double)batch * NN * N * p->relem();
-  RUN(p, 0, Yb, "noise + rows R2C", OPS(p, rows_r2c_noise, N, Y, p->d_seeds, batch, p->d_tw, st));
+  RUN(p, 0, Yb, "noise + rows R2C", OPS(p, rows_r2c_noise, N, Y, d_seeds, batch, p->d_tw, st));
   RUN(p, 0, 2 * Yb, "forward axis 1", OPS(p, pass, N, Y, 1, -1, batch, p->d_tw, st));
   RUN(p, 0, 2 * Yb, "forward axis 0", OPS(p, pass, N, Y, 0, -1, batch, p->d_tw, st));
   if (all_gauss) {
@@ -691,7 +683,7 @@ static sigw_status generate_impl(sigw_plan p, const sigw_pzeta* pz, const sigw_n
     }
     CKP(p, cudaMemsetAsync(p->d_hits, 0, sizeof(unsigned long long) * batch, st), "memset hits");
     RUN(p, 0, Rb + Yb + (any_nonlocal ? 2 * Rb : 0.0), "map + rows R2C",
-        OPS(p, rows_r2c_map, N, R, Y, batch, p->d_maps, p->d_mean, p->d_hits, p->d_tw, st, R2, R3));
+        OPS(p, rows_r2c_map, N, R, Y, batch, d_maps, p->d_mean, p->d_hits, p->d_tw, st, R2, R3));
     RUN(p, 0, 2 * Yb, "forward axis 1", OPS(p, pass, N, Y, 1, -1, batch, p->d_tw, st));
     RUN(p, 0, 2 * Yb, "forward axis 0", OPS(p, pass, N, Y, 0, -1, batch, p->d_tw, st));
     RUN(p, 0, Yb + Xb, "unpack (Phi)",
@@ -744,9 +736,8 @@ struct Jackknife {
   void* Rj = nullptr;
 };
 
-// Queue the hot loop for the shells sh (device copies in d_sh / d_nk) writing [batch][ns][4] to out.
-static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, const int* d_sh, const double* d_nk,
-                                    double* out, const Jackknife* jk = nullptr) {
+// Queue the hot loop for the shells sh writing [batch][ns][4] to out.
+static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, double* out, const Jackknife* jk = nullptr) {
   const int N = p->N, H = N / 2;
   const int ns = (int)sh.size();
   const int batch = p->generated;
@@ -818,8 +809,10 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, con
     }
   }
   const sigw::LaunchShape shp = OPS(p, shape, N);
+  sigw::ShellList list;
+  for (int i = 0; i < ns; ++i) list.n_c[i] = (int16_t)sh[i];
   RUN(p, 6, (double)batch * ns * 2 * p->sz.maxblk * 8, "bin finalise",
-      sigw::launch_fin(p->d_partial, pbs, p->sz.maxblk, ns, d_sh, d_nk, N, p->L, shp.tc_f3, out, batch, st));
+      sigw::launch_fin(p->d_partial, pbs, p->sz.maxblk, ns, list, p->d_Nk, N, p->L, shp.tc_f3, out, batch, st));
   return SIGW_OK;
 }
 
@@ -838,7 +831,7 @@ static bool capture_all_shells(sigw_plan p, const std::vector<int>& sh) {
     (void)cudaGetLastError();
     return false;
   }
-  const sigw_status s = enqueue_spectrum(p, sh, p->d_shells_all, p->d_Nk_all, p->d_out);
+  const sigw_status s = enqueue_spectrum(p, sh, p->d_out);
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(p->st, &g);
   bool ok = (s == SIGW_OK && e == cudaSuccess && g);
@@ -904,14 +897,9 @@ sigw_status sigw_spectrum_async(sigw_plan p, const int* shells, int n_shells, do
         return SIGW_OK;
       }
     }
-    return enqueue_spectrum(p, sh, p->d_shells_all, p->d_Nk_all, out);
+    return enqueue_spectrum(p, sh, out);
   }
-  std::vector<double> nk(ns);
-  for (int i = 0; i < ns; ++i) nk[i] = p->Nk[sh[i]];
-  CKP(p, cudaMemcpyAsync(p->d_shells, sh.data(), sizeof(int) * ns, cudaMemcpyHostToDevice, st), "upload shells");
-  CKP(p, cudaMemcpyAsync(p->d_Nk, nk.data(), sizeof(double) * ns, cudaMemcpyHostToDevice, st), "upload Nk");
-  p->h2d += sizeof(int) * ns + sizeof(double) * ns;
-  return enqueue_spectrum(p, sh, p->d_shells, p->d_Nk, out);
+  return enqueue_spectrum(p, sh, out);
 }
 
 sigw_status sigw_spectrum_jackknife(sigw_plan p, const int* shells, int n_shells, int M, double* omega,
@@ -951,14 +939,7 @@ sigw_status sigw_spectrum_jackknife(sigw_plan p, const int* shells, int n_shells
     p->allocs.erase(std::remove(p->allocs.begin(), p->allocs.end(), (void*)jk.part), p->allocs.end());
     cudaFree(jk.part);
   };
-  std::vector<double> nk(ns);
-  for (int i = 0; i < ns; ++i) nk[i] = p->Nk[sh[i]];
-  sigw_status s = SIGW_OK;
-  if (cudaMemcpyAsync(p->d_shells, sh.data(), sizeof(int) * ns, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemcpyAsync(p->d_Nk, nk.data(), sizeof(double) * ns, cudaMemcpyHostToDevice, st) != cudaSuccess)
-    s = cuda_fail(p, cudaGetLastError(), "upload shells");
-  p->h2d += sizeof(int) * ns + sizeof(double) * ns;
-  if (s == SIGW_OK) s = enqueue_spectrum(p, sh, p->d_shells, p->d_Nk, p->d_out, &jk);
+  sigw_status s = enqueue_spectrum(p, sh, p->d_out, &jk);
   std::vector<double> part(per * 2 * ns), res((size_t)batch * ns * 4);
   if (s == SIGW_OK &&
       (cudaMemcpyAsync(part.data(), jk.part, sizeof(double) * part.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -1279,10 +1260,8 @@ sigw_status sigw_target_scan(sigw_plan p, const sigw_pzeta* pz, const sigw_ngmap
       const int i = i0 + queued;
       p->L = box[i];
       p->generated = 0;
-      if ((s = generate_impl(p, pz, map, &seed, 1, nullptr, strict)) != SIGW_OK) break;
-      if ((s = enqueue_spectrum(p, {nc[i]}, p->d_shells_all + nc[i] - 1, p->d_Nk_all + nc[i] - 1,
-                                p->d_out + 4 * queued)) != SIGW_OK)
-        break;
+      if ((s = generate_impl(p, pz, map, &seed, 1, nullptr, strict, queued)) != SIGW_OK) break;
+      if ((s = enqueue_spectrum(p, {nc[i]}, p->d_out + 4 * queued)) != SIGW_OK) break;
     }
     if (queued) {
       const std::string msg = p->err;

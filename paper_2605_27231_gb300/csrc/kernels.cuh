@@ -2363,11 +2363,11 @@ __global__ void k_amp(const PzArgs* __restrict__ pz, T* __restrict__ amp, long m
 // One CTA per (realisation, shell), two warps per kernel: 64 threads add strided partials, then a
 // fixed tree.  (One thread per pair walked up to 33 k partials: 0.52 ms at 256^3, 1.04 ms at 512^3.)
 __global__ void __launch_bounds__(128) k_fin(const double* __restrict__ partial, long pbstride, int maxblk, int n_shells,
-                                             const int* __restrict__ shells, const double* __restrict__ Nk, int N,
-                                             double L, int tc3, double* __restrict__ out) {
+                                             const __grid_constant__ ShellList shells,
+                                             const double* __restrict__ Nk, int N, double L, int tc3, double* __restrict__ out) {
   __shared__ double red[4];
   const int b = blockIdx.x / n_shells, s = blockIdx.x % n_shells;
-  const int n_c = shells[s];
+  const int n_c = shells.n_c[s];
   const int H = N / 2;
   const int n1lo = max(-n_c, -H + 1), n1hi = min(n_c, H);
   const int nk1 = n1hi - n1lo + 1;
@@ -2384,7 +2384,7 @@ __global__ void __launch_bounds__(128) k_fin(const double* __restrict__ partial,
   const double pi = 3.14159265358979323846;
   const double V = L * L * L, dx = L / N;
   const double C = 4.0 * dx * dx * dx / ((double)n_c * n_c * V * V);
-  const double nk = Nk[s];
+  const double nk = Nk[n_c - 1];
   const double PA = C * C * (red[0] + red[1]) / (V * nk), PB = C * C * (red[2] + red[3]) / (V * nk);
   const double kc = n_c * 2.0 * pi / L;
   double* o = out + (long)blockIdx.x * 4;

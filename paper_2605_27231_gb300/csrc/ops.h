@@ -25,6 +25,10 @@ struct PzArgs {  // P_zeta of one realisation (Eq. eq_lognormal)
   double A, sigma, kstar;
 };
 
+struct ShellList {  // target shells of a spectrum call, passed by value: a queued upload would need its host copy kept
+  int16_t n_c[256];
+};
+
 template <typename T>
 struct OpsRT {
   // ---- synthesis chain (packed layout [b][a0][a1][N/2], standard layout [b][k0][k1][N/2+1])
@@ -98,7 +102,8 @@ extern template struct OpsRT<double>;
 
 // precision-independent kernels (defined in ops_f64.cu)
 cudaError_t launch_reduce_mean(const double* part, int nblk, double* mean, int batch, double inv, cudaStream_t st);
-cudaError_t launch_fin(const double* partial, long pbstride, int maxblk, int n_shells, const int* shells,
+// Nk[n_c - 1]: modes of shell n_c
+cudaError_t launch_fin(const double* partial, long pbstride, int maxblk, int n_shells, const ShellList& shells,
                        const double* Nk, int N, double L, int tc3, double* out, int batch, cudaStream_t st);
 
 // synthesis amplitudes amp[batch][msq1] in the plan precision

@@ -9,7 +9,7 @@ cudaError_t launch_reduce_mean(const double* part, int nblk, double* mean, int b
   return cudaGetLastError();
 }
 
-cudaError_t launch_fin(const double* partial, long pbstride, int maxblk, int n_shells, const int* shells,
+cudaError_t launch_fin(const double* partial, long pbstride, int maxblk, int n_shells, const ShellList& shells,
                        const double* Nk, int N, double L, int tc3, double* out, int batch, cudaStream_t st) {
   k_fin<<<batch * n_shells, 128, 0, st>>>(partial, pbstride, maxblk, n_shells, shells, Nk, N, L, tc3, out);
   return cudaGetLastError();

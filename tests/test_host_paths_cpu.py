@@ -1,0 +1,64 @@
+"""The host side of the library (csrc/api.cu, csrc/serve.cu) on a simulated device (tests/hostsim): buffer sizes, lifetimes
+of host and device memory and the order of launches are checked for the calls a user makes, without a GPU."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2605_27231_gb300", "csrc")
+SIM = os.path.join(ROOT, "tests", "hostsim")
+
+
+@pytest.fixture(scope="module")
+def sim_lib(tmp_path_factory):
+    if not shutil.which("g++"):
+        pytest.skip("no host compiler")
+    from paper_2605_27231_gb300 import build, sigw
+    real = build.build()
+    so = str(tmp_path_factory.mktemp("sim") / "libsim.so")
+    src = [os.path.join(CSRC, f) for f in ("api.cu", "serve.cu", "plan.cpp")] + [os.path.join(SIM, "sim.cpp")]
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", SIM, "-I", CSRC, "-x", "c++",
+                    *src, "-ldl", "-lpthread", "-o", so], check=True)
+    lib = ctypes.CDLL(so)
+    lib.sim_init(real.encode())
+    lib.sim_launches.restype = ctypes.c_long
+    lib.sim_device_bytes.restype = ctypes.c_size_t
+    lib.sim_faults.restype = ctypes.c_char_p
+    return lib, so, sigw
+
+
+@pytest.fixture
+def sim(sim_lib, monkeypatch):
+    """The package's binding on the simulated device; every test has to end without a fault."""
+    lib, so, sigw = sim_lib
+    monkeypatch.setattr(sigw, "LIB_PATH", so)
+    monkeypatch.setattr(sigw, "_lib", None)
+    lib.sim_faults()
+    yield sigw
+    assert lib.sim_faults().decode() == ""
+
+
+def _run(p, batch=1, shells=(1,), **kw):
+    p.generate(1e-2, 0.5, 10.0, seeds=list(range(1, batch + 1)), **kw)
+    p.spectrum(list(shells))
+
+
+# ---- host memory that a queued copy may still read
+
+def test_queued_uploads_keep_their_host_buffers(sim):
+    """Synthesis parameters and shell lists of calls that return, or go on, before the stream was waited for."""
+    import ctypes as C
+    with sim.Plan(16, 1.0, precision=64, n_alpha=5, max_batch=3) as p:
+        p.target_scan(np.geomspace(0.3, 2.5, 19), 1e-2, 0.5, 1.0, "local", 2.0, seed=3)
+        _run(p, 3, (8, 2, 5, 2))
+        p.generate(1e-2, 0.5, 10.0, "nonlocal", alpha_NL=1.0, seeds=(1, 2))
+        p.spectrum_async(None, [3, 1])
+        assert sim.lib().sigw_spectrum_async(p.handle, None, 0, None) == sim.OK  # all shells, captured
+        p.generate(1e-2, 0.5, 10.0, "usr")
+        p.spectrum_async(None, [1])
+        p.synchronize()
+        p.spectrum_jackknife([1, 4])
