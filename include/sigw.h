@@ -239,9 +239,9 @@ sigw_status sigw_server_destroy(sigw_server srv);
 /* Autotuner (no counterpart in the paper).  On the plan's current field, times the two strided inverse passes of
  * one target shell (n_c; 0 picks N/4) for every candidate choice: terms per launch in {4, 5, 8, 10, 16} (at most
  * n_alpha; exactly opts->alpha_batch when that is set) and, where more than one exists (FP32, N >= 64), the forms of
- * the first strided pass (two radices, and its Phi~ tile and cells in tensor memory).  Keeps the fastest in the plan and
- * in a process-wide table keyed by (N, precision, max_batch, n_alpha) from which later plans with alpha_batch = 0 start;
- * then times the forms of the last inverse pass (FP32, N = 128, 256, 512: two radices, and radix 16 with its accumulators
+ * the first strided pass (two radices, and its Phi~ tile and cells in tensor memory).  Keeps the fastest in the plan and,
+ * if opts->alpha_batch is 0, in a process-wide table keyed by (N, precision, max_batch, n_alpha) from which later plans
+ * with alpha_batch = 0 start; then times the forms of the last inverse pass (FP32, N = 128, 256, 512: two radices, and radix 16 with its accumulators
  * in tensor memory) on the terms just produced, and at FP32 N = 64 the fused second and last pass against the three
  * passes.  An untuned FP32 plan starts from 16 terms and the bits measured fastest on GB300 (24 at N = 64, 26 from
  * N = 128 on).  Terms go in equal launches of whole pairs of at most the chosen number; at N = 128 the largest choice, 16,

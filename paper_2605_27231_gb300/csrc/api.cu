@@ -52,14 +52,17 @@ int buffer_terms(int N, const sigw_opts& o) {
   return std::max(2, N == 128 && o.alpha_batch == 0 && b == 16 ? std::min(o.n_alpha, 26) : b);
 }
 
-// Terms per launch for the choice B: equal parts of at most B (N = 128: see buffer_terms) and 256, in whole pairs.
+// Terms per launch for the choice B: equal parts of at most B (N = 128: see buffer_terms), of what the buffer holds and of
+// 256, in whole pairs.
 int launch_terms(int N, const sigw_opts& o, int B) {
-  const int most = std::min(256, std::max(2, B == max_alpha_batch(o) ? buffer_terms(N, o) : B)) & ~1;
+  const int hold = buffer_terms(N, o);
+  const int most = std::min({256, hold, std::max(2, B == max_alpha_batch(o) ? hold : B)}) & ~1;
   const int launches = (o.n_alpha + most - 1) / most;
   return ((o.n_alpha + launches - 1) / launches + 1) & ~1;
 }
 
-// Process-wide autotuning results: (N, precision, realisations, n_alpha) -> (terms per launch, variant).
+// Process-wide autotuning results: (N, precision, realisations, n_alpha) -> (terms per launch, variant), of plans whose
+// options leave the terms per launch open.
 struct TuneKey {
   int N, prec, batch, n_alpha;
   bool operator<(const TuneKey& o) const {
@@ -1183,7 +1186,7 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
     cudaGraphExecDestroy(p->graph);
     p->graph = nullptr;
   }
-  {
+  if (p->opts.alpha_batch == 0) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune[TuneKey{N, p->opts.precision, p->opts.max_batch, n_alpha}] = {bestB, bestV | bestP3};
   }

@@ -30,6 +30,7 @@ struct State {
   std::vector<std::string> bad;
   SimGraph* capture = nullptr;
   long launches = 0;
+  bool values = true;  // whether what a launch reads is checked, not only where
   void* real = nullptr;
 };
 State* S = new State();
@@ -76,11 +77,11 @@ std::string rd(const char* who, const void* p, size_t n) {  // the one writer of
     t = it->second.second;
     at = it->second.first;
   }
-  if (at < (U)p + n) fault(std::string(who) + ": reads what '" + t + "' did not write all of");
+  if (at < (U)p + n && S->values) fault(std::string(who) + ": reads what '" + t + "' did not write all of");
   return t;
 }
 void want(const char* who, const std::string& got, const std::string& start) {
-  if (got.compare(0, start.size(), start)) fault(std::string(who) + ": reads '" + got + "', not '" + start + "'");
+  if (S->values && got.compare(0, start.size(), start)) fault(std::string(who) + ": reads '" + got + "', not '" + start + "'");
 }
 cudaError_t launch(std::function<void()> f) {
   LOCK;
@@ -297,8 +298,9 @@ cudaError_t OpsRT<T>::p2(int N, const void* Ta, const void* Tb, void* W, int n_a
     const Size<T> z(N);
     const std::string t = rd("P2", Ta, batch * nb * z.f), id = owner(t);
     const std::string terms = " terms " + std::to_string(a0) + "+" + std::to_string(nb);
-    if (t != "Ta" + id + terms) fault("P2 reads '" + t + "' for" + terms);
-    if (rd("P2", Tb, batch * nb * z.f) != "Tb" + id + terms) fault("P2: Tb is not Ta's");
+    if (S->values && t != "Ta" + id + terms) fault("P2 reads '" + t + "' for" + terms);
+    const std::string u = rd("P2", Tb, batch * nb * z.f);
+    if (S->values && u != "Tb" + id + terms) fault("P2: Tb is not Ta's");
     if (a0 % 2 || (nb % 2 && a0 + nb < n_alpha)) fault("P2: a pair is split");
     const size_t np = (n_alpha + 1) / 2, row = 2 * z.f;
     for (int b = 0; b < batch; ++b)
@@ -306,7 +308,7 @@ cudaError_t OpsRT<T>::p2(int N, const void* Ta, const void* Tb, void* W, int n_a
         for (int f = 0; f < 3; ++f)
           if (f != 1 || a + 1 < n_alpha) wr("P2", c(W) + (((size_t)b * np + a / 2) * 3 + f) * row, row, "W" + id);
     rd("P2", Ta, batch * nb * z.f);  // not written over
-    if (rd("P2", Tb, batch * nb * z.f) != "Tb" + id + terms) fault("P2 writes over its input");
+    if (rd("P2", Tb, batch * nb * z.f) != u) fault("P2 writes over its input");
   });
 }
 template <typename T>
@@ -443,6 +445,7 @@ cudaError_t launch_fin(const double* part, long pbs, int maxblk, int ns, const S
 extern "C" {
 int sigw_fft3d_noalloc() { return 3; }  // the plan-free transform is not simulated
 void sim_init(const char* real) { S->real = dlopen(real, RTLD_NOW | RTLD_LOCAL); }
+void sim_check_values(int on) { S->values = on; }  // off: the autotuner times launches on what is there
 long sim_launches() { return S->launches; }
 size_t sim_device_bytes() {
   size_t n = 0;

@@ -47,6 +47,13 @@ def _run(p, batch=1, shells=(1,), **kw):
     p.spectrum(list(shells))
 
 
+def _autotune(sim, p):
+    sim.lib().sim_check_values(0)
+    r = p.autotune()
+    sim.lib().sim_check_values(1)
+    return r
+
+
 # ---- host memory that a queued copy may still read
 
 def test_queued_uploads_keep_their_host_buffers(sim):
@@ -62,3 +69,16 @@ def test_queued_uploads_keep_their_host_buffers(sim):
         p.spectrum_async(None, [1])
         p.synchronize()
         p.spectrum_jackknife([1, 4])
+
+
+# ---- buffers
+
+@pytest.mark.parametrize("alpha_batch", [50, 20])
+def test_terms_tuned_on_another_plan_fit_this_plan(sim, alpha_batch):
+    """A plan with its own (larger) terms per launch is tuned; a default plan of the same size keeps within its buffers."""
+    with sim.Plan(16, 1.0, n_alpha=50, alpha_batch=alpha_batch) as p:
+        _run(p)
+        _autotune(sim, p)
+        _run(p)
+    with sim.Plan(16, 1.0, n_alpha=50) as q:
+        _run(q)
