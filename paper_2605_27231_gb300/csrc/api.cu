@@ -52,11 +52,13 @@ int buffer_terms(int N, const sigw_opts& o) {
   return std::max(2, N == 128 && o.alpha_batch == 0 && b == 16 ? std::min(o.n_alpha, 26) : b);
 }
 
-// Terms per launch for the choice B: equal parts of at most B (N = 128: see buffer_terms), of what the buffer holds and of
-// 256, in whole pairs.
+// Terms per launch for the choice B: at most B (N = 128: see buffer_terms), what the buffer holds and 256.  All terms in one
+// launch, an odd last one among them, or equal parts in whole pairs.
 int launch_terms(int N, const sigw_opts& o, int B) {
   const int hold = buffer_terms(N, o);
-  const int most = std::min({256, hold, std::max(2, B == max_alpha_batch(o) ? hold : B)}) & ~1;
+  int most = std::min({256, hold, std::max(2, B == max_alpha_batch(o) ? hold : B)});
+  if (o.n_alpha <= most) return o.n_alpha;
+  most &= ~1;
   const int launches = (o.n_alpha + most - 1) / most;
   return ((o.n_alpha + launches - 1) / launches + 1) & ~1;
 }

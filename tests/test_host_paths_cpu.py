@@ -71,6 +71,19 @@ def test_queued_uploads_keep_their_host_buffers(sim):
         p.spectrum_jackknife([1, 4])
 
 
+# ---- launches
+
+@pytest.mark.parametrize("N,n_alpha", [(32, 1), (32, 3), (32, 9), (32, 15), (32, 16), (256, 7), (128, 17), (128, 25)])
+def test_terms_that_fit_take_one_launch(sim, N, n_alpha):
+    with sim.Plan(N, 1.0, precision=64 if N == 32 else 32, n_alpha=n_alpha) as p:
+        p.generate(1e-2, 0.5, 10.0)
+        p.profile(False)
+        p.spectrum([1, N // 2])
+        r = p.profile_read()
+    kinds = [k for k in r if isinstance(r[k], dict)]
+    assert [r[k]["launches"] for k in kinds[1:4]] == [4, 4, 4]  # passes of two shells, two kernels
+
+
 # ---- buffers
 
 @pytest.mark.parametrize("alpha_batch", [50, 20])
