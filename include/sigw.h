@@ -244,8 +244,8 @@ sigw_status sigw_server_destroy(sigw_server srv);
  * with alpha_batch = 0 start; then times the forms of the last inverse pass (FP32, N = 128, 256, 512: two radices, and radix 16 with its accumulators
  * in tensor memory) on the terms just produced, and at FP32 N = 64 the fused second and last pass against the three
  * passes.  An untuned FP32 plan starts from 16 terms and the bits measured fastest on GB300 (24 at N = 64, 26 from
- * N = 128 on).  Terms go in equal launches of whole pairs of at most the chosen number; at N = 128 the largest choice, 16,
- * takes up to 26.  Outputs nullable: chosen terms per launch, variant bits (1: alternative radix of the first strided
+ * N = 128 on).  Terms go in equal launches of whole pairs of at most the chosen number (an odd number counts as the
+ * next even one); at N = 128 the largest choice, 16, stands for as many as the plan's memory holds.  Outputs nullable: chosen terms per launch, variant bits (1: alternative radix of the first strided
  * pass, 2: radix-16 last pass, 4: accepted and ignored (the second strided pass has one form), 8: radix-16 last pass with
  * its accumulators in tensor memory, which at N = 64 also takes in the second pass and runs all terms in one launch
  * whatever the terms per launch, 16: first pass with its tile in tensor memory) and the time in ms of the chosen strided

@@ -44,25 +44,6 @@ int max_alpha_batch(const sigw_opts& o) {
   return std::min(o.n_alpha, 16);
 }
 
-// Terms the first-pass output buffer holds (at least the pair that the second pass works on).  At N = 128 the largest
-// choice, 16, stands for 26: a launch of 16 terms of one realisation leaves the last of its few waves short (first pass,
-// 50 terms: 253 us in launches of 16, 215 us in two of 25; second pass 325 and 313 us).
-int buffer_terms(int N, const sigw_opts& o) {
-  const int b = max_alpha_batch(o);
-  return std::max(2, N == 128 && o.alpha_batch == 0 && b == 16 ? std::min(o.n_alpha, 26) : b);
-}
-
-// Terms per launch for the choice B: at most B (N = 128: see buffer_terms), what the buffer holds and 256.  All terms in one
-// launch, an odd last one among them, or equal parts in whole pairs.
-int launch_terms(int N, const sigw_opts& o, int B) {
-  const int hold = buffer_terms(N, o);
-  int most = std::min({256, hold, std::max(2, B == max_alpha_batch(o) ? hold : B)});
-  if (o.n_alpha <= most) return o.n_alpha;
-  most &= ~1;
-  const int launches = (o.n_alpha + most - 1) / most;
-  return ((o.n_alpha + launches - 1) / launches + 1) & ~1;
-}
-
 // Process-wide autotuning results: (N, precision, realisations, n_alpha) -> (terms per launch, variant), of plans whose
 // options leave the terms per launch open.
 struct TuneKey {
@@ -74,20 +55,87 @@ struct TuneKey {
 std::mutex g_tune_mu;
 std::map<TuneKey, std::pair<int, int>> g_tune;
 
-// Kernels (I_s, I_c) of a shell whose forward passes, shell sums and jackknife share their launches.  Up to N = 128 these
-// are short (8 to 17 us each at 64^3 and 128^3, mostly latency), and the second kernel's run beside the first's.
-int kernels_at_once(int N) { return N <= 128 ? 2 : 1; }
-
 // Parameters of one realisation in d_gen / h_gen.
 constexpr size_t kGenBytes = sizeof(sigw::MapArgs) + sizeof(sigw::PzArgs) + sizeof(uint64_t);
 
-// Sizes (bytes) of every device buffer of a plan.
-struct Sizes {
-  size_t phi, T, W, synth, F, F2, partial, out, lut, tab, tw, amp, rows_sq;
-  int maxblk;
-  size_t total() const {
-    return phi + T + std::max(W, synth) + F + F2 + partial + out + lut + tab + tw + amp + rows_sq + 4096;
+// ---- the block of device memory that the hot loop passes from launch to launch
+//
+// Bytes per realisation; a field f is a packed half spectrum.  The block is the sum of what one kernel's stages need side by
+// side with one group of term pairs: T (first-pass output, two fields for each term of a launch), W (three fields a term, or
+// the scratch of the synthesis and the jackknife), F and F2 (six pruned half spectra each, at most g).  What is alive at a
+// time is placed in it, so that more groups, larger launches and shared forward passes need no more memory:
+//   bottom  W; in the fused form T of all terms of one kernel.  After the last pass F2, and above it the jackknife's scratch.
+//   end     F: `groups` partial fields, in each of them nm kernels one behind the other.
+//   T       ends at the end of the block or, for the second kernel of nm = 2, where F of the first begins.  With one
+//           realisation it may lie over rows of W that only later launches write.
+struct Layout {
+  size_t f, g, jack, block;
+  bool fused;  // second and last pass in one kernel
+  int nm;      // kernels (I_s, I_c) of a shell that share the forward passes, shell sums and jackknife
+  int groups;  // of term pairs in the last pass
+  size_t rows;  // W, or T of the fused form
+  size_t t_end(bool second) const { return block - (second ? (nm * groups - 1) * g : 0); }
+};
+
+#define OPS_OF(prec, fn, ...) \
+  ((prec) == 64 ? sigw::OpsRT<double>::fn(__VA_ARGS__) : sigw::OpsRT<float>::fn(__VA_ARGS__))
+
+// Up to N = 128 the passes after the product are short (8 to 17 us each at 64^3 and 128^3, mostly latency) and those of the
+// second kernel run beside the first's (nm = 2); more groups of term pairs come first (32^3: seven groups, nm = 1).
+Layout layout_of(int N, const sigw_opts& o, int variant) {
+  Layout l;
+  const size_t H = N / 2, NN = (size_t)N * N, cel = o.precision == 64 ? 16 : 8, h = NN * (H + 1) * cel;
+  const size_t b = max_alpha_batch(o), n = o.n_alpha;
+  l.f = NN * H * cel;
+  l.g = 6 * h;
+  l.jack = 2 * (h + 2 * l.f);  // two standard and two packed half spectra, two real fields
+  l.block = 2 * b * l.f + std::max(3 * n * l.f, l.jack) + 2 * l.g;
+  l.fused = OPS_OF(o.precision, fused, N, variant);
+  l.rows = (l.fused ? 2 * n : 6 * ((n + 1) / 2)) * l.f;
+  const size_t t = l.fused ? 0 : 2 * l.f * std::min(n, (b + 1) & ~(size_t)1);
+  for (l.groups = OPS_OF(o.precision, last_groups, N, variant, o.n_alpha); l.groups >= 1; --l.groups)
+    for (l.nm = N <= 128 ? 2 : 1; l.nm >= 1; --l.nm) {
+      const size_t F = l.nm * l.groups * l.g;
+      if (l.rows + F <= l.block && l.nm * l.g + F <= l.block && l.nm * (l.g + l.jack) <= l.block &&
+          l.rows + t <= l.t_end(l.nm == 2))
+        return l;
+    }
+  l.groups = l.nm = 1;  // not reached: one group and one kernel are what the block is the sum of
+  return l;
+}
+
+struct Terms {
+  int a0, nb;
+};
+
+// The launches of the first and second pass for the choice `most` of terms per launch: equal parts in whole pairs (an odd
+// choice counts as the next even one), an odd last term in the last of them; at most 256 terms, and what T has room for.
+// At N = 128 the largest choice, 16, stands for as many as fit: a launch of 16 terms of one realisation leaves the last of
+// its few waves short (first pass, 50 terms: 253 us in launches of 16, 215 us in two).
+std::vector<Terms> launches_of(int N, const sigw_opts& o, const Layout& l, int most, int batch, bool second) {
+  const int n = o.n_alpha;
+  auto room = [&](int e) {  // terms of a launch that ends with term e
+    return (int)((l.t_end(second) - (batch == 1 ? (size_t)(6 * ((e + 1) / 2)) * l.f : l.rows)) / (2 * l.f));
+  };
+  const bool fit = N == 128 && o.alpha_batch == 0 && most == 16;
+  int part = fit ? (batch == 1 ? 256 : std::min(256, room(n) & ~1)) : std::min(256, (most + 1) & ~1);
+  const int parts = (n + part - 1) / part;
+  part = std::min(part, ((n + parts - 1) / parts + 1) & ~1);
+  std::vector<Terms> out;
+  for (int e = n; e > 0;) {  // from the last launch back: it has the least room
+    int nb = std::min({e, part, room(e)});
+    nb -= (e - nb) & 1;
+    out.insert(out.begin(), {e - nb, nb});
+    e -= nb;
   }
+  return out;
+}
+
+// Sizes (bytes) of the device memory of a plan.
+struct Sizes {
+  size_t phi, block, partial, out, lut, tab, tw, amp, rows_sq;
+  int maxblk;
+  size_t total() const { return phi + block + partial + out + lut + tab + tw + amp + rows_sq + 2048; }
 };
 
 Sizes sizes_of(int N, const sigw_opts& o) {
@@ -95,33 +143,17 @@ Sizes sizes_of(int N, const sigw_opts& o) {
   const size_t H = N / 2, NH = H + 1, NN = (size_t)N * N;
   const size_t rel = o.precision == 64 ? 8 : 4, cel = 2 * rel;
   const size_t mb = (size_t)o.max_batch;
-  const int B = buffer_terms(N, o);
-  sigw::LaunchShape sh = o.precision == 64 ? sigw::OpsRT<double>::shape(N) : sigw::OpsRT<float>::shape(N);
-  s.maxblk = sh.maxblk_f3;
+  s.maxblk = OPS_OF(o.precision, shape, N).maxblk_f3;
   s.phi = mb * NN * NH * cel;
-  s.T = 2 * mb * (size_t)B * NN * H * cel;
-  s.W = mb * 6 * (size_t)((o.n_alpha + 1) / 2) * NN * H * cel;  // three full rows per term pair
-  if (o.precision == 32 && N == 64)  // or the first pass's output of both kernels (fused second and last pass)
-    s.W = std::max(s.W, mb * 4 * (size_t)o.n_alpha * NN * H * cel);
-  // the jackknife reuses W after each shell: two standard + two packed half spectra + two real fields
-  s.W = std::max(s.W, kernels_at_once(N) * mb * 2 * (NN * NH * cel + NN * H * cel + NN * (size_t)N * rel) + 1024);
-  s.synth = mb * (NN * H * cel + NN * NH * cel + 3 * NN * (size_t)N * rel) + 1024;  // + two real fields (non-local map)
-  size_t parts = 1;  // partial fields of the last pass
-  for (int v : {0, 8})
-    parts = std::max(parts, (size_t)(o.precision == 64 ? sigw::OpsRT<double>::last_groups(N, v, o.n_alpha)
-                                                       : sigw::OpsRT<float>::last_groups(N, v, o.n_alpha)));
-  const size_t nm = kernels_at_once(N);
-  s.F = parts * nm * mb * 6 * NN * NH * cel;
-  s.F2 = nm * mb * 6 * NN * NH * cel;
+  s.block = mb * layout_of(N, o, 0).block;
   s.partial = mb * H * 2 * (size_t)s.maxblk * sizeof(double);
   s.out = mb * H * 4 * sizeof(double) + H * sizeof(double);
   const size_t msq = 3 * H * H + 1;
   s.lut = H * msq * sizeof(int16_t);
   s.tab = 2 * ((size_t)o.n_alpha * (o.n_modes + 1) + o.n_alpha) * rel;
   s.tw = (size_t)N * cel;
-  s.amp = mb * msq * rel + mb * (sizeof(sigw::MapArgs) + sizeof(sigw::PzArgs));
-  const int rb = o.precision == 64 ? sigw::OpsRT<double>::rows_blocks(N) : sigw::OpsRT<float>::rows_blocks(N);
-  s.rows_sq = mb * ((size_t)rb * sizeof(double) + 2 * sizeof(double) + 2 * sizeof(uint64_t));
+  s.amp = mb * msq * rel + mb * kGenBytes;
+  s.rows_sq = mb * ((size_t)OPS_OF(o.precision, rows_blocks, N) * sizeof(double) + 2 * sizeof(double));
   return s;
 }
 
@@ -150,10 +182,7 @@ struct sigw_plan_s {
   // device buffers
   std::vector<void*> allocs;
   void* d_phi = nullptr;
-  void* d_T = nullptr;     // first-pass output (two fields per term of an alpha batch)
-  void* d_work = nullptr;  // W during the hot loop, synthesis scratch during sigw_generate / sigw_fft3d
-  void* d_F = nullptr;
-  void* d_F2 = nullptr;
+  void* d_work = nullptr;  // the hot loop's block (see Layout); scratch of the synthesis and of sigw_fft3d
   double* d_partial = nullptr;
   void* d_res = nullptr;  // the error flag (16 bytes), then d_out: read back in one copy
   double* d_out = nullptr;
@@ -331,8 +360,7 @@ std::vector<double> count_shell_modes(int N) {
   return nk;
 }
 
-#define OPS(plan, fn, ...) \
-  ((plan)->opts.precision == 64 ? sigw::OpsRT<double>::fn(__VA_ARGS__) : sigw::OpsRT<float>::fn(__VA_ARGS__))
+#define OPS(plan, fn, ...) OPS_OF((plan)->opts.precision, fn, __VA_ARGS__)
 
 }  // namespace
 
@@ -498,10 +526,7 @@ sigw_status sigw_plan_create(int N, double L, const sigw_opts* opts, void* cuda_
     ptr = reinterpret_cast<decltype(ptr)>(_q);              \
   } while (0)
   ALLOC(p->d_phi, p->sz.phi);
-  ALLOC(p->d_T, p->sz.T);
-  ALLOC(p->d_work, std::max(p->sz.W, p->sz.synth));
-  ALLOC(p->d_F, p->sz.F);
-  ALLOC(p->d_F2, p->sz.F2);
+  ALLOC(p->d_work, p->sz.block);
   ALLOC(p->d_partial, p->sz.partial);
   ALLOC(p->d_res, 16 + mb * H * 4 * sizeof(double));
   p->d_err = (int*)p->d_res;
@@ -730,16 +755,27 @@ sigw_status sigw_generate(sigw_plan p, const sigw_pzeta* pz, const sigw_ngmap* m
   return sigw_generate_batch(p, pzs.data(), ms.data(), seeds, batch, usr_hits);
 }
 
-// Jackknife scratch of one spectrum call (Sec. sec_envelope_obs): M^3 sub-volumes; per (shell, kernel), or per shell where
-// kernels_at_once is 2, the TT amplitudes go to Xj (standard half spectra, 2 per kernel and realisation), are packed into Yj, inverse-transformed into
-// the real fields Rj, and reduced per sub-volume x0-plane into part[(si * 2 + m)][2 batch][M^3][N/M].
+// Jackknife of one spectrum call (Sec. sec_envelope_obs): M^3 sub-volumes.  Per launch of the last forward pass the TT
+// amplitudes go to standard half spectra (2 per kernel and realisation), are packed, inverse-transformed into real fields,
+// and reduced per sub-volume x0-plane into part[(si * 2 + m)][2 batch][M^3][N/M].
 struct Jackknife {
   int M = 4;
   double* part = nullptr;
-  void* Xj = nullptr;
-  void* Yj = nullptr;
-  void* Rj = nullptr;
 };
+
+// First and second pass of one launch of terms into W (kernel m; T placed as Layout says).
+static sigw_status enqueue_terms(sigw_plan p, const Layout& lay, const Terms& t, bool second, int m, const int16_t* lut,
+                                 int batch, int var) {
+  const int N = p->N, n_alpha = p->opts.n_alpha, nm1 = p->opts.n_modes + 1;
+  const double fieldb = (double)batch * lay.f, phib = (double)batch * lay.g / 6;
+  char* Ta = (char*)p->d_work + batch * (lay.t_end(second) - 2 * t.nb * lay.f);
+  char* Tb = Ta + (size_t)batch * t.nb * lay.f;
+  RUN(p, 1, phib + 2.0 * t.nb * fieldb, "P1",
+      OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[m], nm1, t.a0, t.nb, batch, p->d_tw, var, p->st));
+  RUN(p, 2, 5.0 * t.nb * fieldb, "P2",
+      OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, t.a0, t.nb, batch, p->d_tw, p->d_err, p->wait_limit, p->st));
+  return SIGW_OK;
+}
 
 // Queue the hot loop for the shells sh writing [batch][ns][4] to out.
 static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, double* out, const Jackknife* jk = nullptr) {
@@ -751,14 +787,12 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, dou
   const size_t NN = (size_t)N * N;
   const size_t cel = p->celem();
   const int var = p->variant;
-  // the fused second and last pass takes the first pass's output of all terms of both kernels, kept in W's place
-  const bool fused = OPS(p, fused, N, var);
-  const int B = launch_terms(N, p->opts, p->B);
-  void* Ta = fused ? p->d_work : p->d_T;
-  void* Tb = (char*)Ta + (size_t)batch * (fused ? 2 * n_alpha : B) * NN * H * cel;
-  const int groups = OPS(p, last_groups, N, var, n_alpha);
+  const Layout lay = layout_of(N, p->opts, var);
+  const int nm = lay.nm, groups = lay.groups;
+  char* const work = (char*)p->d_work;
+  char* const end = work + batch * lay.block;
   const long pbs = (long)ns * 2 * p->sz.maxblk;
-  const double fieldb = (double)batch * NN * H * cel;  // one packed complex field per realisation batch
+  const double fieldb = (double)batch * lay.f;  // one packed complex field per realisation batch
   const double phib = (double)batch * NN * (H + 1) * cel;
   for (int si = 0; si < ns; ++si) {
     const int n_c = sh[si];
@@ -769,47 +803,49 @@ static sigw_status enqueue_spectrum(sigw_plan p, const std::vector<int>& sh, dou
     long disk = 0;
     for (int n1 = n1lo; n1 < n1lo + nk1; ++n1)
       for (int n2 = 0; n2 <= n_c; ++n2) disk += (n1 * n1 + n2 * n2 <= n_c * n_c + n_c);
-    const int nm = kernels_at_once(N);  // kernels per launch of the passes after the product
     const long fvals = 6L * batch * (long)NN * ncp, fgs = fvals * nm;  // values of one kernel's F; between groups
-    for (int m = 0; m < 2; ++m) {
-      void* F = (char*)p->d_F + (size_t)(m % nm) * fvals * cel;
-      if (fused && m == 0) {  // both kernels
-        RUN(p, 1, phib + 4.0 * n_alpha * fieldb, "P1",
-            OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, 2, (long)n_alpha * nm1, 0, n_alpha, batch, p->d_tw,
-                var, st));
-        RUN(p, 3, 4.0 * n_alpha * fieldb + (double)groups * fgs * cel, "P23",
-            OPS(p, p23, N, Ta, Tb, p->d_sigma[0], n_alpha, F, groups, fgs, n_c, batch, p->d_tw, p->d_err, p->wait_limit,
-                st));
-      }
-      for (int a0 = 0; a0 < n_alpha && !fused; a0 += B) {
-        const int nb = std::min(B, n_alpha - a0);
-        RUN(p, 1, phib + 2.0 * nb * fieldb, "P1",
-            OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[m], nm1, 1, 0L, a0, nb, batch, p->d_tw, var, st));
-        RUN(p, 2, 5.0 * nb * fieldb, "P2",
-            OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, p->d_err, p->wait_limit, st));
-      }
-      if (!fused)
+    char* const F0 = end - groups * fgs * cel;
+    for (int i = 0; i < 2; ++i) {
+      const int m = nm == 2 ? 1 - i : i;  // the kernel whose F lies at the very end goes first
+      const bool second = nm == 2 && i == 1;
+      char* const F = F0 + (nm == 2 ? m * fvals * cel : 0);
+      if (lay.fused) {
+        char* const Tb = work + (size_t)batch * n_alpha * lay.f;
+        RUN(p, 1, phib + 2.0 * n_alpha * fieldb, "P1",
+            OPS(p, p1, N, p->d_phi, work, Tb, lut, p->d_phitab[m], nm1, 0, n_alpha, batch, p->d_tw, var, st));
+        RUN(p, 3, 2.0 * n_alpha * fieldb + (double)groups * fvals * cel, "P23",
+            OPS(p, p23, N, work, Tb, p->d_sigma[m], n_alpha, F, groups, fgs, n_c, batch, p->d_tw, p->d_err,
+                p->wait_limit, st));
+      } else {
+        for (const Terms& t : launches_of(N, p->opts, lay, p->B, batch, second)) {
+          const sigw_status s = enqueue_terms(p, lay, t, second, m, lut, batch, var);
+          if (s != SIGW_OK) return s;
+        }
         RUN(p, 3, 3.0 * n_alpha * fieldb + (double)groups * fvals * cel, "P3",
-            OPS(p, p3, N, p->d_work, p->d_sigma[m], n_alpha, F, groups, fgs, n_c, batch, p->d_tw, p->d_err,
-                p->wait_limit, var, st));
-      if (m % nm != nm - 1) continue;  // the forward passes take both kernels
-      const int nf = nm * batch;       // realisations times kernels
+            OPS(p, p3, N, work, p->d_sigma[m], n_alpha, F, groups, fgs, n_c, batch, p->d_tw, p->d_err, p->wait_limit,
+                var, st));
+      }
+      if (nm == 2 && i == 0) continue;  // the forward passes take both kernels
+      const int nf = nm * batch;        // realisations times kernels
+      const int m0 = nm == 2 ? 0 : m;
       RUN(p, 4, (double)nm * (groups * (double)fvals + 6.0 * batch * N * nk1 * ncp) * cel, "F2",
-          OPS(p, f2, N, p->d_F, groups, fgs, p->d_F2, n_c, nf, p->d_tw, st));
-      double* part = p->d_partial + ((long)si * 2 + m + 1 - nm) * p->sz.maxblk;
-      if (jk) CKP(p, cudaMemsetAsync(jk->Xj, 0, (size_t)2 * nf * NN * (H + 1) * cel, st), "jackknife zero");
+          OPS(p, f2, N, F0, groups, fgs, work, n_c, nf, p->d_tw, st));
+      char* const Xj = work + nf * lay.g;
+      if (jk) CKP(p, cudaMemsetAsync(Xj, 0, (size_t)2 * nf * NN * (H + 1) * cel, st), "jackknife zero");
       RUN(p, 5, 6.0 * nf * (double)N * disk * cel, jk ? "F3 + amplitudes" : "F3",
-          OPS(p, f3, N, p->d_F2, n_c, part, pbs, (long)p->sz.maxblk, nm, batch, p->d_tw, st, jk ? jk->Xj : nullptr));
+          OPS(p, f3, N, work, n_c, p->d_partial + ((long)si * 2 + m0) * p->sz.maxblk, pbs, (long)p->sz.maxblk, nm, batch,
+              p->d_tw, st, jk ? Xj : nullptr));
       if (jk) {
         const double xjb = 2.0 * nf * NN * (H + 1) * cel, yjb = 2.0 * nf * NN * H * cel;
         const double rjb = 2.0 * nf * NN * N * p->relem();
-        RUN(p, 0, xjb + yjb, "jackknife inverse axis 0", OPS(p, pass_pack, N, jk->Xj, jk->Yj, 2 * nf, p->d_tw, st));
-        RUN(p, 0, 2 * yjb, "jackknife inverse axis 1", OPS(p, pass, N, jk->Yj, 1, +1, 2 * nf, p->d_tw, st));
-        RUN(p, 0, yjb + rjb, "jackknife rows C2R",
-            OPS(p, rows_c2r, N, jk->Yj, jk->Rj, 2 * nf, 1.0, nullptr, p->d_tw, st));
+        char* const Yj = Xj + (size_t)2 * nf * NN * (H + 1) * cel;
+        char* const Rj = Yj + 2 * nf * lay.f;
+        RUN(p, 0, xjb + yjb, "jackknife inverse axis 0", OPS(p, pass_pack, N, Xj, Yj, 2 * nf, p->d_tw, st));
+        RUN(p, 0, 2 * yjb, "jackknife inverse axis 1", OPS(p, pass, N, Yj, 1, +1, 2 * nf, p->d_tw, st));
+        RUN(p, 0, yjb + rjb, "jackknife rows C2R", OPS(p, rows_c2r, N, Yj, Rj, 2 * nf, 1.0, nullptr, p->d_tw, st));
         const long per = 2L * batch * jk->M * jk->M * jk->M * (N / jk->M);
         RUN(p, 0, rjb, "jackknife sub-volumes",
-            OPS(p, subvol, N, jk->M, jk->Rj, 2 * nf, jk->part + ((long)si * 2 + m + 1 - nm) * per, st));
+            OPS(p, subvol, N, jk->M, Rj, 2 * nf, jk->part + ((long)si * 2 + m0) * per, st));
       }
     }
   }
@@ -930,10 +966,6 @@ sigw_status sigw_spectrum_jackknife(sigw_plan p, const int* shells, int n_shells
   const size_t per = (size_t)2 * batch * M3 * sv;  // partials per (shell, kernel)
   Jackknife jk;
   jk.M = M;
-  jk.Xj = p->d_work;
-  const size_t nf = (size_t)kernels_at_once(N) * batch;
-  jk.Yj = (char*)jk.Xj + 2 * nf * NN * (H + 1) * cel;
-  jk.Rj = (char*)jk.Yj + 2 * nf * NN * H * cel;
   {
     void* q = nullptr;
     sigw_status s = dev_alloc(p, &q, sizeof(double) * per * 2 * ns);
@@ -1075,20 +1107,26 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
   const int cands[] = {4, 5, 8, 10, 16};
   sigw_status status = SIGW_OK;
   // For each terms-per-launch candidate the two strided passes are timed separately, the first in each of its forms.
+  char* const work = (char*)p->d_work;
+  auto strided = [&](int which, const std::vector<Terms>& ts, const Layout& lay, int v) -> cudaError_t {  // 0, 1; 2: both
+    for (const Terms& t : ts) {
+      char* const Ta = work + batch * (lay.t_end(lay.nm == 2) - 2 * t.nb * lay.f);
+      char* const Tb = Ta + (size_t)batch * t.nb * lay.f;
+      cudaError_t e = cudaSuccess;
+      if (which != 1) e = OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, t.a0, t.nb, batch, p->d_tw, v, st);
+      if (which != 0 && e == cudaSuccess)
+        e = OPS(p, p2, N, Ta, Tb, work, n_alpha, t.a0, t.nb, batch, p->d_tw, p->d_err, sigw::kDefaultWaitLimit, st);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  };
+  const Layout lay0 = layout_of(N, p->opts, 0);
   auto time_pass = [&](int which, int choice, int v, float* ms) -> sigw_status {
-    const int B = launch_terms(N, p->opts, choice);
-    void* Ta = p->d_T;
-    void* Tb = (char*)p->d_T + (size_t)batch * B * NN * H * cel;
+    const std::vector<Terms> ts = launches_of(N, p->opts, lay0, choice, batch, lay0.nm == 2);
     for (int rep = 0; rep < 2; ++rep) {  // first pass warms the variant; the second is timed
       cudaEventRecord(e0, st);
-      for (int a0 = 0; a0 < n_alpha; a0 += B) {
-        const int nb = std::min(B, n_alpha - a0);
-        cudaError_t e = which == 0
-                            ? OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, 1, 0L, a0, nb, batch, p->d_tw, v, st)
-                            : OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, p->d_err,
-                                  sigw::kDefaultWaitLimit, st);
-        if (e != cudaSuccess) return cuda_fail(p, e, "autotune launch");
-      }
+      const cudaError_t e = strided(which, ts, lay0, v);
+      if (e != cudaSuccess) return cuda_fail(p, e, "autotune launch");
       cudaEventRecord(e1, st);
       if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(ms, e0, e1) != cudaSuccess)
         return cuda_fail(p, cudaGetLastError(), "autotune timing");
@@ -1122,18 +1160,8 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
   int bestP3 = 0;
   const bool has_fused = OPS(p, fused, N, 8);
   if (status == SIGW_OK && (OPS(p, p3_variants, N) > 1 || has_fused)) {
-    {
-      const int B = launch_terms(N, p->opts, bestB);
-      void* Ta = p->d_T;
-      void* Tb = (char*)p->d_T + (size_t)batch * B * NN * H * cel;
-      for (int a0 = 0; a0 < n_alpha && status == SIGW_OK; a0 += B) {
-        const int nb = std::min(B, n_alpha - a0);
-        cudaError_t e = OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, 1, 0L, a0, nb, batch, p->d_tw, bestV, st);
-        if (e == cudaSuccess)
-          e = OPS(p, p2, N, Ta, Tb, p->d_work, n_alpha, a0, nb, batch, p->d_tw, p->d_err, sigw::kDefaultWaitLimit, st);
-        if (e != cudaSuccess) status = cuda_fail(p, e, "autotune launch");
-      }
-    }
+    const cudaError_t e = strided(2, launches_of(N, p->opts, lay0, bestB, batch, lay0.nm == 2), lay0, bestV);
+    if (e != cudaSuccess) status = cuda_fail(p, e, "autotune launch");
     auto time_last = [&](float* ms, auto&& launch) {  // second of two runs
       for (int rep = 0; rep < 2 && status == SIGW_OK; ++rep) {
         cudaEventRecord(e0, st);
@@ -1144,15 +1172,17 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
           status = cuda_fail(p, e != cudaSuccess ? e : cudaGetLastError(), "autotune last pass");
       }
     };
-    const long fgs = 6L * batch * (long)NN * (n_c + 1) * kernels_at_once(N);
+    const long fvals = 6L * batch * (long)NN * (n_c + 1);  // of one kernel's F
     const int np3 = OPS(p, p3_variants, N);  // 2: radix 8 / 16; 3: also radix 16 with TMEM accumulators
     const int p3bits[3] = {0, 2, 8};
     float t3[3] = {1e30f, 1e30f, 1e30f};
     for (int v3 = 0; v3 < np3; ++v3) {
-      const int bits = p3bits[v3], groups = OPS(p, last_groups, N, bits, n_alpha);
+      const int bits = p3bits[v3];
+      const Layout lay = layout_of(N, p->opts, bits);
+      const long fgs = fvals * lay.nm;
       time_last(&t3[v3], [&]() {
-        return OPS(p, p3, N, p->d_work, p->d_sigma[0], n_alpha, p->d_F, groups, fgs, n_c, batch, p->d_tw, p->d_err,
-                   sigw::kDefaultWaitLimit, bits, st);
+        return OPS(p, p3, N, work, p->d_sigma[0], n_alpha, work + batch * lay.block - lay.groups * fgs * cel, lay.groups, fgs,
+                   n_c, batch, p->d_tw, p->d_err, sigw::kDefaultWaitLimit, bits, st);
       });
     }
     int bv = 0;
@@ -1162,17 +1192,16 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
     best += t3[bv];
     if (has_fused) {
       float tf = 1e30f;
-      void* Ta = p->d_work;
-      void* Tb = (char*)p->d_work + (size_t)batch * 2 * n_alpha * NN * H * cel;
+      const Layout lay = layout_of(N, p->opts, 8);
+      const long fgs = fvals * lay.nm;
+      char* const Tb = work + (size_t)batch * n_alpha * lay.f;
       time_last(&tf, [&]() {
-        cudaError_t e = OPS(p, p1, N, p->d_phi, Ta, Tb, lut, p->d_phitab[0], nm1, 2, (long)n_alpha * nm1, 0,
-                            n_alpha, batch, p->d_tw, bestV | 8, st);
+        cudaError_t e = OPS(p, p1, N, p->d_phi, work, Tb, lut, p->d_phitab[0], nm1, 0, n_alpha, batch, p->d_tw, bestV | 8, st);
         if (e == cudaSuccess)
-          e = OPS(p, p23, N, Ta, Tb, p->d_sigma[0], n_alpha, p->d_F, OPS(p, last_groups, N, 8, n_alpha), fgs, n_c, batch,
-                  p->d_tw, p->d_err, sigw::kDefaultWaitLimit, st);
+          e = OPS(p, p23, N, work, Tb, p->d_sigma[0], n_alpha, work + batch * lay.block - lay.groups * fgs * cel, lay.groups,
+                  fgs, n_c, batch, p->d_tw, p->d_err, sigw::kDefaultWaitLimit, st);
         return e;
       });
-      tf *= 0.5f;  // it does both kernels
       if (status == SIGW_OK && tf < best) {
         best = tf;
         bestP3 = 8;

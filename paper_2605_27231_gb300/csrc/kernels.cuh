@@ -376,14 +376,13 @@ __global__ void k_reduce_mean(const double* __restrict__ part, int nblk, double*
 // P1: first inverse pass along axis 0 for a tile of TC packed columns at fixed k1.
 //   V_a(n) = phi_a(cell(|n|^2)) Phi~(n)          (column 0: V(k2=0) + i V(k2=H), each with its own cell)
 //   Ta_a = IDFT_0[V_a],  Tb_a = IDFT_0[i n0^D V_a]
-// The nb terms of a launch are split over nag CTAs per tile (blockIdx.z = (m * batch + b) * nag + group), see p1_groups;
-// kernel m's filter table is m * mtab further and its output follows that of the one before.  With
+// The nb terms of a launch are split over nag CTAs per tile (blockIdx.z = b * nag + group), see p1_groups.  With
 // swz = 8 the column index is stored as cc ^ (8 (k1 mod 2)) (the fused second and last pass reads it that way).
 template <typename T, int N, int E_ = Shape<T, N>::ES, int TC_ = Shape<T, N>::TC>
 __global__ void __launch_bounds__(256) k_p1(const cx<T>* __restrict__ phi, cx<T>* __restrict__ Ta,
                                             cx<T>* __restrict__ Tb, const int16_t* __restrict__ lut,
                                             const T* __restrict__ phitab, int nm1, int alpha0, int nb, int nag,
-                                            int swz, int batch, long mtab, const cx<T>* __restrict__ tw) {
+                                            int swz, const cx<T>* __restrict__ tw) {
   constexpr int E = E_, P = N / E_, TC = TC_, H = N / 2, NH = H + 1;
   using Lay = StridedLay<T, N, TC, E>;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -394,12 +393,11 @@ __global__ void __launch_bounds__(256) k_p1(const cx<T>* __restrict__ phi, cx<T>
   const Lay L{reinterpret_cast<cx<T>*>(smraw), c};
   const int cc = blockIdx.x * TC + c;
   const int k1 = blockIdx.y;
-  const int b = blockIdx.z / nag, ag = blockIdx.z % nag;  // b = m * batch + realisation
+  const int b = blockIdx.z / nag, ag = blockIdx.z % nag;
   const int alo = (int)((long)nb * ag / nag), ahi = (int)((long)nb * (ag + 1) / nag);  // terms of this CTA
-  phitab += (b / batch) * mtab;
   const int n1 = wrapn(k1, N);
   for (int i = threadIdx.x; i < (ahi - alo) * nm1; i += blockDim.x) sm_tab[i] = phitab[(long)(alpha0 + alo) * nm1 + i];
-  const cx<T>* pb = phi + ((long)(b % batch) * N * N + k1) * NH;  // + k0 * N * NH + k2
+  const cx<T>* pb = phi + ((long)b * N * N + k1) * NH;  // + k0 * N * NH + k2
   if (blockIdx.x == 0) {
     for (int k0 = threadIdx.x; k0 < N; k0 += blockDim.x) {
       const int n0 = wrapn(k0, N);
@@ -1446,8 +1444,8 @@ struct P1ACfg {
 template <int N>
 __global__ void __launch_bounds__(P1ACfg<N>::THREADS, P1ACfg<N>::CTAS) k_p1_ab(
     const float2* __restrict__ phi, float2* __restrict__ Ta, float2* __restrict__ Tb, const int16_t* __restrict__ lut,
-    const float* __restrict__ phitab, int nm1, int alpha0, int nb, int nag, int swz, int batch,
-    long mtab, const float2* __restrict__ tw) {
+    const float* __restrict__ phitab, int nm1, int alpha0, int nb, int nag, int swz,
+    const float2* __restrict__ tw) {
   using CF = P1ACfg<N>;
   constexpr int E = CF::E, P = CF::P, TC = CF::TC, H = CF::H, NH = H + 1, RL = CF::RL, NB = CF::NB;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1457,8 +1455,7 @@ __global__ void __launch_bounds__(P1ACfg<N>::THREADS, P1ACfg<N>::CTAS) k_p1_ab(
   float2* const sm_nyq = rn + CF::ROOTS;                          // N values (column 0 only)
   int* const sm_cn = reinterpret_cast<int*>(sm_nyq + N);          // N cells
   float* const sm_tab = reinterpret_cast<float*>(sm_cn + N);      // (terms of this CTA) * nm1
-  const int b = blockIdx.z / nag, ag = blockIdx.z % nag;  // b = m * batch + realisation, as in k_p1
-  phitab += (b / batch) * mtab;
+  const int b = blockIdx.z / nag, ag = blockIdx.z % nag;
   const int alo = (int)((long)nb * ag / nag), ahi = (int)((long)nb * (ag + 1) / nag);  // terms of this CTA
   uint32_t* const tslot = reinterpret_cast<uint32_t*>(sm_tab + (ahi - alo) * nm1);
   const int c = threadIdx.x % TC, j = threadIdx.x / TC;
@@ -1475,7 +1472,7 @@ __global__ void __launch_bounds__(P1ACfg<N>::THREADS, P1ACfg<N>::CTAS) k_p1_ab(
     rw[i] = make_float4(w.x, w.x, -w.y, -w.y);
     rn[i] = make_float2(w.y, w.y);
   }
-  const float2* pb = phi + ((long)(b % batch) * N * N + k1) * NH;  // + k0 * N * NH + k2
+  const float2* pb = phi + ((long)b * N * N + k1) * NH;  // + k0 * N * NH + k2
   if (blockIdx.x == 0) {
     for (int k0 = threadIdx.x; k0 < N; k0 += CF::THREADS) {
       const int n0 = wrapn(k0, N);
@@ -1740,9 +1737,10 @@ __global__ void __launch_bounds__(P1TCfg<N>::THREADS, 3) k_p1_tm(const float2* _
 //     8 rows, and the exchange of the row transform (radix 16 then 4) is in place.
 // Bounded waits, error flag and the drain before exit as in k_p3.
 // What bounds it: the shared-memory path (ncu: 277 wavefronts a warp and transform, 62 % of the path's cycles while
-// active) with 16 warps a SM, issue 50 %; DRAM 17 %.  Both kernels of a shell run in one launch, each with two groups of
-// term pairs: 256 CTAs for one realisation, two a SM.  50 terms of both kernels of one realisation take 146 us (with four
-// groups and a launch per kernel 161; k_p2 and k_p3 before 432), of eight 915 us (976; 2044).  The same split at N = 128
+// active) with 16 warps a SM, issue 50 %; DRAM 17 %.  Four groups of term pairs: 256 CTAs for one realisation, two a SM.
+// 50 terms of both kernels of one realisation take 161 us (k_p2 and k_p3 before 432), of eight 976 us (2044).  Both kernels
+// in one launch with two groups each took 146 and 915 us, but T of both, 4 fields a term, is more than the plan's other
+// forms need (+38 % device memory).  The same split at N = 128
 // (two residue classes of a1 per plane) was slower than the two passes there (715 against 690 us then, 545 now): its
 // shared-memory traffic grows while HBM already carries the passes.
 template <int N>
@@ -1777,7 +1775,7 @@ template <int N> struct P23RowLay {
 template <int N>
 __global__ void __launch_bounds__(P23Cfg<N>::THREADS, P23Cfg<N>::CTAS) k_p23(
     const float2* __restrict__ Ta, const float2* __restrict__ Tb, const float* __restrict__ sigma, int n_alpha,
-    int batch, float2* __restrict__ F, long fgstride, int n_c, const float2* __restrict__ tw, int* __restrict__ err,
+    float2* __restrict__ F, long fgstride, int n_c, const float2* __restrict__ tw, int* __restrict__ err,
     long long wait_limit) {
   using CF = P23Cfg<N>;
   using RL = P23RowLay<N>;
@@ -1791,8 +1789,7 @@ __global__ void __launch_bounds__(P23Cfg<N>::THREADS, P23Cfg<N>::CTAS) k_p23(
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + NSLOT);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int a0 = blockIdx.x;
-  const int b = blockIdx.y;  // m * batch + realisation, for the kernels m = 0, 1
-  sigma += b / batch * n_alpha;
+  const int b = blockIdx.y;
   const int allpairs = (n_alpha + 1) / 2;
   const int pr0 = allpairs * (int)blockIdx.z / (int)gridDim.z;
   const int pr1 = allpairs * ((int)blockIdx.z + 1) / (int)gridDim.z;

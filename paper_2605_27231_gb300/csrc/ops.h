@@ -57,10 +57,9 @@ struct OpsRT {
   // ---- hot path
   // variant: radix choice of the first inverse pass (bit 1: the alternative, where variants(N) == 2)
   static int variants(int N);
-  // first inverse pass (axis 0) with the filter phi_a(cell) and the i n_0 gradient factor; nm: kernels of the launch
-  // (2 only up to N = 128), filter tables mtab values apart, outputs one behind the other
+  // first inverse pass (axis 0) with the filter phi_a(cell) and the i n_0 gradient factor
   static cudaError_t p1(int N, const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* phitab, int nm1,
-                        int nm, long mtab, int alpha0, int nb, int batch, const void* tw, int variant, cudaStream_t st);
+                        int alpha0, int nb, int batch, const void* tw, int variant, cudaStream_t st);
   // second inverse pass (axis 1): the last pass's input rows of every term pair; alpha0 is even, and nb too unless it
   // reaches n_alpha
   static cudaError_t p2(int N, const void* Ta, const void* Tb, void* W, int n_alpha, int alpha0, int nb, int batch,
@@ -76,9 +75,8 @@ struct OpsRT {
   static cudaError_t p3(int N, const void* W, const void* sigma, int n_alpha, void* F, int groups, long fgstride,
                         int n_c, int batch, const void* tw, int* err, long long wait_limit, int variant,
                         cudaStream_t st);
-  // FP32, N = 64 with variant bit 8: one kernel for the second and the last inverse pass of both I_s and
-  // I_c, from the first pass's output for all terms (Ta, Tb [2][batch][n_alpha], columns swizzled by p1 for that variant;
-  // sigma [2][n_alpha]); W is not used.
+  // FP32, N = 64 with variant bit 8: one kernel for the second and the last inverse pass, from the first pass's output for
+  // all terms (Ta, Tb [batch][n_alpha], columns swizzled by p1 for that variant); W is not used.
   static bool fused(int N, int variant);
   static cudaError_t p23(int N, const void* Ta, const void* Tb, const void* sigma, int n_alpha, void* F, int groups,
                          long fgstride, int n_c, int batch, const void* tw, int* err, long long wait_limit,

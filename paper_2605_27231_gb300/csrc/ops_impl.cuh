@@ -99,31 +99,29 @@ struct OpsT {
   }
   template <int N, int E, int TC>
   static cudaError_t p1_v(const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* phitab, int nm1,
-                          int nm, long mtab,
                           int alpha0, int nb, int batch, const void* tw, int swz, cudaStream_t st) {
-    const int nag = p1_groups((long)(N / 2) / TC * N * batch * nm, nb, nm1, 456), per = (nb + nag - 1) / nag;
+    const int nag = p1_groups((long)(N / 2) / TC * N * batch, nb, nm1, 456), per = (nb + nag - 1) / nag;
     const size_t sm = strided_bytes<N, TC, E>() + N * sizeof(C) + N * sizeof(int) + (size_t)per * nm1 * sizeof(T);
     auto k = k_p1<T, N, E, TC>;
     SIGW_CHECK_LAUNCH(allow_smem(k, 227 * 1024));
-    dim3 grid((N / 2) / TC, N, nm * batch * nag);
+    dim3 grid((N / 2) / TC, N, batch * nag);
     k<<<grid, TC * (N / E), sm, st>>>((const C*)phi, (C*)Ta, (C*)Tb, lut, (const T*)phitab, nm1, alpha0, nb, nag, swz,
-                                      batch, mtab, (const C*)tw);
+                                      (const C*)tw);
     return cudaGetLastError();
   }
   template <int N>
   static cudaError_t p1_tm_v(const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* phitab, int nm1,
-                          int nm, long mtab,
                              int alpha0, int nb, int batch, const void* tw, int swz, cudaStream_t st) {
     using CF = std::conditional_t<(N <= 128), P1ACfg<(N <= 128 ? N : 128)>, P1TCfg<N>>;
-    const int nag = p1_groups((long)(N / 2) / CF::TC * N * batch * nm, nb, nm1, 152 * CF::CTAS), per = (nb + nag - 1) / nag;
+    const int nag = p1_groups((long)(N / 2) / CF::TC * N * batch, nb, nm1, 152 * CF::CTAS), per = (nb + nag - 1) / nag;
     const size_t sm = CF::smem(per, nm1);
-    dim3 grid((N / 2) / CF::TC, N, nm * batch * nag);
+    dim3 grid((N / 2) / CF::TC, N, batch * nag);
     if constexpr (N <= 128) {
       auto k = k_p1_ab<N>;
       SIGW_CHECK_LAUNCH(allow_smem(k, 227 * 1024));
       k<<<grid, CF::THREADS, sm, st>>>((const float2*)phi, (float2*)Ta, (float2*)Tb, lut, (const float*)phitab, nm1,
-                                       alpha0, nb, nag, swz, batch, mtab, (const float2*)tw);
-    } else {  // one kernel at a time (nm = 1)
+                                       alpha0, nb, nag, swz, (const float2*)tw);
+    } else {
       auto k = k_p1_tm<N>;
       SIGW_CHECK_LAUNCH(allow_smem(k, 227 * 1024));
       k<<<grid, CF::THREADS, sm, st>>>((const float2*)phi, (float2*)Ta, (float2*)Tb, lut, (const float*)phitab, nm1,
@@ -133,18 +131,18 @@ struct OpsT {
   }
   template <int N>
   static cudaError_t p1_n(const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* phitab, int nm1,
-                          int nm, long mtab, int alpha0, int nb, int batch, const void* tw, int variant, cudaStream_t st) {
+                          int alpha0, int nb, int batch, const void* tw, int variant, cudaStream_t st) {
     using SH = Shape<T, N>;
     using AL = AltStrided<T, N>;
     const int swz = fused_n<N>(variant) ? 8 : 0;  // the fused second and last pass reads swizzled columns
     if constexpr (sizeof(T) == 4 && N >= 64) {  // both transforms side by side, Phi~ tile and cells in tensor memory
-      if (variant & 16) return p1_tm_v<N>(phi, Ta, Tb, lut, phitab, nm1, nm, mtab, alpha0, nb, batch, tw, swz, st);
+      if (variant & 16) return p1_tm_v<N>(phi, Ta, Tb, lut, phitab, nm1, alpha0, nb, batch, tw, swz, st);
     }
     if constexpr (AL::exists) {
       if (variant & 1)
-        return p1_v<N, AL::E, AL::TC>(phi, Ta, Tb, lut, phitab, nm1, nm, mtab, alpha0, nb, batch, tw, swz, st);
+        return p1_v<N, AL::E, AL::TC>(phi, Ta, Tb, lut, phitab, nm1, alpha0, nb, batch, tw, swz, st);
     }
-    return p1_v<N, SH::ES, SH::TC>(phi, Ta, Tb, lut, phitab, nm1, nm, mtab, alpha0, nb, batch, tw, swz, st);
+    return p1_v<N, SH::ES, SH::TC>(phi, Ta, Tb, lut, phitab, nm1, alpha0, nb, batch, tw, swz, st);
   }
   template <int N>
   static constexpr bool fused_n(int variant) {
@@ -157,9 +155,9 @@ struct OpsT {
       using CF = P23Cfg<N>;
       auto k = k_p23<N>;
       SIGW_CHECK_LAUNCH(allow_smem(k, CF::SMEM));
-      dim3 grid(N, 2 * batch, groups);  // both kernels
+      dim3 grid(N, batch, groups);
       k<<<grid, CF::THREADS, CF::SMEM, st>>>((const float2*)Ta, (const float2*)Tb, (const float*)sigma, n_alpha,
-                                             batch, (float2*)F, fgstride, n_c, (const float2*)tw, err,
+                                             (float2*)F, fgstride, n_c, (const float2*)tw, err,
                                              wait_limit);
       return cudaGetLastError();
     } else {
@@ -173,7 +171,7 @@ struct OpsT {
   static int last_groups_n(int variant, int n_alpha) {
     long tiles, slots;
     if (fused_n<N>(variant)) {
-      tiles = 2 * N;  // both kernels
+      tiles = N;
       slots = 304;
     } else {
       using CF = P3Cfg<T, N, ((N >= 16) ? 8 : 4)>;
@@ -391,8 +389,8 @@ LaunchShape OpsRT<T>::shape(int N) {
 }
 template <typename T>
 cudaError_t OpsRT<T>::p1(int N, const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* phitab, int nm1,
-                      int nm, long mtab, int alpha0, int nb, int batch, const void* tw, int variant, cudaStream_t st) {
-  SIGW_DISPATCH_N(N, return (OpsT<T>::template p1_n<NN>(phi, Ta, Tb, lut, phitab, nm1, nm, mtab, alpha0, nb, batch, tw, variant, st)));
+                      int alpha0, int nb, int batch, const void* tw, int variant, cudaStream_t st) {
+  SIGW_DISPATCH_N(N, return (OpsT<T>::template p1_n<NN>(phi, Ta, Tb, lut, phitab, nm1, alpha0, nb, batch, tw, variant, st)));
 }
 template <typename T>
 cudaError_t OpsRT<T>::p2(int N, const void* Ta, const void* Tb, void* W, int n_alpha, int alpha0, int nb, int batch,

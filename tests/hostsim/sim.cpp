@@ -270,21 +270,18 @@ cudaError_t OpsRT<T>::pass_pack(int N, const void* X, void* Y, int b, const void
 
 // ---- hot path: T and W carry their kernel (its tables) and shell (its cell table) from pass to pass
 template <typename T>
-cudaError_t OpsRT<T>::p1(int N, const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* tab, int nm1, int nm,
-                         long mtab, int a0, int nb, int batch, const void*, int variant, cudaStream_t) {
+cudaError_t OpsRT<T>::p1(int N, const void* phi, void* Ta, void* Tb, const int16_t* lut, const void* tab, int nm1, int a0,
+                         int nb, int batch, const void*, int variant, cudaStream_t) {
   return launch([=] {
     const Size<T> z(N);
     want("P1", rd("P1", phi, batch * z.h), "X");
-    for (int m = 0; m < nm; ++m) {
-      const char* t = c(tab) + m * mtab * sizeof(T);
-      check("P1 tables", t, (size_t)(a0 + nb) * nm1 * sizeof(T));
-      const std::string id = " " + num(t) + " " + num(lut) + " terms " + std::to_string(a0) + "+" + std::to_string(nb) +
-                             (fused(N, variant) ? " fused" : "");
-      wr("P1", c(Ta) + (size_t)m * batch * nb * z.f, batch * nb * z.f, "Ta" + id);
-      wr("P1", c(Tb) + (size_t)m * batch * nb * z.f, batch * nb * z.f, "Tb" + id);
-    }
+    check("P1 tables", tab, (size_t)(a0 + nb) * nm1 * sizeof(T));
+    const std::string id = " " + num(tab) + " " + num(lut) + " terms " + std::to_string(a0) + "+" + std::to_string(nb) +
+                           (fused(N, variant) ? " fused" : "");
+    wr("P1", Ta, batch * nb * z.f, "Ta" + id);
+    wr("P1", Tb, batch * nb * z.f, "Tb" + id);
     want("P1", rd("P1", phi, batch * z.h), "X");
-    for (int m = 0; m < nm; ++m) want("P1", rd("P1", c(Ta) + (size_t)m * batch * nb * z.f, batch * nb * z.f), "Ta");
+    want("P1", rd("P1", Ta, batch * nb * z.f), "Ta");
   });
 }
 static std::string owner(const std::string& t) {  // kernel and shell
@@ -343,16 +340,13 @@ cudaError_t OpsRT<T>::p23(int N, const void* Ta, const void* Tb, const void* sig
   return launch([=] {
     const Size<T> z(N);
     const size_t n = (size_t)6 * batch * N * N * (n_c + 1) * z.cel;
-    for (int m = 0; m < 2; ++m) {
-      check("P23 sigma", c(sigma) + m * n_alpha * sizeof(T), n_alpha * sizeof(T));
-      const size_t off = (size_t)m * batch * n_alpha * z.f;
-      const std::string t = rd("P23", c(Ta) + off, batch * n_alpha * z.f), id = owner(t);
-      const std::string all = id + " terms 0+" + std::to_string(n_alpha) + " fused";
-      if (t != "Ta" + all || rd("P23", c(Tb) + off, batch * n_alpha * z.f) != "Tb" + all) fault("P23 reads '" + t + "'");
-      for (int g = 0; g < groups; ++g) wr("P23", c(F) + g * fgs * z.cel + m * n, n, "F" + id);
-      rd("P23", c(Ta) + off, batch * n_alpha * z.f);
-      rd("P23", c(Tb) + off, batch * n_alpha * z.f);
-    }
+    check("P23 sigma", sigma, n_alpha * sizeof(T));
+    const std::string t = rd("P23", Ta, batch * n_alpha * z.f), id = owner(t);
+    const std::string all = id + " terms 0+" + std::to_string(n_alpha) + " fused";
+    if (t != "Ta" + all || rd("P23", Tb, batch * n_alpha * z.f) != "Tb" + all) fault("P23 reads '" + t + "'");
+    for (int g = 0; g < groups; ++g) wr("P23", c(F) + g * fgs * z.cel, n, "F" + id);
+    rd("P23", Ta, batch * n_alpha * z.f);  // not written over
+    rd("P23", Tb, batch * n_alpha * z.f);
   });
 }
 static void n1_range(int N, int n_c, int* nk1) { *nk1 = (n_c < N / 2 ? n_c : N / 2) - (n_c < N / 2 ? -n_c : 1 - N / 2) + 1; }

@@ -47,6 +47,14 @@ def _run(p, batch=1, shells=(1,), **kw):
     p.spectrum(list(shells))
 
 
+KINDS = slice(1, 4)  # first, second and last inverse pass among the profile's kinds
+
+
+def _launches(p, kinds=KINDS):
+    r = p.profile_read()
+    return [r[k]["launches"] for k in [k for k in r if isinstance(r[k], dict)][kinds]]
+
+
 def _autotune(sim, p):
     sim.lib().sim_check_values(0)
     r = p.autotune()
@@ -73,15 +81,13 @@ def test_queued_uploads_keep_their_host_buffers(sim):
 
 # ---- launches
 
-@pytest.mark.parametrize("N,n_alpha", [(32, 1), (32, 3), (32, 9), (32, 15), (32, 16), (256, 7), (128, 17), (128, 25)])
+@pytest.mark.parametrize("N,n_alpha", [(32, 1), (32, 3), (32, 9), (32, 15), (32, 16), (256, 7), (128, 17)])
 def test_terms_that_fit_take_one_launch(sim, N, n_alpha):
     with sim.Plan(N, 1.0, precision=64 if N == 32 else 32, n_alpha=n_alpha) as p:
         p.generate(1e-2, 0.5, 10.0)
         p.profile(False)
         p.spectrum([1, N // 2])
-        r = p.profile_read()
-    kinds = [k for k in r if isinstance(r[k], dict)]
-    assert [r[k]["launches"] for k in kinds[1:4]] == [4, 4, 4]  # passes of two shells, two kernels
+        assert _launches(p) == [4, 4, 4]  # passes of two shells, two kernels
 
 
 # ---- buffers
@@ -95,3 +101,54 @@ def test_terms_tuned_on_another_plan_fit_this_plan(sim, alpha_batch):
         _run(p)
     with sim.Plan(16, 1.0, n_alpha=50) as q:
         _run(q)
+
+
+# Device memory (bytes) that admitted a plan when its stages lay side by side, with one group of term pairs and one kernel at a
+# time: (N, precision, n_alpha, alpha_batch, max_batch).  A server's budget is counted in these.
+FOOTPRINT = {(8, 32, 50, 0, 1): 492324,
+             (8, 64, 13, 1, 64): 15125080,
+             (16, 32, 5, 0, 2): 1320216,
+             (32, 64, 50, 0, 1): 51553448,
+             (32, 32, 3, 1, 1): 3314516,
+             (64, 32, 50, 0, 1): 205358500,
+             (64, 32, 50, 0, 8): 1640890752,
+             (64, 32, 50, 50, 1): 276661668,
+             (64, 64, 51, 0, 2): 832923184,
+             (64, 32, 3, 1, 64): 1649457072,
+             (128, 32, 50, 0, 1): 1640377188,
+             (128, 64, 50, 0, 1): 3277990664,
+             (128, 32, 1, 50, 64): 11480740560,
+             (256, 32, 50, 0, 4): 52421434288,
+             (256, 32, 3, 1, 1): 1639170612,
+             (512, 32, 50, 0, 1): 104955218404,
+             (512, 64, 50, 0, 1): 209807398280,
+             (512, 64, 1, 0, 1): 22984552168}
+
+
+@pytest.mark.parametrize("key", FOOTPRINT)
+def test_footprint_does_not_grow(sim, key):
+    o = sim.default_opts(**dict(zip(("precision", "n_alpha", "alpha_batch", "max_batch"), key[1:])))
+    assert sim.footprint(key[0], o) <= FOOTPRINT[key]
+    before = sim.lib().sim_device_bytes()
+    with sim.Plan(key[0], 1.0, o):
+        assert sim.lib().sim_device_bytes() - before <= sim.footprint(key[0], o)
+
+
+@pytest.mark.parametrize("N,precision,bits", [(8, 32, 0), (16, 64, 0), (32, 64, 0), (64, 32, 24), (64, 32, 0), (64, 64, 0),
+                                              (128, 32, 26), (128, 64, 0), (256, 32, 26)])
+@pytest.mark.parametrize("n_alpha,alpha_batch", [(1, 0), (2, 1), (3, 1), (5, 0), (13, 4), (50, 0), (51, 7), (50, 50), (300, 300)])
+def test_every_stage_finds_what_the_one_before_left(sim, N, precision, bits, n_alpha, alpha_batch):
+    """All buffers of the hot loop share one block: spectra, jackknife and the transforms' scratch over every plan form."""
+    o = dict(precision=precision, n_alpha=n_alpha, n_modes=max(200, n_alpha), alpha_batch=alpha_batch, max_batch=3)
+    shells = sorted({1, 2, N // 4, N // 2 - 1, N // 2})
+    with sim.Plan(N, 1.0, **o) as p:
+        for batch, choices in ((1, (None,)), (3, (None, 1, 2, 3, 10))):
+            p.generate(1e-2, 0.5, 10.0, "nonlocal", alpha_NL=1.0, seeds=range(batch))
+            for c in choices:
+                if c is not None and c <= min(n_alpha, alpha_batch or 16):
+                    p.set_tuning(c, bits)
+                p.spectrum(shells)
+            p.spectrum_jackknife(shells[:-1], M=2)
+            p.spectrum([N // 2])
+        _autotune(sim, p)
+        p.spectrum(shells)
