@@ -1386,7 +1386,7 @@ template <bool SC> __device__ __forceinline__ void idft8c(c2* v) {
   bfly_s<SC>(e[3], u, -h, h, v[3], v[7]);
 }
 __device__ __forceinline__ void idft16c(c2* v) {
-  const float h = 0.70710678118654752440f, c = 0.92387953251128675613f, t = 0.41421356237309504880f;  // cos, tan (pi/8)
+  const float h = 0.70710678118654752440f, c = cos_pi_8<float>(), t = 0.41421356237309504880f;  // cos, tan (pi/8)
   c2 e[8], o[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) { e[k] = v[2 * k]; o[k] = v[2 * k + 1]; }
