@@ -312,10 +312,10 @@ sigw_status sigw_cell_table(const sigw_opts* opts, int n_c, int msq_max, int16_t
 sigw_status sigw_fft3d_noalloc(int N, int precision, int direction, const void* in_dev, void* out_dev,
                                void* cuda_stream);
 
-/* Test hook for failure handling (no counterpart in the paper): the bounded waits in the main loop of the last
- * inverse pass (the bulk-copy ring) give up after `cycles` clock cycles instead of about a second (cycles = 0
+/* Test hook for failure handling (no counterpart in the paper): the bounded waits for bulk copies in the main
+ * loops of the second and the last inverse pass give up after `cycles` clock cycles instead of about a second (cycles = 0
  * restores the default).  A tiny limit makes waits give up while every copy still completes normally: the
- * spectrum call then returns SIGW_ETIMEOUT (results invalid), every copy in flight has landed before its CTA
+ * spectrum call then returns SIGW_ETIMEOUT (results invalid; the error text names the passes that gave up), every copy in flight has landed before its CTA
  * exits, and the plan stays usable.  Applies to launches queued after the call (a captured all-shells graph is
  * dropped and captured again).  Errors: SIGW_EINVAL (NULL plan, cycles < 0). */
 sigw_status sigw_plan_debug_wait_limit(sigw_plan plan, long long cycles);

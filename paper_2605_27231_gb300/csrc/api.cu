@@ -199,7 +199,7 @@ struct sigw_plan_s {
   double* d_mean = nullptr;
   unsigned long long* d_hits = nullptr;
   int* d_err = nullptr;  // OR-ed by kernels whose bounded waits gave up
-  long long wait_limit = sigw::kDefaultWaitLimit;  // cycles of P3's main-loop waits (sigw_plan_debug_wait_limit)
+  long long wait_limit = sigw::kDefaultWaitLimit;  // cycles of the main-loop waits (sigw_plan_debug_wait_limit)
   // CUDA graph of the all-shells spectrum loop, per realisation count
   cudaGraphExec_t graph = nullptr;
   int graph_batch = 0;
@@ -307,7 +307,13 @@ sigw_status check_err_flag(sigw_plan p) {
   if (e != cudaSuccess) return cuda_fail(p, e, "read error flag");
   if (h) {
     cudaMemset(p->d_err, 0, sizeof(int));
-    return fail(p, SIGW_ETIMEOUT, "a bounded wait in the bulk-copy pipeline gave up; results are invalid");
+    std::string where;
+    const std::pair<int, const char*> passes[] = {
+        {sigw::kWaitSecond, "second"}, {sigw::kWaitLast, "last"}, {sigw::kWaitFused, "fused second and last"}};
+    for (auto& [bit, name] : passes)
+      if (h & bit) where += (where.empty() ? "" : ", ") + std::string(name);
+    return fail(p, SIGW_ETIMEOUT,
+                "a bounded wait for bulk copies gave up (inverse passes: " + where + "); results are invalid");
   }
   return SIGW_OK;
 }

@@ -482,13 +482,18 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 // With the default limit the wait uses try_wait, which may suspend the thread for a while inside the instruction;
-// with a shorter limit (a test's) it polls with the non-blocking test_wait, so the limit is what decides.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err,
+// with a shorter limit (a test's) it polls with the non-blocking test_wait.  The clock is looked at before the barrier, so
+// that a tiny limit gives up however soon the copy lands.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err, int bit,
                                           long long limit = kDefaultWaitLimit) {
   const uint32_t a = smem_u32(bar);
   const long long t0 = clock64();
   const bool poll = limit < kDefaultWaitLimit;
   while (true) {
+    if (clock64() - t0 > limit) {
+      atomicOr(err, bit);
+      return false;
+    }
     uint32_t done;
     if (poll) {
       asm volatile(
@@ -504,10 +509,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
           : "memory");
     }
     if (done) return true;
-    if (clock64() - t0 > limit) {
-      atomicOr(err, 1);
-      return false;
-    }
   }
 }
 
@@ -647,7 +648,7 @@ __global__ void __launch_bounds__(P3Cfg<T, N, E_>::THREADS, 1) k_p3(const cx<T>*
       issue(pr + STAGES - 1);
       issued = pr + STAGES;
     }
-    if (ok) ok = mbar_wait(bars + s, (uint32_t)((pr / STAGES) & 1), err, wait_limit);
+    if (ok) ok = mbar_wait(bars + s, (uint32_t)((pr / STAGES) & 1), err, kWaitLast, wait_limit);
     const int a = 2 * (pr0 + pr);
     const bool two = a + 1 < n_alpha;
     const cx<T>* z0 = ring + s * CF::STAGE_ELEMS + rr * N;  // f = 0, 1, 2 follow RPC rows apart
@@ -677,7 +678,7 @@ __global__ void __launch_bounds__(P3Cfg<T, N, E_>::THREADS, 1) k_p3(const cx<T>*
     // succeeded; after a wait gave up, the copies still in flight are waited for with the default limit).
     for (int s = 0; s < STAGES && s < issued; ++s) {
       const int last = s + ((issued - 1 - s) / STAGES) * STAGES;
-      mbar_wait(bars + s, (uint32_t)((last / STAGES) & 1), err);
+      mbar_wait(bars + s, (uint32_t)((last / STAGES) & 1), err, kWaitLast);
     }
   }
   // forward R2C of the six real rows (00, 11 | 22, 01 | 02, 12), two per complex transform
@@ -993,7 +994,7 @@ __global__ void __launch_bounds__(P2Cfg<T, N>::THREADS, P2Cfg<T, N>::CTAS) k_p2(
       if (CF::FSPLIT && f != fs) continue;
       const bool last = s == 1 || !two && f == 2;  // this transform completes the field's two rows
       if (s == 0 || f == 2)                        // its tile has arrived
-        if (ok) ok = mbar_wait(bars + (q & 1), (uint32_t)((q >> 1) & 1), err, wait_limit);
+        if (ok) ok = mbar_wait(bars + (q & 1), (uint32_t)((q >> 1) & 1), err, kWaitSecond, wait_limit);
       cx<T>* const x0 = ring + (q & 1) * CF::TILE + j * TC + c;
       cx<T> v[E];
 #pragma unroll
@@ -1102,8 +1103,8 @@ __global__ void __launch_bounds__(P2Cfg<T, N>::THREADS, P2Cfg<T, N>::CTAS) k_p2(
     }
   }
   if (threadIdx.x == 0) {  // the last copy issued into each slot has landed before the CTA may exit
-    mbar_wait(bars + ((issued - 1) & 1), (uint32_t)(((issued - 1) >> 1) & 1), err);
-    if (issued > 1) mbar_wait(bars + ((issued - 2) & 1), (uint32_t)(((issued - 2) >> 1) & 1), err);
+    mbar_wait(bars + ((issued - 1) & 1), (uint32_t)(((issued - 1) >> 1) & 1), err, kWaitSecond);
+    if (issued > 1) mbar_wait(bars + ((issued - 2) & 1), (uint32_t)(((issued - 2) >> 1) & 1), err, kWaitSecond);
   }
   if constexpr (CF::ZTM) {
     tmem_fence_before_sync();
@@ -1196,7 +1197,7 @@ __global__ void __launch_bounds__(P3TCfg<N>::THREADS, 3) k_p3_tm(const float2* _
   const float2* zin = ring + rr * N;  // rows f = 0, 1, 2 follow RPC rows apart
   bool ok = true;
   for (int pr = 0; pr < npairs; ++pr) {
-    if (ok) ok = mbar_wait(bar, (uint32_t)(pr & 1), err, wait_limit);
+    if (ok) ok = mbar_wait(bar, (uint32_t)(pr & 1), err, kWaitLast, wait_limit);
     const int a = 2 * pr;
     const bool two = a + 1 < n_alpha;
     // inputs of the three transforms: (g0^a + i g0^{a+1}), (g2^a + i g1^a), (g2^{a+1} + i g1^{a+1})
@@ -1265,7 +1266,7 @@ __global__ void __launch_bounds__(P3TCfg<N>::THREADS, 3) k_p3_tm(const float2* _
     }
     tmem_wait_st();
   }
-  if (threadIdx.x == 0 && issued > 0) mbar_wait(bar, (uint32_t)((issued - 1) & 1), err);  // drain the last copy
+  if (threadIdx.x == 0 && issued > 0) mbar_wait(bar, (uint32_t)((issued - 1) & 1), err, kWaitLast);  // drain the last copy
   // forward R2C of the six real rows, two per complex transform: (s00, s11), (s22, s01), (s02, s12)
   float2* zo = L.buf(0);
 #pragma unroll 1
@@ -1917,7 +1918,7 @@ __global__ void __launch_bounds__(P23Cfg<N>::THREADS, P23Cfg<N>::CTAS) k_p23(
       float2 v[E];
       const int used = (ph == 0 && two) ? 2 : 1;
       for (int u = 0; u < used; ++u)
-        if (ok) ok = mbar_wait(bars + (q + u) % NSLOT, (uint32_t)(((q + u) / NSLOT) & 1), err, wait_limit);
+        if (ok) ok = mbar_wait(bars + (q + u) % NSLOT, (uint32_t)(((q + u) / NSLOT) & 1), err, kWaitFused, wait_limit);
       const float2* t0 = ring + (q % NSLOT) * CF::TILE;
       if (ph == 0) load_any(std::true_type{}, v, t0, two ? ring + ((q + 1) % NSLOT) * CF::TILE : nullptr);
       else load_any(std::false_type{}, v, t0, nullptr);
@@ -2034,7 +2035,7 @@ __global__ void __launch_bounds__(P23Cfg<N>::THREADS, P23Cfg<N>::CTAS) k_p23(
   if (threadIdx.x == 0) {  // the last copy issued into each slot has landed before the CTA may exit
     for (int s = 0; s < NSLOT && s < issued; ++s) {
       const int last = s + ((issued - 1 - s) / NSLOT) * NSLOT;
-      mbar_wait(bars + s, (uint32_t)((last / NSLOT) & 1), err);
+      mbar_wait(bars + s, (uint32_t)((last / NSLOT) & 1), err, kWaitFused);
     }
   }
   // ---- forward R2C of the six real rows along axis 2, two per complex transform: (s00, s11), (s22, s01), (s02, s12)

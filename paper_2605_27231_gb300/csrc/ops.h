@@ -10,6 +10,9 @@ namespace sigw {
 // Tile shapes chosen per (precision, N); exposed so the host can size buffers.
 constexpr long long kDefaultWaitLimit = 1ll << 31;  // clock cycles of a bounded wait, about one second
 
+// Bits of the error flag: the pass whose bounded wait gave up.
+enum { kWaitSecond = 1, kWaitLast = 2, kWaitFused = 4 };
+
 struct LaunchShape {
   int tc_strided;   // columns per CTA in strided passes
   int tc_f3;        // columns per CTA in the forward-axis-0 / TT / bin pass
@@ -65,7 +68,7 @@ struct OpsRT {
   static cudaError_t p2(int N, const void* Ta, const void* Tb, void* W, int n_alpha, int alpha0, int nb, int batch,
                         const void* tw, int* err, long long wait_limit, cudaStream_t st);
   // last inverse pass (axis 2, C2R) + sum_a sigma_a g_i g_j + forward R2C along axis 2 keeping k2 <= n_c
-  // err: device int, OR-ed with 1 when a bounded wait of the bulk-copy pipeline gives up; wait_limit: clock
+  // err: device int, OR-ed with the pass's bit when a bounded wait of its bulk copies gives up; wait_limit: clock
   // cycles after which a wait of the main loop gives up (kDefaultWaitLimit unless a test shrinks it).
   // variant bit 2 selects the radix-16 form where p3_variants(N) >= 2; bit 8 the radix-16 form with its
   // accumulators in tensor memory where p3_variants(N) == 3 (FP32, N = 128, 256, 512).
