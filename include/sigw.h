@@ -119,7 +119,8 @@ const char* sigw_plan_last_error(sigw_plan plan);
 sigw_status sigw_plan_kernel_terms(sigw_plan plan, int m, double* sigma, double* phi, double* edges);
 
 /* Synthesis (steps 1-2 above) for `batch` realisations, seeds[b] the Philox4x32-10 key of realisation b
- * (noise g(x) ~ N(0,1) per cell from counter (cell, 0, 0, 0), Box-Muller in FP64).  Leaves Phi~ resident
+ * (noise g(x) ~ N(0,1) per cell from counter (cell, 0, 0, 0), Box-Muller in FP64, or at precision 32 in pairs of FP32
+ * values with a relative error below 2^-30 before the one rounding).  Leaves Phi~ resident
  * on the device.  usr_hits (nullable, host, [batch]) receives the USR floor-hit counts.  Waits for the stream.
  * Errors: SIGW_EINVAL (batch out of [1, max_batch], bad parameters), SIGW_EDOMAIN (strict mode), SIGW_ECUDA. */
 sigw_status sigw_generate(sigw_plan plan, const sigw_pzeta* pz, const sigw_ngmap* map, const uint64_t* seeds,
@@ -236,20 +237,21 @@ sigw_status sigw_server_set_express(sigw_server srv, int slots, int max_N);
 /* Finishes running batches, drops queued requests, frees every plan. */
 sigw_status sigw_server_destroy(sigw_server srv);
 
-/* Autotuner (no counterpart in the paper).  On the plan's current field, times the two strided inverse passes of
- * one target shell (n_c; 0 picks N/4) for every candidate choice: terms per launch in {4, 5, 8, 10, 16} (at most
- * n_alpha; exactly opts->alpha_batch when that is set) and, where more than one exists (FP32, N >= 64), the forms of
- * the first strided pass (two radices, and its Phi~ tile and cells in tensor memory).  Keeps the fastest in the plan and,
- * if opts->alpha_batch is 0, in a process-wide table keyed by (N, precision, max_batch, n_alpha) from which later plans
- * with alpha_batch = 0 start; then times the forms of the last inverse pass (FP32, N = 128, 256, 512: two radices, and radix 16 with its accumulators
- * in tensor memory) on the terms just produced, and at FP32 N = 64 the fused second and last pass against the three
- * passes.  An untuned FP32 plan starts from 16 terms and the bits measured fastest on GB300 (24 at N = 64, 26 from
- * N = 128 on).  Terms go in equal launches of whole pairs of at most the chosen number (an odd number counts as the
- * next even one); at N = 128 the largest choice, 16, stands for as many as the plan's memory holds.  Outputs nullable: chosen terms per launch, variant bits (1: alternative radix of the first strided
- * pass, 2: radix-16 last pass, 4: accepted and ignored (the second strided pass has one form), 8: radix-16 last pass with
- * its accumulators in tensor memory, which at N = 64 also takes in the second pass and runs all terms in one launch
- * whatever the terms per launch, 16: first pass with its tile in tensor memory) and the time in ms of the chosen strided
- * passes plus last pass for one kernel (m = s).  Waits for the stream.
+/* Autotuner (no counterpart in the paper).  On the plan's current field, times the two strided inverse passes of one
+ * target shell (n_c; 0 picks N/4) for every candidate choice: terms per launch in {4, 5, 8, 10, 16} and the untuned one
+ * (at most n_alpha; exactly opts->alpha_batch when that is set) and, where more than one exists (FP32, N >= 64), the
+ * forms of the first strided pass (two radices, and its Phi~ tile and cells in tensor memory).  Keeps the fastest in
+ * the plan and, if opts->alpha_batch is 0, in a process-wide table keyed by (N, precision, max_batch, n_alpha) from
+ * which later plans with alpha_batch = 0 start; then times the forms of the last inverse pass (FP32, N = 128, 256, 512:
+ * two radices, and radix 16 with its accumulators in tensor memory) on the terms just produced, and at FP32 N = 64 the
+ * fused second and last pass against the three passes.  An untuned FP32 plan starts from 16 terms and the bits measured
+ * fastest on GB300 (24 at N = 64, 26 from N = 128 on).  Terms go in equal launches of whole pairs of at most the chosen
+ * number (an odd number counts as the next even one); at N = 128 the largest choice, 16, stands for as many as the
+ * plan's memory holds.  Outputs nullable: chosen terms per launch, variant bits (1: alternative radix of the first
+ * strided pass, 2: radix-16 last pass, 4: accepted and ignored (the second strided pass has one form), 8: radix-16 last
+ * pass with its accumulators in tensor memory, which at N = 64 also takes in the second pass and runs all terms in one
+ * launch whatever the terms per launch, 16: first pass with its tile in tensor memory) and the time in ms of the chosen
+ * strided passes plus last pass for one kernel (m = s).  Waits for the stream.
  * Errors: SIGW_ESTATE (no field), SIGW_EINVAL, SIGW_ECUDA. */
 sigw_status sigw_plan_autotune(sigw_plan plan, int n_c, int* out_alpha_batch, int* out_variant, double* out_ms);
 
@@ -315,8 +317,8 @@ sigw_status sigw_fft3d_noalloc(int N, int precision, int direction, const void* 
 /* Test hook for failure handling (no counterpart in the paper): the bounded waits for bulk copies in the main
  * loops of the second and the last inverse pass give up after `cycles` clock cycles instead of about a second (cycles = 0
  * restores the default).  A tiny limit makes waits give up while every copy still completes normally: the
- * spectrum call then returns SIGW_ETIMEOUT (results invalid; the error text names the passes that gave up), every copy in flight has landed before its CTA
- * exits, and the plan stays usable.  Applies to launches queued after the call (a captured all-shells graph is
+ * spectrum call then returns SIGW_ETIMEOUT (results invalid; the error text names the passes that gave up), every
+ * copy in flight has landed before its CTA exits, and the plan stays usable.  Applies to launches queued after the call (a captured all-shells graph is
  * dropped and captured again).  Errors: SIGW_EINVAL (NULL plan, cycles < 0). */
 sigw_status sigw_plan_debug_wait_limit(sigw_plan plan, long long cycles);
 

@@ -106,6 +106,7 @@ Layout layout_of(int N, const sigw_opts& o, int variant) {
 
 struct Terms {
   int a0, nb;
+  bool operator==(const Terms& o) const { return a0 == o.a0 && nb == o.nb; }
 };
 
 // The launches of the first and second pass for the choice `most` of terms per launch: equal parts in whole pairs (an odd
@@ -1110,7 +1111,8 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
   CKP(p, cudaEventCreate(&e1), "event");
   double best = 1e300;
   int bestB = p->B, bestV = p->variant & 17;
-  const int cands[] = {4, 5, 8, 10, 16};
+  const int cands[] = {4, 5, 8, 10, 16, bmax};  // the untuned choice among them; equal launches are timed once
+  std::vector<std::vector<Terms>> timed;
   sigw_status status = SIGW_OK;
   // For each terms-per-launch candidate the two strided passes are timed separately, the first in each of its forms.
   char* const work = (char*)p->d_work;
@@ -1127,8 +1129,7 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
     return cudaSuccess;
   };
   const Layout lay0 = layout_of(N, p->opts, 0);
-  auto time_pass = [&](int which, int choice, int v, float* ms) -> sigw_status {
-    const std::vector<Terms> ts = launches_of(N, p->opts, lay0, choice, batch, lay0.nm == 2);
+  auto time_pass = [&](int which, const std::vector<Terms>& ts, int v, float* ms) -> sigw_status {
     for (int rep = 0; rep < 2; ++rep) {  // first pass warms the variant; the second is timed
       cudaEventRecord(e0, st);
       const cudaError_t e = strided(which, ts, lay0, v);
@@ -1146,9 +1147,12 @@ sigw_status sigw_plan_autotune(sigw_plan p, int n_c, int* out_alpha_batch, int* 
   for (int B : cands) {
     if (p->opts.alpha_batch > 0) B = bmax;  // terms per launch fixed by the options: tune the radices only
     if (B > bmax || status != SIGW_OK) continue;
+    const std::vector<Terms> ts = launches_of(N, p->opts, lay0, B, batch, lay0.nm == 2);
+    if (std::find(timed.begin(), timed.end(), ts) != timed.end()) continue;
+    timed.push_back(ts);
     float t1[3] = {1e30f, 1e30f, 1e30f}, t2 = 1e30f;
-    for (int v = 0; v < np1 && status == SIGW_OK; ++v) status = time_pass(0, B, v == nvar ? 16 : p1bits[v], &t1[v]);
-    if (status == SIGW_OK) status = time_pass(1, B, 0, &t2);  // P1 wrote the T that P2 reads
+    for (int v = 0; v < np1 && status == SIGW_OK; ++v) status = time_pass(0, ts, v == nvar ? 16 : p1bits[v], &t1[v]);
+    if (status == SIGW_OK) status = time_pass(1, ts, 0, &t2);  // P1 wrote the T that P2 reads
     if (status != SIGW_OK) break;
     int v1 = 0;
     for (int v = 1; v < np1; ++v)

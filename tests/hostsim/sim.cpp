@@ -28,12 +28,12 @@ struct State {
   struct Copy { U lo, hi; std::vector<unsigned char> at_call; };
   std::vector<Copy> pending;  // host sources of queued copies
   std::vector<std::string> bad;
-  SimGraph* capture = nullptr;
   long launches = 0;
   bool values = true;  // whether what a launch reads is checked, not only where
   void* real = nullptr;
 };
 State* S = new State();
+thread_local SimGraph* capture = nullptr;  // capture mode is thread-local
 std::recursive_mutex mu;
 #define LOCK std::lock_guard<std::recursive_mutex> lock(mu)
 
@@ -85,7 +85,7 @@ void want(const char* who, const std::string& got, const std::string& start) {
 }
 cudaError_t launch(std::function<void()> f) {
   LOCK;
-  if (S->capture) S->capture->ops.push_back(f);
+  if (capture) capture->ops.push_back(f);
   else {
     S->launches++;
     f();
@@ -177,8 +177,8 @@ cudaError_t cudaStreamSynchronize(cudaStream_t) {
     if (memcmp((const void*)q.lo, q.at_call.data(), q.hi - q.lo)) fault("a buffer changed before its copy was over");
   return cudaSuccess;
 }
-cudaError_t cudaStreamBeginCapture(cudaStream_t, int) { return S->capture = new SimGraph(), cudaSuccess; }
-cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { return *g = S->capture, S->capture = nullptr, cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, int) { return capture = new SimGraph(), cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { return *g = capture, capture = nullptr, cudaSuccess; }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t g, unsigned long long) {
   return *e = new SimGraph(*g), cudaSuccess;
 }

@@ -90,6 +90,18 @@ def test_terms_that_fit_take_one_launch(sim, N, n_alpha):
         assert _launches(p) == [4, 4, 4]  # passes of two shells, two kernels
 
 
+@pytest.mark.parametrize("n_alpha", [2, 3, 6, 9, 13, 15])
+def test_autotuner_times_the_untuned_choice(sim, n_alpha):
+    """A launch takes a millisecond here, so all terms at once, the untuned choice, are the fastest."""
+    with sim.Plan(32, 1.0, precision=64, n_alpha=n_alpha) as p:
+        _run(p)
+        _, _, ms = _autotune(sim, p)
+        assert ms == 2.0  # a launch of either pass
+        p.profile(False)
+        p.spectrum([1])
+        assert _launches(p) == [2, 2, 2]
+
+
 # ---- buffers
 
 @pytest.mark.parametrize("alpha_batch", [50, 20])
