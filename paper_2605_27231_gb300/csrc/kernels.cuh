@@ -453,15 +453,12 @@ __global__ void __launch_bounds__(256) k_p1(const cx<T>* __restrict__ phi, cx<T>
 // rows over k2, the inputs of the last pass's three complex transforms:
 //   f = 0: g2^a + i g1^a      f = 1: the same of a + 1      f = 2: g0^a + i g0^{a+1}       W[b][pair][f][a0][a1][N]
 // Element c < N/2 of a row is the value at k2 = c, element N - 1 - c the one at k2 = -c; element N - 1 is the value at
-// k2 = N/2.
+// k2 = N/2.  All rows carry a common factor -1 (the products do not see it), which saves sign changes in k_p2.
 // With 64-bit values at N = 128 the index is xor-ed with 8 on odd rows: a half warp of the radix-16 last pass reads two
 // rows there, and they then fall into different banks (see k_p3_tm).
 template <typename T, int N> struct ZRow {
   static constexpr int SWZ = sizeof(T) == 4 && N == 128 ? 8 : 0;
 };
-
-// All rows carry a common factor -1 (the products do not see it), which saves sign changes here.
-//
 
 // ---------------------------------------------------------------- bulk-copy pipeline helpers
 // cp.async.bulk (TMA, 1-D) global -> shared with mbarrier completion.  Waits are bounded: after `limit` clock
@@ -1598,7 +1595,7 @@ template <int N>
 __global__ void __launch_bounds__(P1TCfg<N>::THREADS, 3) k_p1_tm(const float2* __restrict__ phi, float2* __restrict__ Ta,
                                                                   float2* __restrict__ Tb, const int16_t* __restrict__ lut,
                                                                   const float* __restrict__ phitab, int nm1, int alpha0,
-                                                                  int nb, int nag, int swz,
+                                                                  int nb, int nag,
                                                                   const float2* __restrict__ tw) {
   using CF = P1TCfg<N>;
   constexpr int E = CF::E, P = CF::P, TC = CF::TC, H = CF::H, NH = H + 1;
@@ -1654,7 +1651,6 @@ __global__ void __launch_bounds__(P1TCfg<N>::THREADS, 3) k_p1_tm(const float2* _
   }
   const long fstride = (long)N * N * H;  // one field
   const float fj = (float)j;
-  const int cs = cc ^ ((k1 & 1) * swz);
   for (int a = alo; a < ahi; ++a) {
     const float* tab = sm_tab + (a - alo) * nm1;
 #pragma unroll 1
@@ -1712,7 +1708,7 @@ __global__ void __launch_bounds__(P1TCfg<N>::THREADS, 3) k_p1_tm(const float2* _
       }
       if constexpr (N <= 256) fft_pencil_tw8_tm<N, Lay, SyncBlock>(v, j, L, tw, tbase + 48, SyncBlock());
       else fft_pencil<float, N, E, +1, Lay, SyncBlock>(v, j, L, tw, SyncBlock());
-      float2* dst = (D ? Tb : Ta) + ((long)b * nb + a) * fstride + t_index<float, N>(k1, cs);
+      float2* dst = (D ? Tb : Ta) + ((long)b * nb + a) * fstride + t_index<float, N>(k1, cc);
 #pragma unroll
       for (int r = 0; r < E; ++r) dst[(long)(j + r * P) * N * H] = v[r];
     }

@@ -121,11 +121,11 @@ struct OpsT {
       SIGW_CHECK_LAUNCH(allow_smem(k, 227 * 1024));
       k<<<grid, CF::THREADS, sm, st>>>((const float2*)phi, (float2*)Ta, (float2*)Tb, lut, (const float*)phitab, nm1,
                                        alpha0, nb, nag, swz, (const float2*)tw);
-    } else {
+    } else {  // the columns are never swizzled here
       auto k = k_p1_tm<N>;
       SIGW_CHECK_LAUNCH(allow_smem(k, 227 * 1024));
       k<<<grid, CF::THREADS, sm, st>>>((const float2*)phi, (float2*)Ta, (float2*)Tb, lut, (const float*)phitab, nm1,
-                                       alpha0, nb, nag, swz, (const float2*)tw);
+                                       alpha0, nb, nag, (const float2*)tw);
     }
     return cudaGetLastError();
   }
