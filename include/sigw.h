@@ -199,8 +199,8 @@ const char* sigw_strerror(sigw_status s);
  * a shared pool; plans own their streams, so slots overlap on the device.  A plan is created only if its
  * footprint (sigw_plan_footprint) fits hbm_budget_bytes beside the resident plans.  Only the oldest queued
  * request may evict idle plans (least-recently-used first, and only if that frees enough); later requests may
- * allocate only budget that is free and not needed by the oldest one, and start nothing while the oldest one
- * cannot be admitted even by eviction (no starvation).
+ * allocate only budget that is free and not needed by the oldest one, may not use an idle plan that the oldest one
+ * would have to evict, and start nothing while the oldest one cannot be admitted even by eviction (no starvation).
  * All server calls are thread-safe.  No counterpart in the paper (which reports single timings,
  * Sec. sec_conclusions); this is the serving layer around its method. */
 typedef struct sigw_server_stats {

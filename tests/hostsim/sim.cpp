@@ -5,11 +5,14 @@
 #include <dlfcn.h>
 #include <sys/mman.h>
 
+#include <atomic>
+#include <chrono>
 #include <functional>
 #include <map>
 #include <mutex>
 #include <set>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "cuda_runtime.h"
@@ -33,6 +36,7 @@ struct State {
   void* real = nullptr;
 };
 State* S = new State();
+std::atomic<int> hold_N{0};  // the synthesis of this lattice waits
 thread_local SimGraph* capture = nullptr;  // capture mode is thread-local
 std::recursive_mutex mu;
 #define LOCK std::lock_guard<std::recursive_mutex> lock(mu)
@@ -221,6 +225,7 @@ template <typename T> struct Size {
 // ---- synthesis and utility passes
 template <typename T>
 cudaError_t OpsRT<T>::rows_r2c_noise(int N, void* Y, const uint64_t* seeds, int b, const void*, cudaStream_t) {
+  while (hold_N == N) std::this_thread::sleep_for(std::chrono::milliseconds(1));
   return launch([=] { check("noise", seeds, 8 * b); wr("noise", Y, b * Size<T>(N).f, "Y"); });
 }
 template <typename T>
@@ -439,6 +444,7 @@ cudaError_t launch_fin(const double* part, long pbs, int maxblk, int ns, const S
 extern "C" {
 int sigw_fft3d_noalloc() { return 3; }  // the plan-free transform is not simulated
 void sim_init(const char* real) { S->real = dlopen(real, RTLD_NOW | RTLD_LOCAL); }
+void sim_hold(int N) { hold_N = N; }
 void sim_check_values(int on) { S->values = on; }  // off: the autotuner times launches on what is there
 long sim_launches() { return S->launches; }
 size_t sim_device_bytes() {

@@ -4,9 +4,12 @@ import ctypes
 import os
 import shutil
 import subprocess
+import time
 
 import numpy as np
 import pytest
+
+import workloads
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2605_27231_gb300", "csrc")
@@ -77,6 +80,40 @@ def test_queued_uploads_keep_their_host_buffers(sim):
         p.spectrum_async(None, [1])
         p.synchronize()
         p.spectrum_jackknife([1, 4])
+
+
+# ---- server
+
+def _spec(N, seed):
+    return workloads.Spec(N=N, L=1.0, A=1e-2, sigma=0.5, kstar=12.0, kind="gauss", seed=seed)
+
+
+def test_express_slot_leaves_the_head_what_it_has_to_evict(sim):
+    """A 64^3 request at the head of the queue fits once the idle 32^3 plan is evicted, and waits for the general slot, which
+    is busy.  The express slot must not keep that plan busy with a later 32^3 request; it may run a 16^3 one, whose idle plan
+    the head does not need."""
+    o = dict(precision=32, n_alpha=5)
+    fp = {N: sim.footprint(N, sim.default_opts(**o)) for N in (32, 64, 128)}
+    with sim.Server(fp[128] + fp[64] + fp[32] // 2, max_slots=1, **o) as s:
+        for N in (32, 16):
+            s.wait(s.submit(_spec(N, 1)), timeout_s=60)
+        sim.lib().sim_hold(128)
+        try:
+            busy = s.submit(_spec(128, 2))
+            while s.stats()["queued"]:
+                time.sleep(0.001)
+            s.set_express(1, 32)
+            head, small, free = s.submit(_spec(64, 3)), s.submit(_spec(32, 4)), s.submit(_spec(16, 5))
+            s.wait(free, timeout_s=60)
+            with pytest.raises(sim.SigwError) as e:
+                s.wait(small, timeout_s=0.2)
+            assert e.value.status == sim.ETIMEOUT
+        finally:
+            sim.lib().sim_hold(0)
+        for t in (busy, head, small):
+            s.wait(t, timeout_s=60)
+        st = s.stats()
+    assert st["completed"] == 6 and st["failed"] == 0 and st["plans_evicted"] >= 1
 
 
 # ---- launches
