@@ -92,7 +92,7 @@ typedef struct sigw_opts {
   double umin, umax;  /* u-grid range */
   double upiv, sigp, Ap; /* grid density bump of Eq. eq_grid_density */
   int precision;      /* 32: FP32 fields and FFTs (FP64 plan, twiddles and bin sums); 64: FP64 throughout */
-  int alpha_batch;    /* terms per first/second-pass launch; 0 picks a value */
+  int alpha_batch;    /* terms per first/second-pass launch (whole pairs: odd counts as the next even); 0 picks a value */
   int max_batch;      /* most realisations handled by one sigw_generate / sigw_spectrum call */
   int strict_domain;  /* nonzero: USR floor hits make sigw_generate return SIGW_EDOMAIN */
 } sigw_opts;

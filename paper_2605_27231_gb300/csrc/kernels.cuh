@@ -1733,13 +1733,12 @@ __global__ void __launch_bounds__(P1TCfg<N>::THREADS, 3) k_p1_tm(const float2* _
 //   - Rows: the transformed columns go to the row buffer (two block barriers a transform, the only ones), a warp owns
 //     8 rows, and the exchange of the row transform (radix 16 then 4) is in place.
 // Bounded waits, error flag and the drain before exit as in k_p3.
-// What bounds it: the shared-memory path (ncu: 277 wavefronts a warp and transform, 62 % of the path's cycles while
+// What bounds it: the shared-memory path (ncu: 283 wavefronts a warp and transform, 61 % of the path's cycles while
 // active) with 16 warps a SM, issue 50 %; DRAM 17 %.  Four groups of term pairs: 256 CTAs for one realisation, two a SM.
 // 50 terms of both kernels of one realisation take 161 us (k_p2 and k_p3 before 432), of eight 976 us (2044).  Both kernels
 // in one launch with two groups each took 146 and 915 us, but T of both, 4 fields a term, is more than the plan's other
-// forms need (+38 % device memory).  The same split at N = 128
-// (two residue classes of a1 per plane) was slower than the two passes there (715 against 690 us then, 545 now): its
-// shared-memory traffic grows while HBM already carries the passes.
+// forms need (+38 % device memory).  The same split at N = 128 (two residue classes of a1 per plane) was slower than the
+// two passes there (715 against 690 us then, 520 now): its shared-memory traffic grows while HBM already carries them.
 template <int N>
 struct P23Cfg {
   static_assert(N == 64, "one plane per CTA, two CTAs per SM");

@@ -166,7 +166,8 @@ struct OpsT {
   }
   // Groups of term pairs the last pass splits a launch into (each writes a partial F, which the second forward pass
   // adds up): enough for the SMs where one realisation has few tiles.  Not a function of the batch, so a
-  // realisation's sums are grouped the same way, and have the same bits, alone and in a batch.
+  // realisation's sums are grouped the same way, and have the same bits, alone and in a batch.  The plan's memory may allow
+  // fewer (Layout in api.cu).
   template <int N>
   static int last_groups_n(int variant, int n_alpha) {
     long tiles, slots;
