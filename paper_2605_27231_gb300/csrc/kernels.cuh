@@ -479,20 +479,18 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 // With the default limit the wait uses try_wait, which may suspend the thread for a while inside the instruction;
-// with a shorter limit (a test's) it polls with the non-blocking test_wait.  The clock is looked at before the barrier, so
-// that a tiny limit gives up however soon the copy lands.
+// with a shorter limit (a test's) it polls with the non-blocking test_wait and looks at the clock first, so that a tiny
+// limit gives up however soon the copy lands.  The default looks at the barrier first: a thread that was switched out for
+// longer than the limit finds its copy.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err, int bit,
                                           long long limit = kDefaultWaitLimit) {
   const uint32_t a = smem_u32(bar);
   const long long t0 = clock64();
   const bool poll = limit < kDefaultWaitLimit;
   while (true) {
-    if (clock64() - t0 > limit) {
-      atomicOr(err, bit);
-      return false;
-    }
     uint32_t done;
     if (poll) {
+      if (clock64() - t0 > limit) break;
       asm volatile(
           "{ .reg .pred p; mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
           : "=r"(done)
@@ -506,7 +504,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
           : "memory");
     }
     if (done) return true;
+    if (!poll && clock64() - t0 > limit) break;
   }
+  atomicOr(err, bit);
+  return false;
 }
 
 template <typename T, int N, int E_ = ((N >= 16) ? 8 : 4)> struct P3Cfg {
