@@ -46,9 +46,9 @@ METRIC = "SIGW spectra/s at 256^3 (FP32 path; FP64 path on the same GPU under fp
 # proportion to the term-realisations of a launch, so the traffic of a bench launch is the algorithmic bytes of
 # that launch times the captured ratio.  Valid only while the kernel source is unchanged since the capture.
 NCU_TRAFFIC_256 = {
-    "p1_inv_axis0_filter": (0.068036e9 + 1.280607e9, 0.0676e9 + 20 * 67.108864e6),  # k_p1_tm (tile in TMEM)
-    "p2_inv_axis1": (1.343491e9 + 1.957547e9, 50 * 67.108864e6),
-    "p3_inv_axis2_product_fwd_axis2": (2.014203e9 + 0.100286e9, 30 * 67.108864e6 + 6 * 65536 * 33 * 8),  # k_p3_tm
+    "p1_inv_axis0_filter": (0.068001e9 + 1.280478e9, 0.0676e9 + 20 * 67.108864e6),  # k_p1_tm (tile in TMEM)
+    "p2_inv_axis1": (1.343568e9 + 1.957457e9, 50 * 67.108864e6),
+    "p3_inv_axis2_product_fwd_axis2": (2.013361e9 + 0.097999e9, 30 * 67.108864e6 + 6 * 65536 * 33 * 8),  # k_p3_tm
 }
 
 

@@ -113,7 +113,7 @@ struct Terms {
 // choice counts as the next even one), an odd last term in the last of them; at most 256 terms, and what T has room for.
 // At N = 128 the largest choice, 16, stands for as many as fit: a launch of 16 terms of one realisation leaves the last of
 // its few waves short (first pass of 50 terms, when it took them one transform after the other: 253 us in launches of 16,
-// 215 us in two; 173 us now in launches of 32 and 18).
+// 215 us in two; 172 us now in launches of 28 and 22).
 std::vector<Terms> launches_of(int N, const sigw_opts& o, const Layout& l, int most, int batch, bool second) {
   const int n = o.n_alpha;
   auto room = [&](int e) {  // terms of a launch that ends with term e
